@@ -1419,7 +1419,7 @@ int run_in_scratch(recon_plan_t p, const float* images, float* volume, char* scr
 namespace {
 
 struct TrainLayout {
-  size_t S, G, T, pow, eps, acts, deps, theta, grad, m1, m2, sums, loss, total;
+  size_t S, G, T, pow, eps, inputs, deps, theta, grad, m1, m2, sums, loss, total;
 };
 
 int train_plan(const recon_train_cfg* c, recon_plan_t* out) {
@@ -1459,8 +1459,8 @@ TrainLayout train_layout(recon_plan_t p, const recon_train_cfg* c) {
   off = align256(off + N * NB * 4);
   L.eps = off;
   off = align256(off + N * K * NB * 4);
-  L.acts = off;
-  off = align256(off + N * K * NB * recon::kActStride * 4);
+  L.inputs = off;
+  off = align256(off + N * K * NB * sizeof(float4));
   L.deps = off;
   off = align256(off + N * K * NB * 8);
   L.theta = off;
@@ -1522,7 +1522,7 @@ extern "C" int recon_mlp_train(const recon_train_cfg* cfg, float* weights, float
   float2* T = (float2*)(b + L.T);
   float* pow = (float*)(b + L.pow);
   float* eps = (float*)(b + L.eps);
-  float* acts = (float*)(b + L.acts);
+  float4* inputs = (float4*)(b + L.inputs);
   double* deps = (double*)(b + L.deps);
   float* theta = (float*)(b + L.theta);
   float* g = (float*)(b + L.grad);
@@ -1558,9 +1558,9 @@ extern "C" int recon_mlp_train(const recon_train_cfg* cfg, float* weights, float
   for (int it = 0; it < iters && e == cudaSuccess; ++it) {
     e = cudaMemsetAsync(sums, 0, 2 * sizeof(double), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(deps, 0, sizeof(double) * (size_t)N * K * p->lc.n_bins, s);
-    if (e == cudaSuccess) e = recon::launch_eps_table(p->lc, pow, cnt, x2, theta, eps, acts, N, K, 0, s);
+    if (e == cudaSuccess) e = recon::launch_eps_table(p->lc, pow, cnt, x2, theta, eps, inputs, N, K, 0, s);
     if (e == cudaSuccess)
-      e = recon::launch_train_step(p->ca, p->lc, G, T, eps, w.uA, acts, theta, theta, g, m1, m2, N, sums, deps,
+      e = recon::launch_train_step(p->ca, p->lc, G, T, eps, w.uA, inputs, theta, theta, g, m1, m2, N, sums, deps,
                                    cfg->steps > 0 ? cfg->adam_step + it + 1 : 0, cfg->lr, loss + it, s);
   }
   if (e == cudaSuccess)

@@ -203,3 +203,20 @@ def test_trained_regulariser_beats_the_fixed_eps_on_held_out_128cubed_tomograms(
     mean = {k: float(np.mean(v)) for k, v in errs.items()}
     print("held-out 128^3 rel-L2 to the phantoms:", mean)
     assert mean["learned"] < 0.95 * mean["eps=0.3"] < mean["eps=0.1"], mean
+
+
+@pytest.mark.parametrize("n,views,nzl", [(16, 1, 1), (20, 3, 5), (40, 2, 9), (70, 1, 17)])
+def test_training_gradient_at_the_edges_of_its_tiles(n, views, nzl):
+    """Loss and gradient where the rows (image, layer, bin) do not fill the backward pass's
+    chunks, the layers not the loss pass's and the columns not a block's (transforms of 32 to
+    256 points), at the tolerances of the larger case above."""
+    from paper_2206_09151_gb300.recon import train_mlp
+    img, tgt, rot, R, grid = _train_set(1, views, n, nzl, seed=50 + n)
+    w = _weights(11).astype(np.float32)
+    _, loss, grad = train_mlp(w, torch.from_numpy(img).cuda(), torch.from_numpy(tgt).cuda(), rot, R, grid,
+                              nz_layers=nzl, nsr=1e-2, steps=0, want_grad=True, **PHYS)
+    r_eff = R[:, None] - O.layer_centres(rot, grid, nzl, PHYS["delta"])
+    ref_loss, ref_grad = L.train_loss_grad(w.astype(np.float64), img.astype(np.float64), tgt.astype(np.float64),
+                                           r_eff=r_eff, nsr=1e-2, **PHYS)
+    assert abs(loss[0] - ref_loss) <= 1e-5 * ref_loss, (loss[0], ref_loss)
+    assert rel_l2(grad, ref_grad) <= 1e-4, rel_l2(grad, ref_grad)
