@@ -810,26 +810,28 @@ def run_fourier(args):
     # launches per step: the layered CT step twice (cos and sin volumes) or the per-view
     # spectra and splats, plus the 3D passes
     P3 = [1 << int(np.ceil(np.log2(2 * n))) for n in cfg["grid"]]
-    fft3 = sum(1 for q in P3 if q > 1)
+    fft3 = len(P3)  # line-FFT passes of one 3D transform
     sub = max(r.stage_block, 1)
     nsub = sum(-(-min(r.dir_block, D - b * r.dir_block) // sub) for b in range(r.n_blocks))
     dens = 2 if cfg["ramp"] == "density" else 0  # the sampling density, once per call
     if args.form == "swap":
-        launches = dens + 2 * (3 * nsub + r.n_blocks) + 1 + fft3 + (1 + fft3 + 1)
-        # the inversion: the phase kernel reads Z and writes the work grid, each 3D pass reads
-        # and writes it, the crop reads the kept voxels and writes the volume
+        launches = dens + 2 * (3 * nsub + r.n_blocks) + 2 * fft3
+        # the inversion: the z pass reads Z once and writes the kept planes of the half spectrum,
+        # the x pass reads them and writes the kept columns, the y pass reads those and writes the
+        # volume
         cells = float(np.prod(P3))
-        algo = cells * 8 * 2 + fft3 * cells * 8 * 2 + V * 12
+        kept = cfg["grid"][2] * (P3[1] // 2 + 1) * 8.0
+        algo = cells * 8 + kept * (2 * P3[0] + 2 * cfg["grid"][0]) + V * 4
         peaks, peak_src = load_peaks()
         achieved = algo / (phase_ms / 1e3) / 1e9
         roofline = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                    "frac": achieved / peaks["hbm_gbs"], "kernel": "swap_phase (k_swap_phase, k_fft3_lines x3, "
-                    "k_crop_real)", "traffic": None, "algorithmic_bytes_per_launch": algo, "launches": 1,
+                    "frac": achieved / peaks["hbm_gbs"], "kernel": "swap_phase (k_lines x2, k_lines_c2r)",
+                    "traffic": None, "algorithmic_bytes_per_launch": algo, "launches": 1,
                     "ms_per_launch": phase_ms, "peak_source": f"{peak_src} hbm_gbs (MEASURED_PEAKS.json)"}
     else:
         gsub = -(-D // max(1, min(D, (1 << 30) // (cfg["nv"] * (r.padded // 2 + 1) * 8 + (r.padded // 2 + 1)
                                                    * r.padded * 8))))
-        launches = dens + 3 * gsub + 2 + fft3 + 1
+        launches = dens + 3 * gsub + 1 + fft3
         roofline = None
     line = {"metric": METRIC, "value": U / (ms_step / 1e3), "unit": UNIT, "n_gpus": 1, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",

@@ -1115,7 +1115,7 @@ SwapLayout swap_layout(recon_plan_t p) {
   L.Z = off;
   off = align256(off + grid3_cells(p) * sizeof(float2));
   L.work = off;
-  off = align256(off + grid3_cells(p) * sizeof(float2));
+  off = align256(off + recon::swap_half_cells(p->f3) * sizeof(float2));
   for (int a = 0; a < 3; ++a) {
     L.tw[a] = off;
     off = align256(off + p->tw3[a].size() * sizeof(float2));
@@ -1125,7 +1125,7 @@ SwapLayout swap_layout(recon_plan_t p) {
 }
 
 struct GridLayout {
-  size_t Srows, G, dirs, acc, raw, S, stats, tw[3], total;
+  size_t Srows, G, dirs, acc, S, H, stats, tw[3], total;
   int sub;
 };
 
@@ -1141,11 +1141,11 @@ GridLayout grid_layout(recon_plan_t p) {
   L.dirs = off;
   off = align256(off + p->gdirs.size() * sizeof(recon::GridDir));
   L.acc = off;
-  off = align256(off + grid3_cells(p) * sizeof(float2));
-  L.raw = off;
-  off = align256(off + grid3_cells(p) * sizeof(float2));
+  off = align256(off + grid3_cells(p) * sizeof(float4));
   L.S = off;
   off = align256(off + grid3_cells(p) * sizeof(float));
+  L.H = off;
+  off = align256(off + recon::grid_half_cells(p->f3) * sizeof(float2));
   L.stats = off;
   off = align256(off + 2 * sizeof(double));
   for (int a = 0; a < 3; ++a) {
@@ -1175,7 +1175,7 @@ int upload_tw3(recon_plan_t p, char* b, const size_t off[3], float2* dev[3], cud
   return RECON_OK;
 }
 
-// the twiddle table of one axis as the line FFT of that length reads it (fft3.cu)
+// the twiddle table of one axis as the line FFT of that length reads it (fft3.cuh)
 const float2* axis_tw(recon_plan_t p, float2* dev, int a) {
   return p->f3.P3[a] >= 1024 ? dev + (p->f3.P3[a] - 8) : dev;
 }
@@ -1237,9 +1237,8 @@ int recon_swap_ct(recon_plan_t p, const float* images, void* workspace, size_t w
   rc = tma_end(p, workspace, s, "recon_swap_ct");
   if (rc) return rc;
   float2* Z = (float2*)(b + L.Z);
-  cudaError_t e = recon::launch_swap_pack(vc, vs, Z, p->f3, s);
   const float2* twa[3] = {axis_tw(p, tw[0], 0), axis_tw(p, tw[1], 1), axis_tw(p, tw[2], 2)};
-  if (e == cudaSuccess) e = recon::launch_fft3(Z, p->f3.P3, twa, false, s);
+  const cudaError_t e = recon::launch_swap_forward(vc, vs, Z, p->f3, twa, s);
   if (e != cudaSuccess) return cuda_fail(e, "recon_swap_ct: 3D transform");
   return RECON_OK;
 }
@@ -1258,10 +1257,8 @@ int recon_swap_phase(recon_plan_t p, double sigma, double eps, float* volume, vo
   char* b = (char*)workspace;
   float2* tw[3] = {(float2*)(b + L.tw[0]), (float2*)(b + L.tw[1]), (float2*)(b + L.tw[2])};
   const float2* twa[3] = {axis_tw(p, tw[0], 0), axis_tw(p, tw[1], 1), axis_tw(p, tw[2], 2)};
-  float2* work = (float2*)(b + L.work);
-  cudaError_t e = recon::launch_swap_phase((const float2*)(b + L.Z), work, p->f3, p->R0, sigma, eps, p->opt.cs, s);
-  if (e == cudaSuccess) e = recon::launch_fft3(work, p->f3.P3, twa, true, s);
-  if (e == cudaSuccess) e = recon::launch_crop_real(work, volume, p->f3, s);
+  const cudaError_t e = recon::launch_swap_phase((const float2*)(b + L.Z), (float2*)(b + L.work), volume, p->f3, p->R0,
+                                                 sigma, eps, p->opt.cs, twa, s);
   if (e != cudaSuccess) return cuda_fail(e, "recon_swap_phase");
   return RECON_OK;
 }
@@ -1295,14 +1292,12 @@ int recon_grid_run(recon_plan_t p, const float* images, float* volume, double ns
   rc = upload_tw3(p, b, L.tw, tw, s);
   if (rc) return rc;
   recon::GridDir* gd = (recon::GridDir*)(b + L.dirs);
-  float2* acc = (float2*)(b + L.acc);
-  float2* raw = (float2*)(b + L.raw);
+  void* acc = b + L.acc;
   float* S = (float*)(b + L.S);
   const size_t cells = grid3_cells(p);
   cudaError_t e = cudaMemcpyAsync(gd, p->gdirs.data(), sizeof(recon::GridDir) * p->gdirs.size(),
                                   cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, cells * sizeof(float2), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(raw, 0, cells * sizeof(float2), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, cells * (nsr > 0.0 ? sizeof(float4) : sizeof(float2)), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(S, 0, cells * sizeof(float), s);
   float2* Srows = (float2*)(b + L.Srows);
   float2* G = (float2*)(b + L.G);
@@ -1310,13 +1305,12 @@ int recon_grid_run(recon_plan_t p, const float* images, float* volume, double ns
     const int cnt = std::min(L.sub, p->D - d0);
     e = recon::launch_rows_fwd(p->ca, Srows, w.twp, images, d0, cnt, s);
     if (e == cudaSuccess) e = recon::launch_cols_forward(p->ca, p->lc, Srows, G, nullptr, w.twp, cnt, s);
-    if (e == cudaSuccess) e = recon::launch_grid_splat(G, gd, d0, cnt, p->ca, p->f3, acc, raw, S, nsr > 0.0, s);
+    if (e == cudaSuccess) e = recon::launch_grid_splat(G, gd, d0, cnt, p->ca, p->f3, acc, S, nsr > 0.0, s);
   }
   const float nsr_m = (float)(nsr * std::sqrt((double)p->nu * p->nv));
-  if (e == cudaSuccess) e = recon::launch_grid_finish(acc, raw, S, (double*)(b + L.stats), p->f3, nsr_m, s);
   const float2* twa[3] = {axis_tw(p, tw[0], 0), axis_tw(p, tw[1], 1), axis_tw(p, tw[2], 2)};
-  if (e == cudaSuccess) e = recon::launch_fft3(acc, p->f3.P3, twa, true, s);
-  if (e == cudaSuccess) e = recon::launch_crop_real(acc, volume, p->f3, s);
+  if (e == cudaSuccess)
+    e = recon::launch_grid_finish(acc, S, (double*)(b + L.stats), (float2*)(b + L.H), volume, p->f3, nsr_m, twa, s);
   if (e != cudaSuccess) return cuda_fail(e, "recon_grid_run");
   return RECON_OK;
 }

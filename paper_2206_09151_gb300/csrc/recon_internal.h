@@ -180,7 +180,7 @@ void describe_backproject(const BackprojConst& c, const DirParams* dirs, const v
 cudaError_t launch_backproject_persistent(const BatchBp* desc_dev, int n_desc, unsigned long long total,
                                           unsigned long long* counter, size_t smem, cudaStream_t stream);
 
-// The 3D-Fourier forms (fft3.cu, fourier.cu): a zero-padded complex grid [P3z][P3y][P3x]
+// The 3D-Fourier forms (fft3.cuh, fourier.cu): a zero-padded complex grid [P3z][P3y][P3x]
 // holding an n[0] x n[1] x n[2] volume at offset off (centred); scale[a] = P3[a] / P
 // converts a 2D frequency in units of 1 / (P delta) to bins of grid axis a.
 struct Fourier3Const {
@@ -197,16 +197,20 @@ struct GridDir {
   float qz_coef;
   uint64_t uR;
 };
-cudaError_t launch_fft3(float2* data, const int P3[3], const float2* const tw[3], bool inverse, cudaStream_t s);
-cudaError_t launch_swap_pack(const float* vc, const float* vs, float2* grid, const Fourier3Const& f, cudaStream_t s);
-cudaError_t launch_swap_phase(const float2* Z, float2* out, const Fourier3Const& f, double R, double sigma, double eps,
-                              double cs, cudaStream_t s);
-cudaError_t launch_crop_real(const float2* grid, float* vol, const Fourier3Const& f, cudaStream_t s);
+// Eq. 12: the spectrum Z of V_c + i V_s; then, per (sigma, eps), the CTF inversion of it into the
+// volume through the half spectrum H (swap_half_cells complex cells).  tw: FFT twiddles per axis.
+cudaError_t launch_swap_forward(const float* vc, const float* vs, float2* Z, const Fourier3Const& f,
+                                const float2* const tw[3], cudaStream_t s);
+cudaError_t launch_swap_phase(const float2* Z, float2* H, float* vol, const Fourier3Const& f, double R, double sigma,
+                              double eps, double cs, const float2* const tw[3], cudaStream_t s);
+size_t swap_half_cells(const Fourier3Const& f);
+// The gridding: acc holds per cell of the padded grid a float4 (gridded bracket x contrast, gridded
+// contrast; with_raw) or a float2 (the first alone), S its weight; H: grid_half_cells complex cells.
 cudaError_t launch_grid_splat(const float2* G, const GridDir* dirs, int dir_begin, int n_dirs, const StageAConst& c,
-                              const Fourier3Const& f, float2* acc, float2* raw, float* S, bool with_raw,
-                              cudaStream_t s);
-cudaError_t launch_grid_finish(float2* acc, const float2* raw, const float* S, double* stats, const Fourier3Const& f,
-                               float nsr_m, cudaStream_t s);
+                              const Fourier3Const& f, void* acc, float* S, bool with_raw, cudaStream_t s);
+cudaError_t launch_grid_finish(const void* acc, const float* S, double* stats, float2* H, float* vol,
+                               const Fourier3Const& f, float nsr_m, const float2* const tw[3], cudaStream_t s);
+size_t grid_half_cells(const Fourier3Const& f);
 
 // Whole-operator run with its workspace carved from `scratch` (tables first, then
 // the largest direction block that fits); used by recon_run_noalloc.

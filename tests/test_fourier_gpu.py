@@ -79,3 +79,34 @@ def test_gridding_noise_filter_matches_oracle():
     r.close()
     ref = F.recon_gridding(img, rot, lam=lam, delta=1e-9, defocus=Rs, grid=grid, sigma=0.3, eps=1e-2, nsr=1e-2)
     assert rel_l2(got, ref) <= 1e-3, rel_l2(got, ref)
+
+
+@pytest.mark.parametrize("grid", [(1, 5, 9), (17, 3, 33), (300, 2, 3), (2, 3, 520)])
+def test_line_transforms_of_every_length_match_oracle(grid):
+    """Grid sides whose padded lengths run from 2 to 2048 (a thread per line, the 8-value and
+    the 16-value transform), odd sides (a last unpaired line of the complex-to-real pass) and
+    sides that leave part of a thread block without lines.  Both forms, the gridding on the
+    grids whose cells are near the images' bins."""
+    from paper_2206_09151_gb300.recon import Reconstructor
+    nu, nv, D, lam = 21, 18, 7, 4e-10
+    rng = np.random.default_rng(5)
+    img = (1.0 + 0.05 * rng.standard_normal((D, nv, nu))).astype(np.float32)
+    Rs = np.full(D, 20e-9)
+    kw = dict(lam=lam, delta=1e-9, defocus=Rs, nz_layers=3)
+    rot = ph.single_axis_rotations(D, span=2 * math.pi, start=0.1)
+    r = Reconstructor(rot, nu, nv, grid, sigma=0.3, eps=1e-2, filter="pair", **kw)
+    got = r.swap_phase(r.swap_ct(torch.from_numpy(img).cuda()), 0.3, 1e-2).cpu().numpy()
+    r.close()
+    vc, vs = F.swap_ct(img, rot, grid=grid, **kw)
+    ref = F.swap_phase(vc, vs, lam=lam, delta=1e-9, defocus=20e-9, sigma=0.3, eps=1e-2)
+    assert rel_l2(got, ref) <= TOL_F32, rel_l2(got, ref)
+    if max(grid) > 64:
+        # a 64-bin image spectrum stretched over 1024 or 2048 cells: the float32 coordinates of the
+        # splat (up to 1000 cells, 6e-5 cell of rounding) are further off than the transforms
+        return
+    rot = ph.cone_rotations(D, 60.0, seed=3)
+    r = Reconstructor(rot, nu, nv, grid, sigma=0.3, eps=1e-2, ramp="density", **kw)
+    got = r.grid_run(torch.from_numpy(img).cuda()).cpu().numpy()
+    r.close()
+    ref = F.recon_gridding(img, rot, lam=lam, delta=1e-9, defocus=Rs, grid=grid, sigma=0.3, eps=1e-2)
+    assert rel_l2(got, ref) <= TOL_F32, rel_l2(got, ref)
