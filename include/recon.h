@@ -96,7 +96,12 @@ extern "C" {
 #define RECON_BP_AUTO 0          /* the variant measured faster on sm_103a: DIRECT for a
                                     single axis along y with the nearest layer, TMA for
                                     every other case where its footprint box fits shared
-                                    memory (else the general direct kernel)              */
+                                    memory (else the general direct kernel).  Whole runs
+                                    of the first kind (recon_run and its forms, the batch)
+                                    keep single values along the detector columns instead
+                                    of tap pairs between the two stages where that layout
+                                    fits; its kernel's bounded waits leave NaN if one runs
+                                    out, and the call stays asynchronous                  */
 #define RECON_BP_DIRECT 1        /* bilinear gathers straight from the stack (single-axis
                                     kernel, or the general kernel)                       */
 #define RECON_BP_STAGED 2        /* single-axis: footprint staged in shared memory        */

@@ -670,7 +670,7 @@ cudaError_t launch_backproject(const BackprojConst& c, const DirParams* dirs, co
                                                                         accumulate, stream));
 }
 
-void describe_backproject(const BackprojConst& c, const DirParams* dirs, const void* stack, int dir_begin,
+cudaError_t describe_backproject(const BackprojConst& c, const DirParams* dirs, const void* stack, int dir_begin,
                           int dir_count, float* volume, int accumulate, BatchBp* out) {
   out->c = c;
   out->dirs = dirs;
@@ -679,6 +679,9 @@ void describe_backproject(const BackprojConst& c, const DirParams* dirs, const v
   out->dir_begin = dir_begin;
   out->dir_count = dir_count;
   out->accumulate = accumulate;
+  if (c.cols_j) {
+    return describe_backproject_cols(c, out);
+  }
   const bool axis = c.axis_y && !c.layer_linear;
   if (axis) {
     out->kind = 2 + (c.stack_bf16 ? 2 : 0) + (c.b_frac != 0.f ? 1 : 0);
@@ -692,6 +695,7 @@ void describe_backproject(const BackprojConst& c, const DirParams* dirs, const v
     out->gz = (c.nz + kTZ - 1) / kTZ;
   }
   out->smem = (size_t)dir_count * (axis ? sizeof(AxisDir) : sizeof(TileDir));
+  return cudaSuccess;
 }
 
 cudaError_t launch_backproject_persistent(const BatchBp* desc_dev, int n_desc, unsigned long long total,

@@ -23,15 +23,13 @@
 //    a status word in device memory and the thread stops; the producer then waits (again
 //    bounded) for its copies in flight before the CTA exits.  A box that the footprint
 //    does not fit (cannot happen for boxes sized by tma_box_for) sets bit 1.
-#include <cuda.h>
-#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
 #include <cstdint>
-#include <mutex>
 
 #include "recon_internal.h"
+#include "tma.cuh"
 
 namespace recon {
 namespace {
@@ -52,10 +50,7 @@ namespace {
 constexpr int kMX = 16, kMY = 16;
 constexpr int kConsumerWarps = 8;
 constexpr int kThreads = (kConsumerWarps + 1) * 32;
-constexpr unsigned long long kWaitNs = 2000000000ull;  // bounded waits: 2 s
 constexpr long long kMargin = 1LL << 30;               // 2^-10 pixel in 2^-40 pixel units
-// a waiting thread may be suspended up to this long (it resumes when the phase completes)
-constexpr uint32_t kSuspendNs = 20000;
 
 struct alignas(16) Rec {  // per item, written by the producer (64 bytes)
   float a, b;       // box-local tile-origin coordinates (+1 - box origin, pixels)
@@ -67,48 +62,6 @@ struct alignas(16) Rec {  // per item, written by the producer (64 bytes)
 };
 static_assert(sizeof(Rec) == 64, "Rec layout");
 
-__device__ __forceinline__ unsigned long long now_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(kSuspendNs)
-      : "memory");
-  return ok != 0;
-}
-// Wait for the phase with the given parity to complete; false after kWaitNs.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = now_ns();
-  for (;;) {
-    if (mbar_try(bar, parity)) return true;
-    if (now_ns() - t0 > kWaitNs) return false;
-  }
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
-                                            uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
-      "[%6];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
-      : "memory");
-}
 __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
   uint32_t v;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a));
@@ -408,19 +361,6 @@ __global__ void __launch_bounds__(kThreads, RECON_TMA_MIN_CTAS) k_backproject_tm
       for (int q = 0; q < kMZ / 2; ++q) acc[q] = make_float2(0.f, 0.f);
     }
   }
-}
-
-PFN_cuTensorMapEncodeTiled_v12000 encode_tiled() {
-  static std::once_flag once;
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  std::call_once(once, [] {
-    void* f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
-  });
-  return fn;
 }
 
 template <typename ST, bool LIN, int kMZ>

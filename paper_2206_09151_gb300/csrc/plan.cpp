@@ -91,8 +91,10 @@ struct recon_plan_s {
   std::vector<float> theta, cnt, x2;  // learned regulariser: weights, bin counts, defocus feature
   recon::LearnConst lc;
   bool training = false;
-  recon::StageAConst ca;
+  recon::StageAConst ca;       // of whole runs (column stacks where the scan takes them)
+  recon::StageAConst ca_pair;  // of recon_filter_stage, whose layout is the tap pairs
   recon::BackprojConst cb;
+  int t_rows = 0;              // rows of T: nv, or the column stack's where those are more
   recon::TmaBox tma{};   // footprint box of the TMA-staged backprojection
   bool use_tma = false;  // stage B runs k_backproject_tma
   // workspace layout (byte offsets)
@@ -500,6 +502,24 @@ static int plan_create(const recon_geometry* geom, double lambda, double delta, 
   cb.staged = o.bp_kernel == RECON_BP_STAGED;
   cb.layer_linear = o.layer_interp == RECON_LAYER_LINEAR;
   cb.warp_cols = o.bp_warp ? o.bp_warp : 8;
+  // Column stacks (backproject_cols.cuh) where AUTO would run the single-axis kernel on tap pairs and
+  // the scan fits them, measured against the pairs per whole run: 64^3 / 90 views 78 us (106), 151 x 133 x 141 /
+  // 151 views between detector rows 1051 (1564), 512 x 256 x 512 / 360 views / 1 layer 5459 (8177), 256^3 / 360
+  // views / 32 layers 7.9 ms (the same: most lines span layers there).  An explicit DIRECT or STAGED keeps the pairs.
+  ca.cols = 0;
+  ca.nw = p->nv;
+  ca.r_lo = ca.wp = 0;
+  ca.b_frac = 0.f;
+  p->ca_pair = ca;
+  if (o.bp_kernel == RECON_BP_AUTO && P >= 16 && !training) recon::cols_setup(cb, p->dirs.data(), D);
+  if (cb.cols_j) {
+    ca.cols = 1;
+    ca.nw = cb.nw;
+    ca.r_lo = cb.j_lo + cb.b_int;
+    ca.wp = cb.wp;
+    ca.b_frac = cb.b_frac;
+  }
+  p->t_rows = std::max(p->nv, ca.nw);
   // The TMA-staged kernel where the general kernel would run (any geometry but a single
   // axis along y, or the layer blend), measured faster on sm_103a; on request for any geometry.
   const bool general = !cb.axis_y || cb.layer_linear;
@@ -550,9 +570,9 @@ static int plan_create(const recon_geometry* geom, double lambda, double delta, 
     }
   }
   const size_t elem = ca.stack_bf16 ? 4 : 8;  // one tap pair
-  p->stack_dir_bytes = (size_t)nz_layers * ca.layer_elems * elem;
+  p->stack_dir_bytes = (size_t)nz_layers * std::max(ca.layer_elems * elem, (size_t)p->nu * ca.wp * (elem / 2));
   // S and T of one direction (the stage-A intermediates)
-  const size_t inter_dir = (size_t)p->nv * p->half * 8 * (1 + (size_t)nz_layers);
+  const size_t inter_dir = (size_t)p->half * 8 * (p->nv + (size_t)p->t_rows * nz_layers);
   const size_t per_dir = inter_dir + p->stack_dir_bytes;
   // Where one direction's intermediates are large (big images, many layers), stage A runs
   // in sub-blocks whose intermediates fit 2 GiB by default (two directions of 1024^2 images
@@ -623,7 +643,7 @@ static int plan_create(const recon_geometry* geom, double lambda, double delta, 
   p->off_S = off;
   off = align256(off + (size_t)ca.sub_block * p->nv * p->half * 8);
   p->off_T = off;
-  off = align256(off + (size_t)ca.sub_block * nz_layers * p->nv * p->half * 8);
+  off = align256(off + (size_t)ca.sub_block * nz_layers * p->t_rows * p->half * 8);
   p->off_stack = off;
   off = align256(off + (size_t)db * p->stack_dir_bytes);
   p->off_pow = off;
@@ -634,6 +654,7 @@ static int plan_create(const recon_geometry* geom, double lambda, double delta, 
     off = align256(off + sizeof(float) * (size_t)ca.sub_block * nz_layers * p->lc.n_bins);
   }
   p->ws_bytes = off;
+  p->ca_pair.sub_block = ca.sub_block;
   if (o.filter == RECON_FILTER_MLP && !training && P < 16) {
     delete p;
     return fail(RECON_E_UNSUPPORTED_SIZE, "recon_plan: the learned filter needs images of more than 4 pixels");
@@ -794,6 +815,7 @@ unsigned int* tma_status(recon_plan_t p, void* ws) { return (unsigned int*)((cha
 // Stage B of one direction block through the plan's backprojection kernel.
 cudaError_t backproject_block(recon_plan_t p, const recon::DirParams* dirs, const void* stack, int d0, int cnt,
                               float* vol, int accumulate, void* ws, cudaStream_t s) {
+  if (p->cb.cols_j) return recon::launch_backproject_cols(p->cb, dirs, stack, d0, cnt, vol, accumulate, s);
   if (p->use_tma)
     return recon::launch_backproject_tma(p->cb, p->tma, dirs, stack, d0, cnt, vol, accumulate, tma_status(p, ws), s);
   return recon::launch_backproject(p->cb, dirs, stack, d0, cnt, vol, accumulate, s);
@@ -998,7 +1020,7 @@ int recon_filter_stage(recon_plan_t p, const float* images, int dir_begin, int d
   if (rc) return rc;
   MlpHookCtx hctx{p, (const char*)workspace, (float*)((char*)workspace + p->off_pow), w.eps, w.S, w.twp};
   const recon::StageAHook hook{mlp_hook, &hctx};
-  cudaError_t e = recon::launch_stage_a(p->ca, w, images, dir_begin, dir_count, s, nullptr,
+  cudaError_t e = recon::launch_stage_a(p->ca_pair, w, images, dir_begin, dir_count, s, nullptr,
                                         p->ca.filter == RECON_FILTER_MLP ? &hook : nullptr);
   if (e != cudaSuccess) return cuda_fail(e, "recon_filter_stage: launch");
   *stack_out = w.stack;
@@ -1028,7 +1050,10 @@ int recon_backproject(recon_plan_t p, const void* stack, int dir_begin, int dir_
   if (rc) return rc;
   rc = tma_begin(p, workspace, s, "recon_backproject");
   if (rc) return rc;
-  cudaError_t e = backproject_block(p, w.dirs, stack, dir_begin, dir_count, volume, accumulate, workspace, s);
+  // the caller's stack holds tap pairs (recon_filter_stage's layout)
+  cudaError_t e = p->cb.cols_j
+                      ? recon::launch_backproject(p->cb, w.dirs, stack, dir_begin, dir_count, volume, accumulate, s)
+                      : backproject_block(p, w.dirs, stack, dir_begin, dir_count, volume, accumulate, workspace, s);
   if (e != cudaSuccess) return cuda_fail(e, "recon_backproject: launch");
   return tma_end(p, workspace, s, "recon_backproject");
 }
@@ -1342,7 +1367,7 @@ int run_in_scratch(recon_plan_t p, const float* images, float* volume, char* scr
   // Same table head as the caller-owned workspace, then the largest direction block
   // whose spectra, intermediates and stacks still fit the scratch.
   const size_t spec = (size_t)p->nv * p->half * 8;
-  const size_t inter = spec * p->nzl;
+  const size_t inter = (size_t)p->t_rows * p->half * 8 * p->nzl;
   const bool mlp = p->ca.filter == RECON_FILTER_MLP;
   const size_t sub = (size_t)(p->ca.sub_block > 0 ? p->ca.sub_block : 1);
   auto need = [&](size_t db) {
@@ -1401,7 +1426,10 @@ int run_in_scratch(recon_plan_t p, const float* images, float* volume, char* scr
     const int cnt = (p->D - d0) < (int)db ? (p->D - d0) : (int)db;
     cudaError_t e = recon::launch_stage_a(ca, w, images, d0, cnt, s, nullptr, mlp ? &hook : nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "recon_run_noalloc: stage A launch");
-    e = recon::launch_backproject(p->cb, w.dirs, w.stack, d0, cnt, volume, p->opt.accumulate || b > 0, s);
+    // direct kernels only: no wait inside the GPU, so the call need not synchronise
+    e = p->cb.cols_j ? recon::launch_backproject_cols(p->cb, w.dirs, w.stack, d0, cnt, volume,
+                                                      p->opt.accumulate || b > 0, s)
+                     : recon::launch_backproject(p->cb, w.dirs, w.stack, d0, cnt, volume, p->opt.accumulate || b > 0, s);
     if (e != cudaSuccess) return cuda_fail(e, "recon_run_noalloc: backprojection launch");
   }
   return RECON_OK;
@@ -1579,9 +1607,13 @@ struct recon_batch_s {
   int n = 0, dbb = 0, n_rounds = 0;
   std::vector<recon_plan_t> plans;
   std::vector<size_t> off_tables, off_stack;
-  size_t off_S = 0, off_T = 0, off_pow = 0, off_eps = 0, off_desc = 0, off_ctr = 0, ws_bytes = 0, smem = 0;
-  std::vector<recon::BatchBp> desc;        // [n_rounds][n] (first round_count[r] used)
-  std::vector<int> round_count;
+  size_t off_S = 0, off_T = 0, off_pow = 0, off_eps = 0, off_desc = 0, off_ctr = 0, ws_bytes = 0;
+  // classes of tomograms, a kernel each: tap pairs, column stacks with 64-row and with 32-row tiles
+  static constexpr int kClasses = 3;
+  static int class_of(recon_plan_t p) { return p->cb.cols_j == 0 ? 0 : (p->cb.cols_j == 64 ? 1 : 2); }
+  size_t smem[kClasses] = {};
+  std::vector<recon::BatchBp> desc;        // [n_rounds][n]: a round's tomograms by class
+  std::vector<int> round_count;            // [n_rounds][kClasses]
   std::vector<unsigned long long> round_total;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
@@ -1619,23 +1651,27 @@ int batch_prepare(recon_batch_t bt, const float* const* images, float* const* vo
     if (rc) return rc;
   }
   for (int r = 0; r < bt->n_rounds; ++r) {
-    unsigned long long first = 0;
     int cntr = 0;
-    for (int q = 0; q < bt->n; ++q) {
-      recon_plan_t p = bt->plans[q];
-      const int d0 = r * bt->dbb;
-      if (d0 >= p->D) continue;
-      const int cnt = (p->D - d0) < bt->dbb ? (p->D - d0) : bt->dbb;
-      recon::BatchBp& d = bt->desc[(size_t)r * bt->n + cntr];
-      const recon::Workspace w = carve(p, base + bt->off_tables[q]);
-      recon::describe_backproject(p->cb, w.dirs, base + bt->off_stack[q], d0, cnt, volumes[q],
-                                  p->opt.accumulate || r > 0, &d);
-      d.first_item = first;
-      first += (unsigned long long)d.gx * d.gy * d.gz;
-      ++cntr;
+    for (int cls = 0; cls < bt->kClasses; ++cls) {
+      unsigned long long first = 0;
+      const int begin = cntr;
+      for (int q = 0; q < bt->n; ++q) {
+        recon_plan_t p = bt->plans[q];
+        const int d0 = r * bt->dbb;
+        if (d0 >= p->D || bt->class_of(p) != cls) continue;
+        const int cnt = (p->D - d0) < bt->dbb ? (p->D - d0) : bt->dbb;
+        recon::BatchBp& d = bt->desc[(size_t)r * bt->n + cntr];
+        const recon::Workspace w = carve(p, base + bt->off_tables[q]);
+        const cudaError_t e = recon::describe_backproject(p->cb, w.dirs, base + bt->off_stack[q], d0, cnt, volumes[q],
+                                                          p->opt.accumulate || r > 0, &d);
+        if (e != cudaSuccess) return cuda_fail(e, "recon_batch: tensor map");
+        d.first_item = first;
+        first += (unsigned long long)d.gx * d.gy * d.gz;
+        ++cntr;
+      }
+      bt->round_count[r * bt->kClasses + cls] = cntr - begin;
+      bt->round_total[r * bt->kClasses + cls] = first;
     }
-    bt->round_count[r] = cntr;
-    bt->round_total[r] = first;
   }
   cudaError_t e = cudaMemcpyAsync(base + bt->off_desc, bt->desc.data(), sizeof(recon::BatchBp) * bt->desc.size(),
                                   cudaMemcpyHostToDevice, s);
@@ -1719,9 +1755,15 @@ int batch_launch(recon_batch_t bt, const float* const* images, float* const* vol
       e = cudaEventRecord(bt->ev_free[r % 2], s);
       if (e != cudaSuccess) return cuda_fail(e, "recon_batch: slot release");
     }
-    e = recon::launch_backproject_persistent((const recon::BatchBp*)(base + bt->off_desc) + (size_t)r * bt->n,
-                                             bt->round_count[r], bt->round_total[r],
-                                             (unsigned long long*)(base + bt->off_ctr) + r, bt->smem, s);
+    const recon::BatchBp* desc = (const recon::BatchBp*)(base + bt->off_desc) + (size_t)r * bt->n;
+    const int* count = &bt->round_count[r * bt->kClasses];
+    const unsigned long long* total = &bt->round_total[r * bt->kClasses];
+    e = recon::launch_backproject_persistent(desc, count[0], total[0], (unsigned long long*)(base + bt->off_ctr) + r,
+                                             bt->smem[0], s);
+    if (e == cudaSuccess)
+      e = recon::launch_backproject_cols_persistent(desc + count[0], count[1], total[1], 64, bt->smem[1], s);
+    if (e == cudaSuccess)
+      e = recon::launch_backproject_cols_persistent(desc + count[0] + count[1], count[2], total[2], 32, bt->smem[2], s);
     if (e != cudaSuccess) return cuda_fail(e, "recon_batch: persistent backprojection launch");
   }
   return RECON_OK;
@@ -1756,7 +1798,7 @@ int recon_batch_create(int n, const recon_plan_t* plans, int dir_block, recon_ba
   bt->n = n;
   bt->plans.assign(plans, plans + n);
   bt->dbb = dir_block > 0 ? dir_block : 32;
-  size_t off = 0, maxS = 0, maxT = 0, maxpow = 0, maxeps = 0, smem = 0;
+  size_t off = 0, maxS = 0, maxT = 0, maxpow = 0, maxeps = 0;
   bt->off_tables.resize(n);
   bt->off_stack.resize(n);
   int rounds = 0;
@@ -1767,10 +1809,11 @@ int recon_batch_create(int n, const recon_plan_t* plans, int dir_block, recon_ba
     const size_t db = (size_t)bt->dbb;
     const size_t sb = std::min(db, (size_t)(p->ca.sub_block > 0 ? p->ca.sub_block : 1));
     maxS = std::max(maxS, sb * p->nv * p->half * 8);
-    maxT = std::max(maxT, sb * p->nzl * p->nv * p->half * 8);
+    maxT = std::max(maxT, sb * p->nzl * p->t_rows * p->half * 8);
     maxpow = std::max(maxpow, sb * p->lc.n_bins * 4);
     maxeps = std::max(maxeps, sb * p->nzl * p->lc.n_bins * 4);
-    smem = std::max(smem, db * 64);
+    size_t& smem = bt->smem[bt->class_of(p)];
+    smem = std::max(smem, p->cb.cols_j ? recon::cols_smem_bytes(p->cb) : db * 64);
     rounds = std::max(rounds, (p->D + bt->dbb - 1) / bt->dbb);
   }
   for (int q = 0; q < n; ++q) {
@@ -1791,7 +1834,6 @@ int recon_batch_create(int n, const recon_plan_t* plans, int dir_block, recon_ba
   bt->off_ctr = off;
   off = align256(off + sizeof(unsigned long long) * (size_t)(rounds > 0 ? rounds : 1));
   bt->ws_bytes = off;
-  bt->smem = smem;
   bt->off_img.resize(n);
   size_t soff = 0;
   for (int q = 0; q < n; ++q) {
@@ -1800,8 +1842,8 @@ int recon_batch_create(int n, const recon_plan_t* plans, int dir_block, recon_ba
   }
   bt->slot_bytes = soff;
   bt->desc.assign((size_t)rounds * n, recon::BatchBp{});
-  bt->round_count.assign(rounds, 0);
-  bt->round_total.assign(rounds, 0);
+  bt->round_count.assign(bt->kClasses * (size_t)rounds, 0);
+  bt->round_total.assign(bt->kClasses * (size_t)rounds, 0);
   *out = bt;
   return RECON_OK;
 }

@@ -4,6 +4,7 @@
 #include <cstddef>
 #include <cstdint>
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 struct recon_plan_s;
@@ -68,6 +69,12 @@ struct StageAConst {
   int su;               // stack row pitch in tap pairs, nu + 1
   size_t layer_elems;   // pairs per layer, (nv + 2) * (nu + 1)
   DensityConst dens;
+  // The stack's layout and rows.  cols = 0: tap pairs [n][k][nv + 2][su].  cols = 1 (single-axis scans
+  // about y, backproject_cols.cuh): single values [n][k][nu][wp], detector rows fastest.  T and
+  // the stack hold rows w = 0 .. nw - 1, detector row r_lo + w (b_frac = 0; with tap pairs r_lo = 0,
+  // nw = nv) or that row and the next blended with weight b_frac on the next.
+  int cols, nw, r_lo, wp;
+  float b_frac;
   int sub_block;        // directions per stage-A sub-block (S and T sized for it), 0 = whole block
   int pair_mode;        // filter 3 only: 0 the opposite-pair bracket; 1 / 2 the depth factor
                         // cos / sin of pi lambda z_k q^2 alone (the CT step of Eq. 12)
@@ -137,11 +144,21 @@ struct BackprojConst {
   float b_frac;   // b_off - floor(b_off), 0 or 1/2
   int staged;     // single-axis kernel with shared-memory staging of each footprint
   int layer_linear;  // blend the two layers whose centres bracket the depth (general kernel)
+  // column stack (backproject_cols.cuh): cols_j rows per tile (0: not used), the staged box of cols_w
+  // columns x cols_l layers in stages of cols_stage bytes; nw rows from volume row j_lo, wp entries apart
+  int cols_j, cols_w, cols_l, cols_stage, nw, j_lo, wp;
   int warp_cols;     // general kernel: a warp's patch of voxel columns is warp_cols x 32/warp_cols
 };
 
 cudaError_t launch_backproject(const BackprojConst& c, const DirParams* dirs, const void* stack, int dir_begin,
                                int dir_count, float* volume, int accumulate, cudaStream_t stream);
+
+// The column-stack backprojection of single-axis scans about y.  cols_setup fills c.cols_j,
+// cols_w, cols_l, cols_stage, nw, j_lo and wp (cols_j = 0 where the scan does not fit it).
+void cols_setup(BackprojConst& c, const DirParams* dirs, int n_dirs);
+size_t cols_smem_bytes(const BackprojConst& c);
+cudaError_t launch_backproject_cols(const BackprojConst& c, const DirParams* dirs, const void* stack, int dir_begin,
+                                    int dir_count, float* volume, int accumulate, cudaStream_t stream);
 
 // Footprint box of the TMA-staged backprojection: every (tile, direction) footprint of the
 // plan's directions fits W pairs x H rows x L layers of the stack.
@@ -163,8 +180,8 @@ cudaError_t launch_tma_wait_probe(void* buf, size_t buf_bytes, unsigned int* sta
 
 // One tomogram's share of a persistent batched backprojection: its constants, pointers,
 // kernel kind (general 0/1, single-axis 2..5 (float32 / bfloat16 stack, one or two detector
-// rows), general with the layer blend 6/7),
-// tile grid and the index of its first work item.
+// rows), general with the layer blend 6/7, column stack 8..11 (float32 / bfloat16, 64 or 32 rows per
+// tile)), tile grid and the index of its first work item.
 struct BatchBp {
   BackprojConst c;
   const DirParams* dirs;
@@ -173,12 +190,17 @@ struct BatchBp {
   int dir_begin, dir_count, accumulate, kind;
   int gx, gy, gz;
   unsigned long long first_item;
-  size_t smem;  // shared bytes its tiles need
+  size_t smem;      // shared bytes its tiles need
+  alignas(64) CUtensorMap map;  // kinds 8..11: the round's column stacks
 };
-void describe_backproject(const BackprojConst& c, const DirParams* dirs, const void* stack, int dir_begin,
+cudaError_t describe_backproject(const BackprojConst& c, const DirParams* dirs, const void* stack, int dir_begin,
                           int dir_count, float* volume, int accumulate, BatchBp* out);
 cudaError_t launch_backproject_persistent(const BatchBp* desc_dev, int n_desc, unsigned long long total,
                                           unsigned long long* counter, size_t smem, cudaStream_t stream);
+// The tomograms of kinds 8..11 run in kernels of their own, one for 64-row and one for 32-row tiles (`rows`).
+cudaError_t describe_backproject_cols(const BackprojConst& c, BatchBp* out);
+cudaError_t launch_backproject_cols_persistent(const BatchBp* desc_dev, int n_desc, unsigned long long total, int rows,
+                                               size_t smem, cudaStream_t stream);
 
 // The 3D-Fourier forms (fft3.cuh, fourier.cu): a zero-padded complex grid [P3z][P3y][P3x]
 // holding an n[0] x n[1] x n[2] volume at offset off (centred); scale[a] = P3[a] / P

@@ -117,13 +117,64 @@ __global__ void __launch_bounds__(kThreads) k_rows_fwd(const float* __restrict__
   }
 }
 
+// Column stacks whose volume rows fall between two detector rows: row w is detector rows r_lo + w and
+// the next blended, zero outside the detector (the blend commutes with the row transform, so it
+// is done on the column's values, once per stack entry instead of once per voxel).
+template <class Idx>
+__device__ __forceinline__ void store_blended(const float2* buf, float2* out, const StageAConst& c, int j, int step,
+                                              Idx idx) {
+  for (int w = j; w < c.nw; w += step) {
+    const int r = w + c.r_lo;
+    const float2 a = r >= 0 && r < c.nv ? buf[idx(r)] : make_float2(0.f, 0.f);
+    const float2 b = r + 1 >= 0 && r + 1 < c.nv ? buf[idx(r + 1)] : make_float2(0.f, 0.f);
+    out[w] = make_float2(fmaf(c.b_frac, b.x - a.x, a.x), fmaf(c.b_frac, b.y - a.y, a.y));
+  }
+}
+
+// Column-stack rows (backproject_cols.cuh) from the G row pairs of a CTA: `pairs` holds (row 2g, row
+// 2g + 1) of pair g at column u, at entry u G + (g ^ swizzle(u)), so that the stores of 16
+// consecutive columns and the 16-byte loads of two neighbouring pairs are free of bank conflicts;
+// `out` is the layer's entry of column 0 and the CTA's first row.  Rows up to the padded length wp
+// are written (zeros past the last row), 32 contiguous bytes per column for float32 and G = 4.
+template <int G>
+__device__ __forceinline__ int col_swizzle(int u) {
+  constexpr int sh = G >= 16 ? 0 : (G == 8 ? 1 : (G == 4 ? 2 : 3));
+  return (u >> sh) & ((G < 16 ? G : 16) - 1);
+}
+template <int G, int NTH>
+__device__ __forceinline__ void store_columns(const float2* pairs, float* out, int nu, int rows_left, int wp) {
+  constexpr int U = G / 2;  // 16-byte units per column
+  for (int q = threadIdx.x; q < nu * U; q += NTH) {
+    const int h = q % U, u = q / U, sw = col_swizzle<G>(u);
+    if (4 * h >= rows_left) continue;
+    const float4 v = *reinterpret_cast<const float4*>(pairs + u * G + ((2 * h) ^ (sw & ~1)));
+    *reinterpret_cast<float4*>(out + (size_t)u * wp + 4 * h) = sw & 1 ? make_float4(v.z, v.w, v.x, v.y) : v;
+  }
+}
+template <int G, int NTH>
+__device__ __forceinline__ void store_columns(const float2* pairs, __nv_bfloat16* out, int nu, int rows_left, int wp) {
+  constexpr int U = G / 4;
+  for (int q = threadIdx.x; q < nu * U; q += NTH) {
+    const int h = q % U, u = q / U, sw = col_swizzle<G>(u);
+    if (8 * h >= rows_left) continue;
+    __nv_bfloat162 b[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 v = pairs[u * G + ((4 * h + e) ^ sw)];
+      b[e] = __floats2bfloat162_rn(v.x, v.y);
+    }
+    *reinterpret_cast<uint4*>(out + (size_t)u * wp + 8 * h) = *reinterpret_cast<const uint4*>(b);
+  }
+}
+
 // FILT: 0 ramp only (filter off), 1 Tikhonov eps, 2 learned eps table, 3 the opposite-pair
 // form of Eq. 10 / 11 (real part of the complex bracket at the image plane carried to the
 // layer depth); DENS: density
 // weighting (any geometry) instead of the ramp.  Compile-time, so that each variant keeps
 // only the registers it uses.
 // 3 resident CTAs per SM (80 registers) measured faster than 4 (64 registers) at P = 512.
-template <int P, int FILT, bool DENS>
+// BLEND: rows between two detector rows (c.b_frac != 0).
+template <int P, int FILT, bool DENS, bool BLEND>
 __global__ void __launch_bounds__(kThreads, 3) k_cols(const float2* __restrict__ S, float2* __restrict__ T,
                                                     const float2* __restrict__ twg, const uint64_t* __restrict__ uA,
                                                     const float* __restrict__ ramp, const DirParams* __restrict__ dirs,
@@ -225,7 +276,11 @@ __global__ void __launch_bounds__(kThreads, 3) k_cols(const float2* __restrict__
       cp[s] = c.pair_mode == 0 ? __fdividef(cs, fmaf(cs, cs, c.eps)) : (c.pair_mode == 1 ? 0.f : -1.f);
     }
   }
-  float2* Tn = T + (size_t)n * c.nz_layers * c.half * c.nv;
+  // this thread's rows w = j + s TT - r_lo of T (s < 4: nv <= P/2), stored where 0 <= w < nw
+  float2* Tj = T + ((size_t)n * c.nz_layers * c.half + col) * c.nw + (BLEND ? 0 : j - c.r_lo);
+  bool keep[4];
+#pragma unroll
+  for (int s = 0; s < 4; ++s) keep[s] = ok && (unsigned)(j + s * TT - c.r_lo) < (unsigned)c.nw;
   // this CTA's layers: group blockIdx.z of gridDim.z equal groups
   const int lg = (c.nz_layers + gridDim.z - 1) / gridDim.z;
   const int k_begin = blockIdx.z * lg;
@@ -253,19 +308,24 @@ __global__ void __launch_bounds__(kThreads, 3) k_cols(const float2* __restrict__
       x[s] = make_float2(xg[s].x * f, xg[s].y * f);
     }
     fft::block_fft<P, true>(x, buf, tw, j, gsync);
-    if (ok) {
-      float2* out = Tn + ((size_t)k * c.half + col) * c.nv;
-      // nv <= P/2: elements s >= 4 (v >= P/2) are never kept (their last butterflies drop)
+    float2* out = Tj + (size_t)k * c.half * c.nw;
+    if constexpr (!BLEND) {
+      // elements s >= 4 (v >= P/2) are never kept (their last butterflies drop)
 #pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        const int v = j + s * TT;
-        if (v < c.nv) out[v] = x[s];
-      }
+      for (int s = 0; s < 4; ++s)
+        if (keep[s]) out[s * TT] = x[s];
+    } else {
+      gsync();  // the transform's last reads of the buffer
+#pragma unroll
+      for (int s = 0; s < 4; ++s) buf[padded(j + s * TT)] = x[s];
+      gsync();
+      if (ok) store_blended(buf, out, c, j, TT, [](int v) { return padded(v); });
     }
   }
 }
 
-template <int P, typename PairT>
+// PairT: the stack's entry, a tap pair (float2, bfloat162) or with COLS a single value.
+template <int P, typename PairT, bool COLS>
 __global__ void __launch_bounds__(kThreads) k_rows_inv(const float2* __restrict__ T, PairT* __restrict__ stack,
                                                         const float2* __restrict__ twg, StageAConst c) {
   constexpr int TT = P / 8, G = groups_per_cta<P>(), L = fft::buffer_len(P, G), H = P / 2 + 1;
@@ -279,14 +339,14 @@ __global__ void __launch_bounds__(kThreads) k_rows_inv(const float2* __restrict_
   __shared__ float2 tw[NT];
   // the half-spectrum tile is read once, before the FFT's first exchange: the
   // exchange buffer reuses its memory
-  __shared__ float2 shared_mem[TILE > BUF ? TILE : BUF];
+  __shared__ __align__(16) float2 shared_mem[TILE > BUF ? TILE : BUF];
   float2* tile = shared_mem;
   const int g = threadIdx.x / TT, j = threadIdx.x % TT;
   float2* buf = shared_mem + g * L;
   for (int i = threadIdx.x; i < NT; i += kThreads) tw[i] = twg[i];
   const int n = blockIdx.z, k = blockIdx.y;
   const int vbase = blockIdx.x * 2 * G;
-  const float2* Tk = T + ((size_t)n * c.nz_layers + k) * H * c.nv;
+  const float2* Tk = T + ((size_t)n * c.nz_layers + k) * H * c.nw;
   {  // all loads in flight before the shared stores
     float2 tmp[FILL];
 #pragma unroll
@@ -294,7 +354,7 @@ __global__ void __launch_bounds__(kThreads) k_rows_inv(const float2* __restrict_
       const int idx = threadIdx.x + it * kThreads;
       const int vv = idx % (2 * G), cc = idx / (2 * G);
       const int v = vbase + vv;
-      tmp[it] = (idx < USED && v < c.nv) ? Tk[(size_t)cc * c.nv + v] : make_float2(0.f, 0.f);
+      tmp[it] = (idx < USED && v < c.nw) ? Tk[(size_t)cc * c.nw + v] : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int it = 0; it < FILL; ++it) {
@@ -333,6 +393,17 @@ __global__ void __launch_bounds__(kThreads) k_rows_inv(const float2* __restrict_
   // u < P/2 only, i.e. x[s] for s < 4, so the last pass's butterflies feeding s >= 4 drop;
   // column P/2 (s = 4, thread 0, when nu = P/2) is (Y[nu - 1], 0)
   __syncthreads();
+  if constexpr (COLS) {
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      const int u = j + s * TT;
+      shared_mem[u * G + (g ^ col_swizzle<G>(u))] = x[s];
+    }
+    __syncthreads();
+    store_columns<G, kThreads>(shared_mem, stack + ((size_t)n * c.nz_layers + k) * c.nu * c.wp + vbase, c.nu,
+                               c.wp - vbase, c.wp);
+    return;
+  } else {
 #pragma unroll
   for (int s = 0; s < 4; ++s) buf[padded(j + s * TT)] = x[s];
   __syncthreads();
@@ -357,6 +428,7 @@ __global__ void __launch_bounds__(kThreads) k_rows_inv(const float2* __restrict_
     for (int i = threadIdx.x; i < sp; i += kThreads) Lk[i] = make_pair<PairT>(0.f, 0.f);
   if (vbase + 2 * G >= c.nv)  // bottom border row
     for (int i = threadIdx.x; i < sp; i += kThreads) Lk[(size_t)(c.nv + 1) * sp + i] = make_pair<PairT>(0.f, 0.f);
+  }
 }
 
 
@@ -376,7 +448,7 @@ __host__ __device__ constexpr int cols16_per_cta() {
 // The forward FFT along v stays in registers, multiplied once by the column's weight (ramp
 // or density weight, with the filter prefactor and 1/P^2); per layer: the CTF filter,
 // inverse FFT, store v < nv.
-template <int P, int FILT, bool DENS>
+template <int P, int FILT, bool DENS, bool BLEND>
 __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const float2* __restrict__ S, float2* __restrict__ T,
                                                           const float2* __restrict__ twg,
                                                           const uint64_t* __restrict__ uA,
@@ -387,7 +459,7 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
                                                           const float* __restrict__ eps_tab, int n_bins,
                                                           int bin_width, StageAConst c, int dir_begin) {
   constexpr int TT = P / 16, CB = cols16_per_cta<P>(), L = fft16::buffer_len(P), NT = fft16::table_len(P);
-  extern __shared__ float2 smem16[];
+  extern __shared__ __align__(16) float2 smem16[];
   float2* tw = smem16;
   const int g = threadIdx.x / TT, j = threadIdx.x % TT;
   float2* buf0 = smem16 + NT + (2 * g) * L;
@@ -467,7 +539,12 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
       cp[s] = c.pair_mode == 0 ? __fdividef(cs, fmaf(cs, cs, c.eps)) : (c.pair_mode == 1 ? 0.f : -1.f);
     }
   }
-  float2* Tn = T + (size_t)n * c.nz_layers * c.half * c.nv;
+  // this thread's rows w = j + s TT - r_lo of T (s < 8: nv <= P/2, P being at least twice the image
+  // size), stored where 0 <= w < nw
+  float2* Tj = T + ((size_t)n * c.nz_layers * c.half + col) * c.nw + (BLEND ? 0 : j - c.r_lo);
+  bool keep[8];
+#pragma unroll
+  for (int s = 0; s < 8; ++s) keep[s] = ok && (unsigned)(j + s * TT - c.r_lo) < (unsigned)c.nw;
   const int lg = (c.nz_layers + gridDim.z - 1) / gridDim.z;
   const int k_begin = blockIdx.z * lg;
   const int k_end = min(c.nz_layers, k_begin + lg);
@@ -497,20 +574,25 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
       }
     }
     fft16::group_fft_db<P, true>(x, buf0, buf1, tw, j, gsync);
-    if (ok) {
-      float2* out = Tn + ((size_t)k * c.half + col) * c.nv;
-      // nv <= P/2 (P is at least twice the image size): elements s >= 8 (v >= P/2) are
-      // never kept, so the last pass's butterflies that only feed them are dropped
+    float2* out = Tj + (size_t)k * c.half * c.nw;
+    if constexpr (!BLEND) {
+      // elements s >= 8 (v >= P/2) are never kept, so the last pass's butterflies that only feed them are
+      // dropped
 #pragma unroll
-      for (int s = 0; s < 8; ++s) {
-        const int v = j + s * TT;
-        if (v < c.nv) out[v] = x[s];
-      }
+      for (int s = 0; s < 8; ++s)
+        if (keep[s]) out[s * TT] = x[s];
+    } else {
+      // the transform's second pass, before its last barrier, was the last to read buf0
+#pragma unroll
+      for (int s = 0; s < 8; ++s) buf0[fft16::pad(j + s * TT)] = x[s];
+      gsync();
+      if (ok) store_blended(buf0, out, c, j, TT, [](int v) { return fft16::pad(v); });
+      gsync();  // the next transform's first pass writes buf0
     }
   }
 }
 
-template <int P, int FILT, bool DENS>
+template <int P>
 constexpr size_t cols16_smem() {
   return sizeof(float2) * ((size_t)fft16::table_len(P) + 2 * (size_t)cols16_per_cta<P>() * fft16::buffer_len(P));
 }
@@ -540,7 +622,7 @@ constexpr size_t rows16_smem() {
   return sizeof(float2) * ((size_t)fft16::table_len(P) + (tile > bufs ? tile : bufs));
 }
 
-template <int P, typename PairT>
+template <int P, typename PairT, bool COLS>
 __global__ void __launch_bounds__(rows16_threads<P>(), 2) k_rows_inv16(const float2* __restrict__ T,
                                                                         PairT* __restrict__ stack,
                                                                         const float2* __restrict__ twg,
@@ -549,7 +631,7 @@ __global__ void __launch_bounds__(rows16_threads<P>(), 2) k_rows_inv16(const flo
   constexpr int ROWS = 2 * kRowPairs16, L = fft16::buffer_len(P), NT = fft16::table_len(P);
   constexpr int USED = ROWS * H;
   constexpr int FILL = (USED + NTH - 1) / NTH;
-  extern __shared__ float2 smem16[];
+  extern __shared__ __align__(16) float2 smem16[];
   float2* tw = smem16;
   // the half-spectrum tile is read once, before the first exchange: the exchange buffers
   // reuse its memory
@@ -559,7 +641,7 @@ __global__ void __launch_bounds__(rows16_threads<P>(), 2) k_rows_inv16(const flo
   for (int i = threadIdx.x; i < NT; i += NTH) tw[i] = twg[i];
   const int n = blockIdx.z, k = blockIdx.y;
   const int vbase = blockIdx.x * ROWS;
-  const float2* Tk = T + ((size_t)n * c.nz_layers + k) * H * c.nv;
+  const float2* Tk = T + ((size_t)n * c.nz_layers + k) * H * c.nw;
   {  // all loads in flight before the shared stores
     float2 tmp[FILL];
 #pragma unroll
@@ -567,7 +649,7 @@ __global__ void __launch_bounds__(rows16_threads<P>(), 2) k_rows_inv16(const flo
       const int idx = threadIdx.x + it * NTH;
       const int vv = idx % ROWS, cc = idx / ROWS;
       const int v = vbase + vv;
-      tmp[it] = (idx < USED && v < c.nv) ? Tk[(size_t)cc * c.nv + v] : make_float2(0.f, 0.f);
+      tmp[it] = (idx < USED && v < c.nw) ? Tk[(size_t)cc * c.nw + v] : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int it = 0; it < FILL; ++it) {
@@ -602,6 +684,19 @@ __global__ void __launch_bounds__(rows16_threads<P>(), 2) k_rows_inv16(const flo
   __syncthreads();  // every group has read its rows: the tile is free for the exchange buffers
   const fft::GroupSync gsync{1 + g, TT};
   fft16::group_fft_sb<P, true, fft::GroupSync, true>(x, buf, tw, j, gsync);
+  if constexpr (COLS) {
+    constexpr int G = kRowPairs16;
+    __syncthreads();  // every group's last reads of its buffer
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const int u = j + s * TT;
+      tile[u * G + (g ^ col_swizzle<G>(u))] = x[s];
+    }
+    __syncthreads();
+    store_columns<G, NTH>(tile, stack + ((size_t)n * c.nz_layers + k) * c.nu * c.wp + vbase, c.nu, c.wp - vbase,
+                          c.wp);
+    return;
+  } else {
   // rows v0 (real part) and v0 + 1 (imaginary part) at u = j + s*TT.  The tap pair of column
   // cc = j + s*TT is (Y[cc - 1], Y[cc]): the left value comes from lane l - 1 by a warp
   // shuffle; lane 0 takes the last lane of the group's previous warp (same s), and thread 0
@@ -646,6 +741,7 @@ __global__ void __launch_bounds__(rows16_threads<P>(), 2) k_rows_inv16(const flo
     for (int i = threadIdx.x; i < sp; i += NTH) Lk[i] = make_pair<PairT>(0.f, 0.f);
   if (vbase + ROWS >= c.nv)  // bottom border row
     for (int i = threadIdx.x; i < sp; i += NTH) Lk[(size_t)(c.nv + 1) * sp + i] = make_pair<PairT>(0.f, 0.f);
+  }
 }
 
 // ------------------------------------------------------------------ radix-2 fallback (P <= 8)
@@ -822,16 +918,16 @@ int pick_layer_groups(int ctas_per_group, int nz_layers, int slots, double setup
   return best;
 }
 
-template <int P, int FILT, bool DENS>
+template <int P, int FILT, bool DENS, bool BLEND>
 cudaError_t launch_cols16(const StageAConst& c, const Workspace& ws, const float2* twq, int d0, int cnt, int sms,
                           cudaStream_t stream) {
-  constexpr size_t smem = cols16_smem<P, FILT, DENS>();
+  constexpr size_t smem = cols16_smem<P>();
   static unsigned long long attr_set = 0;  // devices on which the shared-memory limit is raised
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 64 || !(attr_set >> dev & 1ull)) {
     const cudaError_t e =
-        cudaFuncSetAttribute(k_cols16<P, FILT, DENS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_cols16<P, FILT, DENS, BLEND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (dev < 64) attr_set |= 1ull << dev;
   }
@@ -840,12 +936,12 @@ cudaError_t launch_cols16(const StageAConst& c, const Workspace& ws, const float
   // set-up per group: the forward FFT (about one layer's work), and with the density
   // weighting about one more for the weights' trilinear lookups
   const int lg = pick_layer_groups(col_groups * cnt, c.nz_layers, (FILT == 3 ? 1 : 2) * sms, DENS ? 2.2 : 1.2);
-  k_cols16<P, FILT, DENS><<<dim3(col_groups, cnt, lg), kThreads16, smem, stream>>>(
+  k_cols16<P, FILT, DENS, BLEND><<<dim3(col_groups, cnt, lg), kThreads16, smem, stream>>>(
       ws.S, ws.T, twq, ws.uA, ws.ramp, ws.dirs, ws.dens, ws.band_sum, ws.eps, ws.n_bins, ws.bin_width, c, d0);
   return cudaGetLastError();
 }
 
-template <int P, typename PairT>
+template <int P, typename PairT, bool COLS>
 cudaError_t launch_rows_inv16(const StageAConst& c, const float2* T, PairT* stack, const float2* twq, int cnt,
                               cudaStream_t stream) {
   constexpr size_t smem = rows16_smem<P>();
@@ -854,13 +950,36 @@ cudaError_t launch_rows_inv16(const StageAConst& c, const float2* T, PairT* stac
   cudaGetDevice(&dev);
   if (dev >= 64 || !(attr_set >> dev & 1ull)) {
     const cudaError_t e =
-        cudaFuncSetAttribute(k_rows_inv16<P, PairT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_rows_inv16<P, PairT, COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (dev < 64) attr_set |= 1ull << dev;
   }
-  const dim3 gi((c.nv + 2 * kRowPairs16 - 1) / (2 * kRowPairs16), c.nz_layers, cnt);
-  k_rows_inv16<P, PairT><<<gi, rows16_threads<P>(), smem, stream>>>(T, stack, twq, c);
+  const dim3 gi((c.nw + 2 * kRowPairs16 - 1) / (2 * kRowPairs16), c.nz_layers, cnt);
+  k_rows_inv16<P, PairT, COLS><<<gi, rows16_threads<P>(), smem, stream>>>(T, stack, twq, c);
   return cudaGetLastError();
+}
+
+// The row stage of one sub-block into the stacks from direction s0 of the block on.
+template <int P, typename PairT, bool COLS>
+cudaError_t launch_rows(const StageAConst& c, const Workspace& ws, int s0, int cnt, cudaStream_t stream) {
+  const size_t layer = COLS ? (size_t)c.nu * c.wp : c.layer_elems;
+  PairT* stack = (PairT*)ws.stack + (size_t)s0 * c.nz_layers * layer;
+  if constexpr (P >= 1024) {
+    return launch_rows_inv16<P, PairT, COLS>(c, ws.T, stack, ws.twp + (P - 8), cnt, stream);
+  } else {
+    constexpr int G = groups_per_cta<P>();
+    const dim3 gi((c.nw + 2 * G - 1) / (2 * G), c.nz_layers, cnt);
+    k_rows_inv<P, PairT, COLS><<<gi, kThreads, 0, stream>>>(ws.T, stack, ws.twp, c);
+    return cudaGetLastError();
+  }
+}
+template <int P>
+cudaError_t launch_rows(const StageAConst& c, const Workspace& ws, int s0, int cnt, cudaStream_t stream) {
+  if (c.cols)
+    return c.stack_bf16 ? launch_rows<P, __nv_bfloat16, true>(c, ws, s0, cnt, stream)
+                        : launch_rows<P, float, true>(c, ws, s0, cnt, stream);
+  return c.stack_bf16 ? launch_rows<P, __nv_bfloat162, false>(c, ws, s0, cnt, stream)
+                      : launch_rows<P, float2, false>(c, ws, s0, cnt, stream);
 }
 
 template <int P>
@@ -882,25 +1001,21 @@ cudaError_t launch_reg(const StageAConst& c, const Workspace& ws, const float* i
     }
     if (rec) rec->mark(0, stream);
     const bool dens = c.dens.enabled != 0;
-    const size_t stack_off = (size_t)s0 * c.nz_layers * c.layer_elems;
     if constexpr (P >= 1024) {
       // 16-value FFTs (fft16.cuh); their twiddle table follows the 8-value one
       const float2* twq = ws.twp + (P - 8);
       cudaError_t e;
-      if (c.filter == 0) e = dens ? launch_cols16<P, 0, true>(c, ws, twq, d0, cnt, sms, stream)
-                                  : launch_cols16<P, 0, false>(c, ws, twq, d0, cnt, sms, stream);
-      else if (c.filter == 3) e = dens ? launch_cols16<P, 3, true>(c, ws, twq, d0, cnt, sms, stream)
-                                       : launch_cols16<P, 3, false>(c, ws, twq, d0, cnt, sms, stream);
-      else if (c.filter == 2) e = dens ? launch_cols16<P, 2, true>(c, ws, twq, d0, cnt, sms, stream)
-                                       : launch_cols16<P, 2, false>(c, ws, twq, d0, cnt, sms, stream);
-      else e = dens ? launch_cols16<P, 1, true>(c, ws, twq, d0, cnt, sms, stream)
-                    : launch_cols16<P, 1, false>(c, ws, twq, d0, cnt, sms, stream);
+#define RECON_K_COLS16(F)                                                                                       \
+  (dens ? (c.b_frac != 0.f ? launch_cols16<P, F, true, true>(c, ws, twq, d0, cnt, sms, stream)                   \
+                           : launch_cols16<P, F, true, false>(c, ws, twq, d0, cnt, sms, stream))                 \
+        : (c.b_frac != 0.f ? launch_cols16<P, F, false, true>(c, ws, twq, d0, cnt, sms, stream)                  \
+                           : launch_cols16<P, F, false, false>(c, ws, twq, d0, cnt, sms, stream)))
+      e = c.filter == 0 ? RECON_K_COLS16(0)
+                        : (c.filter == 3 ? RECON_K_COLS16(3) : (c.filter == 2 ? RECON_K_COLS16(2) : RECON_K_COLS16(1)));
+#undef RECON_K_COLS16
       if (e != cudaSuccess) return e;
       if (rec) rec->mark(1, stream);
-      if (c.stack_bf16)
-        e = launch_rows_inv16<P, __nv_bfloat162>(c, ws.T, (__nv_bfloat162*)ws.stack + stack_off, twq, cnt, stream);
-      else
-        e = launch_rows_inv16<P, float2>(c, ws.T, (float2*)ws.stack + stack_off, twq, cnt, stream);
+      e = launch_rows<P>(c, ws, s0, cnt, stream);
       if (e != cudaSuccess) return e;
       if (rec) rec->mark(2, stream);
       continue;
@@ -910,26 +1025,29 @@ cudaError_t launch_reg(const StageAConst& c, const Workspace& ws, const float* i
     int lgroups = (target + col_groups * cnt - 1) / (col_groups * cnt);
     lgroups = max(1, min(lgroups, c.nz_layers / 2 > 0 ? c.nz_layers / 2 : 1));
     const dim3 gc(col_groups, cnt, lgroups);
-#define RECON_K_COLS(F, D)                                                                                      \
-  k_cols<P, F, D><<<gc, kThreads, 0, stream>>>(ws.S, ws.T, ws.twp, ws.uA, ws.ramp, ws.dirs, ws.dens, ws.band_sum, \
-                                               ws.eps, ws.n_bins, ws.bin_width, c, d0)
+#define RECON_K_COLS3(F, D, B)                                                                                     \
+  k_cols<P, F, D, B><<<gc, kThreads, 0, stream>>>(ws.S, ws.T, ws.twp, ws.uA, ws.ramp, ws.dirs, ws.dens, ws.band_sum, \
+                                                  ws.eps, ws.n_bins, ws.bin_width, c, d0)
+#define RECON_K_COLS(F)                                                                             \
+  if (c.b_frac != 0.f) {                                                                            \
+    if (dens) RECON_K_COLS3(F, true, true); else RECON_K_COLS3(F, false, true);                     \
+  } else {                                                                                          \
+    if (dens) RECON_K_COLS3(F, true, false); else RECON_K_COLS3(F, false, false);                   \
+  }
     if (c.filter == 0) {
-      if (dens) RECON_K_COLS(0, true); else RECON_K_COLS(0, false);
+      RECON_K_COLS(0)
     } else if (c.filter == 2) {
-      if (dens) RECON_K_COLS(2, true); else RECON_K_COLS(2, false);
+      RECON_K_COLS(2)
     } else if (c.filter == 3) {
-      if (dens) RECON_K_COLS(3, true); else RECON_K_COLS(3, false);
+      RECON_K_COLS(3)
     } else {
-      if (dens) RECON_K_COLS(1, true); else RECON_K_COLS(1, false);
+      RECON_K_COLS(1)
     }
+#undef RECON_K_COLS3
 #undef RECON_K_COLS
     if (rec) rec->mark(1, stream);
-    const dim3 gi((c.nv + 2 * G - 1) / (2 * G), c.nz_layers, cnt);
-    if (c.stack_bf16)
-      k_rows_inv<P, __nv_bfloat162><<<gi, kThreads, 0, stream>>>(ws.T, (__nv_bfloat162*)ws.stack + stack_off, ws.twp,
-                                                                 c);
-    else
-      k_rows_inv<P, float2><<<gi, kThreads, 0, stream>>>(ws.T, (float2*)ws.stack + stack_off, ws.twp, c);
+    const cudaError_t er = launch_rows<P>(c, ws, s0, cnt, stream);
+    if (er != cudaSuccess) return er;
     if (rec) rec->mark(2, stream);
   }
   return cudaGetLastError();

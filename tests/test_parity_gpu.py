@@ -330,3 +330,36 @@ def test_arbitrary_geometry_whole_run_matches_oracle():
     got = r.run(torch.from_numpy(img).cuda()).cpu().numpy()
     r.close()
     assert rel_l2(got, ref) <= TOL_F32, rel_l2(got, ref)
+
+
+@pytest.mark.parametrize("stack", ["f32", "bf16"])
+@pytest.mark.parametrize("grid,nu,nv,nzl,D,filt", [
+    ((37, 33, 21), 41, 33, 5, 7, "tikhonov"),    # sides that leave part of a tile and of a line's block
+    ((37, 20, 9), 41, 23, 5, 7, "tikhonov"),     # rows between two detector rows (blended on the column stage)
+    ((20, 51, 10), 30, 24, 3, 5, "pair"),        # volume rows beside the detector, blended
+    ((70, 65, 33), 24, 70, 4, 3, "tikhonov"),    # voxels beside the detector's columns; more rows than the volume
+    ((24, 32, 40), 40, 32, 40, 6, "tikhonov"),   # lines that cross several layers
+    ((18, 96, 18), 20, 96, 1, 150, "off"),       # one layer; more directions than a warp forms at a time; 32-row tiles
+    ((40, 24, 40), 300, 40, 2, 2, "tikhonov"),   # transforms of 1024 points
+    ((1, 1, 1), 9, 9, 2, 1, "tikhonov"),
+], ids=["ragged", "half", "beside-half", "narrow", "thin", "long", "p1024", "one"])
+def test_column_stack_runs_match_oracle_and_the_tap_pair_kernel(grid, nu, nv, nzl, D, filt, stack):
+    """Whole single-axis runs as AUTO takes them (column stacks) against the oracle and against the
+    tap-pair kernel that bp_kernel="direct" keeps; twice the same bits (the split of the directions over
+    a cluster adds in a fixed order)."""
+    rng = np.random.default_rng(nu + D)
+    img = (1.0 + 0.05 * rng.standard_normal((D, nv, nu))).astype(np.float32)
+    rot = ph.single_axis_rotations(D, span=2 * math.pi, start=0.3)
+    kw = dict(lam=1e-10, delta=1e-9, defocus=rng.uniform(50e-9, 80e-9, D), nz_layers=nzl, sigma=0.05, eps=0.02)
+    ref = O.recon(img, rot, grid=grid, filt={"tikhonov": O.FILTER_TIKHONOV, "pair": O.FILTER_PAIR, "off": O.FILTER_OFF}[filt],
+                  **kw)
+    out = {}
+    for kernel in ("auto", "direct"):
+        r = make(rot, nu, nv, grid, filter=filt, stack_dtype=stack, bp_kernel=kernel, **kw)
+        vol = r.run(torch.from_numpy(img).cuda())
+        out[kernel] = vol.cpu().numpy()
+        if kernel == "auto":
+            assert torch.equal(r.run(torch.from_numpy(img).cuda()), vol)
+        r.close()
+    assert rel_l2(out["auto"], ref) <= (TOL_F32 if stack == "f32" else TOL_BF16)
+    assert rel_l2(out["auto"], out["direct"]) <= TOL_F32
