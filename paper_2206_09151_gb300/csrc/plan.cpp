@@ -94,7 +94,7 @@ struct recon_plan_s {
   recon::StageAConst ca;       // of whole runs (column stacks where the scan takes them)
   recon::StageAConst ca_pair;  // of recon_filter_stage, whose layout is the tap pairs
   recon::BackprojConst cb;
-  int t_rows = 0;              // rows of T: nv, or the column stack's where those are more
+  int t_rows = 0;              // rows of T: nv, or the column stack's where those are more, rounded up to even
   recon::TmaBox tma{};   // footprint box of the TMA-staged backprojection
   bool use_tma = false;  // stage B runs k_backproject_tma
   // workspace layout (byte offsets)
@@ -508,6 +508,7 @@ static int plan_create(const recon_geometry* geom, double lambda, double delta, 
   // views / 32 layers 7.9 ms (the same: most lines span layers there).  An explicit DIRECT or STAGED keeps the pairs.
   ca.cols = 0;
   ca.nw = p->nv;
+  ca.tp = (p->nv + 1) & ~1;
   ca.r_lo = ca.wp = 0;
   ca.b_frac = 0.f;
   p->ca_pair = ca;
@@ -515,11 +516,12 @@ static int plan_create(const recon_geometry* geom, double lambda, double delta, 
   if (cb.cols_j) {
     ca.cols = 1;
     ca.nw = cb.nw;
+    ca.tp = (cb.nw + 1) & ~1;
     ca.r_lo = cb.j_lo + cb.b_int;
     ca.wp = cb.wp;
     ca.b_frac = cb.b_frac;
   }
-  p->t_rows = std::max(p->nv, ca.nw);
+  p->t_rows = std::max(p->ca_pair.tp, ca.tp);
   // The TMA-staged kernel where the general kernel would run (any geometry but a single
   // axis along y, or the layer blend), measured faster on sm_103a; on request for any geometry.
   const bool general = !cb.axis_y || cb.layer_linear;

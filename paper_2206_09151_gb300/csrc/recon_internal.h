@@ -74,6 +74,7 @@ struct StageAConst {
   // the stack hold rows w = 0 .. nw - 1, detector row r_lo + w (b_frac = 0; with tap pairs r_lo = 0,
   // nw = nv) or that row and the next blended with weight b_frac on the next.
   int cols, nw, r_lo, wp;
+  int tp;  // entries between the columns of T: nw rounded up to even, so that a row pair is 16-byte aligned
   float b_frac;
   int sub_block;        // directions per stage-A sub-block (S and T sized for it), 0 = whole block
   int pair_mode;        // filter 3 only: 0 the opposite-pair bracket; 1 / 2 the depth factor
@@ -126,6 +127,9 @@ cudaError_t launch_stage_a(const StageAConst& c, const Workspace& ws, const floa
                            const StageAHook* hook = nullptr);
 // Adds to *count the number of NaN / Inf values among x[0..n).
 cudaError_t launch_count_nonfinite(const float* x, size_t n, unsigned int* count, cudaStream_t stream);
+// The row stage of stage A for 16 <= P <= 2048 (rows_inv.cu): `cnt` directions of T into the stack.
+cudaError_t launch_rows_inv(const StageAConst& c, const float2* T, void* stack, const float2* twp, int cnt,
+                            cudaStream_t stream);
 // The row FFTs alone (S of `count` images starting at image `first`), P >= 16.
 cudaError_t launch_rows_fwd(const StageAConst& c, float2* S, const float2* twp, const float* images, int first,
                             int count, cudaStream_t stream);

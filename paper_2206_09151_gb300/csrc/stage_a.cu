@@ -8,8 +8,8 @@
 //               >= nv are the zero padding), kept in registers; then for every layer
 //               k: multiply by H_k(q) W(q_u), inverse FFT along v, store v < nv
 //                                                                   -> T[n][k][col][v]
-//   k_rows_inv  two rows of one layer per group: Hermitian-extend both half spectra,
-//               pack as real + i real, inverse FFT, crop u < nu    -> stack of tap pairs
+//   k_rows_inv  (rows_inv.cu) two rows of one layer: Hermitian-extend both half spectra, pack
+//               as real + i real, inverse FFT, crop u < nu         -> the stack
 // For P >= 16 the FFTs are register-resident mixed-radix Stockham transforms
 // (fft_reg.cuh); tiny images (P <= 8) use a shared-memory radix-2 transform.
 // The image sits at offset 0 of the P x P frame; by the shift invariance of the
@@ -131,42 +131,6 @@ __device__ __forceinline__ void store_blended(const float2* buf, float2* out, co
   }
 }
 
-// Column-stack rows (backproject_cols.cuh) from the G row pairs of a CTA: `pairs` holds (row 2g, row
-// 2g + 1) of pair g at column u, at entry u G + (g ^ swizzle(u)), so that the stores of 16
-// consecutive columns and the 16-byte loads of two neighbouring pairs are free of bank conflicts;
-// `out` is the layer's entry of column 0 and the CTA's first row.  Rows up to the padded length wp
-// are written (zeros past the last row), 32 contiguous bytes per column for float32 and G = 4.
-template <int G>
-__device__ __forceinline__ int col_swizzle(int u) {
-  constexpr int sh = G >= 16 ? 0 : (G == 8 ? 1 : (G == 4 ? 2 : 3));
-  return (u >> sh) & ((G < 16 ? G : 16) - 1);
-}
-template <int G, int NTH>
-__device__ __forceinline__ void store_columns(const float2* pairs, float* out, int nu, int rows_left, int wp) {
-  constexpr int U = G / 2;  // 16-byte units per column
-  for (int q = threadIdx.x; q < nu * U; q += NTH) {
-    const int h = q % U, u = q / U, sw = col_swizzle<G>(u);
-    if (4 * h >= rows_left) continue;
-    const float4 v = *reinterpret_cast<const float4*>(pairs + u * G + ((2 * h) ^ (sw & ~1)));
-    *reinterpret_cast<float4*>(out + (size_t)u * wp + 4 * h) = sw & 1 ? make_float4(v.z, v.w, v.x, v.y) : v;
-  }
-}
-template <int G, int NTH>
-__device__ __forceinline__ void store_columns(const float2* pairs, __nv_bfloat16* out, int nu, int rows_left, int wp) {
-  constexpr int U = G / 4;
-  for (int q = threadIdx.x; q < nu * U; q += NTH) {
-    const int h = q % U, u = q / U, sw = col_swizzle<G>(u);
-    if (8 * h >= rows_left) continue;
-    __nv_bfloat162 b[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 v = pairs[u * G + ((4 * h + e) ^ sw)];
-      b[e] = __floats2bfloat162_rn(v.x, v.y);
-    }
-    *reinterpret_cast<uint4*>(out + (size_t)u * wp + 8 * h) = *reinterpret_cast<const uint4*>(b);
-  }
-}
-
 // FILT: 0 ramp only (filter off), 1 Tikhonov eps, 2 learned eps table, 3 the opposite-pair
 // form of Eq. 10 / 11 (real part of the complex bracket at the image plane carried to the
 // layer depth); DENS: density
@@ -277,7 +241,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_cols(const float2* __restrict__
     }
   }
   // this thread's rows w = j + s TT - r_lo of T (s < 4: nv <= P/2), stored where 0 <= w < nw
-  float2* Tj = T + ((size_t)n * c.nz_layers * c.half + col) * c.nw + (BLEND ? 0 : j - c.r_lo);
+  float2* Tj = T + ((size_t)n * c.nz_layers * c.half + col) * c.tp + (BLEND ? 0 : j - c.r_lo);
   bool keep[4];
 #pragma unroll
   for (int s = 0; s < 4; ++s) keep[s] = ok && (unsigned)(j + s * TT - c.r_lo) < (unsigned)c.nw;
@@ -308,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_cols(const float2* __restrict__
       x[s] = make_float2(xg[s].x * f, xg[s].y * f);
     }
     fft::block_fft<P, true>(x, buf, tw, j, gsync);
-    float2* out = Tj + (size_t)k * c.half * c.nw;
+    float2* out = Tj + (size_t)k * c.half * c.tp;
     if constexpr (!BLEND) {
       // elements s >= 4 (v >= P/2) are never kept (their last butterflies drop)
 #pragma unroll
@@ -323,114 +287,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_cols(const float2* __restrict__
     }
   }
 }
-
-// PairT: the stack's entry, a tap pair (float2, bfloat162) or with COLS a single value.
-template <int P, typename PairT, bool COLS>
-__global__ void __launch_bounds__(kThreads) k_rows_inv(const float2* __restrict__ T, PairT* __restrict__ stack,
-                                                        const float2* __restrict__ twg, StageAConst c) {
-  constexpr int TT = P / 8, G = groups_per_cta<P>(), L = fft::buffer_len(P, G), H = P / 2 + 1;
-  // tile row stride HS = 8/G (mod 16) float2: a half-warp of the coalesced fill below
-  // (2G rows x 8/G consecutive columns) then writes 16 distinct bank pairs; with G >= 8 a
-  // half-warp fills one column and the odd stride H already does
-  constexpr int HS = G >= 8 ? H : H + ((8 / G - H % 16) % 16 + 16) % 16;
-  constexpr int TILE = 2 * G * HS, BUF = G * L, NT = fft::pass_table_len(P);
-  constexpr int USED = 2 * G * H;  // tile entries that hold spectrum values
-  constexpr int FILL = (USED + kThreads - 1) / kThreads;
-  __shared__ float2 tw[NT];
-  // the half-spectrum tile is read once, before the FFT's first exchange: the
-  // exchange buffer reuses its memory
-  __shared__ __align__(16) float2 shared_mem[TILE > BUF ? TILE : BUF];
-  float2* tile = shared_mem;
-  const int g = threadIdx.x / TT, j = threadIdx.x % TT;
-  float2* buf = shared_mem + g * L;
-  for (int i = threadIdx.x; i < NT; i += kThreads) tw[i] = twg[i];
-  const int n = blockIdx.z, k = blockIdx.y;
-  const int vbase = blockIdx.x * 2 * G;
-  const float2* Tk = T + ((size_t)n * c.nz_layers + k) * H * c.nw;
-  {  // all loads in flight before the shared stores
-    float2 tmp[FILL];
-#pragma unroll
-    for (int it = 0; it < FILL; ++it) {
-      const int idx = threadIdx.x + it * kThreads;
-      const int vv = idx % (2 * G), cc = idx / (2 * G);
-      const int v = vbase + vv;
-      tmp[it] = (idx < USED && v < c.nw) ? Tk[(size_t)cc * c.nw + v] : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int it = 0; it < FILL; ++it) {
-      const int idx = threadIdx.x + it * kThreads;
-      if (idx < USED) tile[(idx % (2 * G)) * HS + idx / (2 * G)] = tmp[it];
-    }
-  }
-  __syncthreads();
-  const int v0 = vbase + 2 * g;
-  const float2* X1 = tile + (2 * g) * HS;
-  const float2* X2 = X1 + HS;
-  float2 x[8];
-#pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const int m = j + s * TT;
-    float2 a, b;
-    if (m <= P / 2) {
-      a = X1[m];
-      b = X2[m];
-      if (m == 0 || m == P / 2) {  // C2R: DC and Nyquist bins are real
-        a.y = 0.f;
-        b.y = 0.f;
-      }
-    } else {  // Hermitian extension X[m] = conj X[P - m]
-      a = X1[P - m];
-      b = X2[P - m];
-      a.y = -a.y;
-      b.y = -b.y;
-    }
-    x[s] = make_float2(a.x - b.y, a.y + b.x);  // a + i b
-  }
-  fft::block_fft<P, true>(x, buf, tw, j);
-  // rows v0 (real part) and v0 + 1 (imaginary part) at u = j + s*TT; pair them with
-  // their right-hand neighbours through the (now free) exchange buffer
-  // nu <= P/2 (P is at least twice the image size): the pairs of columns cc <= nu read
-  // u < P/2 only, i.e. x[s] for s < 4, so the last pass's butterflies feeding s >= 4 drop;
-  // column P/2 (s = 4, thread 0, when nu = P/2) is (Y[nu - 1], 0)
-  __syncthreads();
-  if constexpr (COLS) {
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      const int u = j + s * TT;
-      shared_mem[u * G + (g ^ col_swizzle<G>(u))] = x[s];
-    }
-    __syncthreads();
-    store_columns<G, kThreads>(shared_mem, stack + ((size_t)n * c.nz_layers + k) * c.nu * c.wp + vbase, c.nu,
-                               c.wp - vbase, c.wp);
-    return;
-  } else {
-#pragma unroll
-  for (int s = 0; s < 4; ++s) buf[padded(j + s * TT)] = x[s];
-  __syncthreads();
-  PairT* Lk = stack + ((size_t)n * c.nz_layers + k) * c.layer_elems;
-  const int sp = c.su;
-  if (v0 < c.nv) {
-    const bool two = v0 + 1 < c.nv;
-    PairT* r1 = Lk + (size_t)(v0 + 1) * sp;
-    PairT* r2 = r1 + sp;
-#pragma unroll
-    for (int s = 0; s < 5; ++s) {
-      const int cc = j + s * TT;  // pair column: (Y[cc - 1], Y[cc])
-      if (cc <= c.nu) {
-        const float2 left = cc >= 1 ? buf[padded(cc - 1)] : make_float2(0.f, 0.f);
-        const float2 right = cc < c.nu ? buf[padded(cc)] : make_float2(0.f, 0.f);
-        r1[cc] = make_pair<PairT>(left.x, right.x);
-        if (two) r2[cc] = make_pair<PairT>(left.y, right.y);
-      }
-    }
-  }
-  if (blockIdx.x == 0)  // top border row
-    for (int i = threadIdx.x; i < sp; i += kThreads) Lk[i] = make_pair<PairT>(0.f, 0.f);
-  if (vbase + 2 * G >= c.nv)  // bottom border row
-    for (int i = threadIdx.x; i < sp; i += kThreads) Lk[(size_t)(c.nv + 1) * sp + i] = make_pair<PairT>(0.f, 0.f);
-  }
-}
-
 
 // ------------------------------------------------------------------ 16-value kernels (P >= 1024)
 // The same column and row stages with the 16-value FFT of fft16.cuh: three passes and two
@@ -541,7 +397,7 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
   }
   // this thread's rows w = j + s TT - r_lo of T (s < 8: nv <= P/2, P being at least twice the image
   // size), stored where 0 <= w < nw
-  float2* Tj = T + ((size_t)n * c.nz_layers * c.half + col) * c.nw + (BLEND ? 0 : j - c.r_lo);
+  float2* Tj = T + ((size_t)n * c.nz_layers * c.half + col) * c.tp + (BLEND ? 0 : j - c.r_lo);
   bool keep[8];
 #pragma unroll
   for (int s = 0; s < 8; ++s) keep[s] = ok && (unsigned)(j + s * TT - c.r_lo) < (unsigned)c.nw;
@@ -574,7 +430,7 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
       }
     }
     fft16::group_fft_db<P, true>(x, buf0, buf1, tw, j, gsync);
-    float2* out = Tj + (size_t)k * c.half * c.nw;
+    float2* out = Tj + (size_t)k * c.half * c.tp;
     if constexpr (!BLEND) {
       // elements s >= 8 (v >= P/2) are never kept, so the last pass's butterflies that only feed them are
       // dropped
@@ -595,153 +451,6 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
 template <int P>
 constexpr size_t cols16_smem() {
   return sizeof(float2) * ((size_t)fft16::table_len(P) + 2 * (size_t)cols16_per_cta<P>() * fft16::buffer_len(P));
-}
-
-// Row stage: four row pairs (eight detector rows) of one layer per CTA, a group of P/16
-// threads per pair.  The CTA reads eight consecutive v of every column of T (64 bytes per
-// column), Hermitian-extends both half spectra of a pair, packs them as real + i real,
-// inverse FFT, crop u < nu, stores tap pairs.
-constexpr int kRowPairs16 = 4;
-
-template <int P>
-__host__ __device__ constexpr int rows16_threads() {
-  return kRowPairs16 * (P / 16);
-}
-
-template <int P>
-__host__ __device__ constexpr int rows16_tile_stride() {
-  // stride = 2 (mod 16) float2: a half-warp of the fill (8 rows x 2 columns) writes 16
-  // distinct bank pairs
-  return (P / 2 + 1) + ((2 - (P / 2 + 1) % 16) % 16 + 16) % 16;
-}
-
-template <int P>
-constexpr size_t rows16_smem() {
-  constexpr size_t tile = (size_t)2 * kRowPairs16 * rows16_tile_stride<P>();
-  constexpr size_t bufs = (size_t)kRowPairs16 * fft16::buffer_len(P);
-  return sizeof(float2) * ((size_t)fft16::table_len(P) + (tile > bufs ? tile : bufs));
-}
-
-template <int P, typename PairT, bool COLS>
-__global__ void __launch_bounds__(rows16_threads<P>(), 2) k_rows_inv16(const float2* __restrict__ T,
-                                                                        PairT* __restrict__ stack,
-                                                                        const float2* __restrict__ twg,
-                                                                        StageAConst c) {
-  constexpr int TT = P / 16, NTH = rows16_threads<P>(), H = P / 2 + 1, HS = rows16_tile_stride<P>();
-  constexpr int ROWS = 2 * kRowPairs16, L = fft16::buffer_len(P), NT = fft16::table_len(P);
-  constexpr int USED = ROWS * H;
-  constexpr int FILL = (USED + NTH - 1) / NTH;
-  extern __shared__ __align__(16) float2 smem16[];
-  float2* tw = smem16;
-  // the half-spectrum tile is read once, before the first exchange: the exchange buffers
-  // reuse its memory
-  float2* tile = smem16 + NT;
-  const int g = threadIdx.x / TT, j = threadIdx.x % TT;
-  float2* buf = smem16 + NT + g * L;
-  for (int i = threadIdx.x; i < NT; i += NTH) tw[i] = twg[i];
-  const int n = blockIdx.z, k = blockIdx.y;
-  const int vbase = blockIdx.x * ROWS;
-  const float2* Tk = T + ((size_t)n * c.nz_layers + k) * H * c.nw;
-  {  // all loads in flight before the shared stores
-    float2 tmp[FILL];
-#pragma unroll
-    for (int it = 0; it < FILL; ++it) {
-      const int idx = threadIdx.x + it * NTH;
-      const int vv = idx % ROWS, cc = idx / ROWS;
-      const int v = vbase + vv;
-      tmp[it] = (idx < USED && v < c.nw) ? Tk[(size_t)cc * c.nw + v] : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int it = 0; it < FILL; ++it) {
-      const int idx = threadIdx.x + it * NTH;
-      if (idx < USED) tile[(idx % ROWS) * HS + idx / ROWS] = tmp[it];
-    }
-  }
-  __syncthreads();
-  const int v0 = vbase + 2 * g;
-  const float2* X1 = tile + (2 * g) * HS;
-  const float2* X2 = X1 + HS;
-  float2 x[16];
-#pragma unroll
-  for (int s = 0; s < 16; ++s) {
-    const int m = j + s * TT;
-    float2 a, b;
-    if (m <= P / 2) {
-      a = X1[m];
-      b = X2[m];
-      if (m == 0 || m == P / 2) {  // C2R: DC and Nyquist bins are real
-        a.y = 0.f;
-        b.y = 0.f;
-      }
-    } else {  // Hermitian extension X[m] = conj X[P - m]
-      a = X1[P - m];
-      b = X2[P - m];
-      a.y = -a.y;
-      b.y = -b.y;
-    }
-    x[s] = make_float2(a.x - b.y, a.y + b.x);  // a + i b
-  }
-  __syncthreads();  // every group has read its rows: the tile is free for the exchange buffers
-  const fft::GroupSync gsync{1 + g, TT};
-  fft16::group_fft_sb<P, true, fft::GroupSync, true>(x, buf, tw, j, gsync);
-  if constexpr (COLS) {
-    constexpr int G = kRowPairs16;
-    __syncthreads();  // every group's last reads of its buffer
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      const int u = j + s * TT;
-      tile[u * G + (g ^ col_swizzle<G>(u))] = x[s];
-    }
-    __syncthreads();
-    store_columns<G, NTH>(tile, stack + ((size_t)n * c.nz_layers + k) * c.nu * c.wp + vbase, c.nu, c.wp - vbase,
-                          c.wp);
-    return;
-  } else {
-  // rows v0 (real part) and v0 + 1 (imaginary part) at u = j + s*TT.  The tap pair of column
-  // cc = j + s*TT is (Y[cc - 1], Y[cc]): the left value comes from lane l - 1 by a warp
-  // shuffle; lane 0 takes the last lane of the group's previous warp (same s), and thread 0
-  // the group's last thread at s - 1, both published through the exchange buffer.
-  gsync();  // the last pass's reads of the buffer are done
-  const int lane = threadIdx.x & 31, wg = j >> 5;
-  float2* edge = buf;  // [TT / 32][16]
-  // nu <= P/2 (P is at least twice the image size): the pair columns cc <= nu need
-  // x[s] for s < 8 only (and column P/2, when nu = P/2, the left value x[7] of the last
-  // thread and a zero right value), so the last pass's butterflies feeding s >= 8 drop
-  if (lane == 31) {
-#pragma unroll
-    for (int s = 0; s < 8; ++s) edge[wg * 16 + s] = x[s];
-  }
-  gsync();
-  PairT* Lk = stack + ((size_t)n * c.nz_layers + k) * c.layer_elems;
-  const int sp = c.su;
-  const bool row1 = v0 < c.nv, two = v0 + 1 < c.nv;
-  PairT* r1 = Lk + (size_t)(v0 + 1) * sp;
-  PairT* r2 = r1 + sp;
-#pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    if (s * TT > c.nu) break;  // the same for every thread of the group
-    const int cc = j + s * TT;  // pair column: (Y[cc - 1], Y[cc])
-    float2 left = make_float2(__shfl_up_sync(0xffffffffu, x[s].x, 1), __shfl_up_sync(0xffffffffu, x[s].y, 1));
-    if (lane == 0) {
-      if (wg > 0) left = edge[(wg - 1) * 16 + s];
-      else left = s > 0 ? edge[(TT / 32 - 1) * 16 + s - 1] : make_float2(0.f, 0.f);
-    }
-    const float2 right = cc < c.nu ? x[s] : make_float2(0.f, 0.f);
-    if (row1 && cc <= c.nu) {
-      r1[cc] = make_pair<PairT>(left.x, right.x);
-      if (two) r2[cc] = make_pair<PairT>(left.y, right.y);
-    }
-  }
-  if (j == 0 && row1 && c.nu == P / 2) {  // pair column P/2 = nu: (Y[nu - 1], 0)
-    const float2 left = edge[(TT / 32 - 1) * 16 + 7];
-    r1[P / 2] = make_pair<PairT>(left.x, 0.f);
-    if (two) r2[P / 2] = make_pair<PairT>(left.y, 0.f);
-  }
-  if (blockIdx.x == 0)  // top border row
-    for (int i = threadIdx.x; i < sp; i += NTH) Lk[i] = make_pair<PairT>(0.f, 0.f);
-  if (vbase + ROWS >= c.nv)  // bottom border row
-    for (int i = threadIdx.x; i < sp; i += NTH) Lk[(size_t)(c.nv + 1) * sp + i] = make_pair<PairT>(0.f, 0.f);
-  }
 }
 
 // ------------------------------------------------------------------ radix-2 fallback (P <= 8)
@@ -941,45 +650,11 @@ cudaError_t launch_cols16(const StageAConst& c, const Workspace& ws, const float
   return cudaGetLastError();
 }
 
-template <int P, typename PairT, bool COLS>
-cudaError_t launch_rows_inv16(const StageAConst& c, const float2* T, PairT* stack, const float2* twq, int cnt,
-                              cudaStream_t stream) {
-  constexpr size_t smem = rows16_smem<P>();
-  static unsigned long long attr_set = 0;  // devices on which the shared-memory limit is raised
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev >= 64 || !(attr_set >> dev & 1ull)) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_rows_inv16<P, PairT, COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev < 64) attr_set |= 1ull << dev;
-  }
-  const dim3 gi((c.nw + 2 * kRowPairs16 - 1) / (2 * kRowPairs16), c.nz_layers, cnt);
-  k_rows_inv16<P, PairT, COLS><<<gi, rows16_threads<P>(), smem, stream>>>(T, stack, twq, c);
-  return cudaGetLastError();
-}
-
 // The row stage of one sub-block into the stacks from direction s0 of the block on.
-template <int P, typename PairT, bool COLS>
 cudaError_t launch_rows(const StageAConst& c, const Workspace& ws, int s0, int cnt, cudaStream_t stream) {
-  const size_t layer = COLS ? (size_t)c.nu * c.wp : c.layer_elems;
-  PairT* stack = (PairT*)ws.stack + (size_t)s0 * c.nz_layers * layer;
-  if constexpr (P >= 1024) {
-    return launch_rows_inv16<P, PairT, COLS>(c, ws.T, stack, ws.twp + (P - 8), cnt, stream);
-  } else {
-    constexpr int G = groups_per_cta<P>();
-    const dim3 gi((c.nw + 2 * G - 1) / (2 * G), c.nz_layers, cnt);
-    k_rows_inv<P, PairT, COLS><<<gi, kThreads, 0, stream>>>(ws.T, stack, ws.twp, c);
-    return cudaGetLastError();
-  }
-}
-template <int P>
-cudaError_t launch_rows(const StageAConst& c, const Workspace& ws, int s0, int cnt, cudaStream_t stream) {
-  if (c.cols)
-    return c.stack_bf16 ? launch_rows<P, __nv_bfloat16, true>(c, ws, s0, cnt, stream)
-                        : launch_rows<P, float, true>(c, ws, s0, cnt, stream);
-  return c.stack_bf16 ? launch_rows<P, __nv_bfloat162, false>(c, ws, s0, cnt, stream)
-                      : launch_rows<P, float2, false>(c, ws, s0, cnt, stream);
+  const size_t entry = c.cols ? (c.stack_bf16 ? 2 : 4) : (c.stack_bf16 ? 4 : 8);
+  const size_t layer = c.cols ? (size_t)c.nu * c.wp : (size_t)c.layer_elems;
+  return launch_rows_inv(c, ws.T, (char*)ws.stack + (size_t)s0 * c.nz_layers * layer * entry, ws.twp, cnt, stream);
 }
 
 template <int P>
@@ -1015,7 +690,7 @@ cudaError_t launch_reg(const StageAConst& c, const Workspace& ws, const float* i
 #undef RECON_K_COLS16
       if (e != cudaSuccess) return e;
       if (rec) rec->mark(1, stream);
-      e = launch_rows<P>(c, ws, s0, cnt, stream);
+      e = launch_rows(c, ws, s0, cnt, stream);
       if (e != cudaSuccess) return e;
       if (rec) rec->mark(2, stream);
       continue;
@@ -1046,7 +721,7 @@ cudaError_t launch_reg(const StageAConst& c, const Workspace& ws, const float* i
 #undef RECON_K_COLS3
 #undef RECON_K_COLS
     if (rec) rec->mark(1, stream);
-    const cudaError_t er = launch_rows<P>(c, ws, s0, cnt, stream);
+    const cudaError_t er = launch_rows(c, ws, s0, cnt, stream);
     if (er != cudaSuccess) return er;
     if (rec) rec->mark(2, stream);
   }

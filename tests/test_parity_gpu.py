@@ -89,6 +89,13 @@ def test_stage_a_layer_stack_matches_oracle(case):
     r.close()
 
 
+@pytest.mark.parametrize("nu,nv", [(8, 7), (16, 1), (31, 32), (9, 63), (128, 1), (256, 17), (511, 3), (1024, 9)])
+def test_row_stage_edges_match_oracle(nu, nv):
+    """Every transform length (16 .. 2048) at the edges of a CTA's row pairs: one row, an odd last row, rows
+    beyond a full set of pairs, images as wide as half the transform."""
+    test_stage_a_layer_stack_matches_oracle((nu, nv, 2, "tikhonov", "intensity", 0.0, 0.1, 0.05, 1e-10, 1e-9, 60e-9))
+
+
 # ---------------------------------------------------------------- stage B
 def _stage_b_case(grid, nu, nv, nzl, D, seed, start=0.1, span=math.pi, axis=None, bp_kernel="auto",
                   interp="nearest", rot=None):
