@@ -127,6 +127,9 @@ cudaError_t launch_stage_a(const StageAConst& c, const Workspace& ws, const floa
                            const StageAHook* hook = nullptr);
 // Adds to *count the number of NaN / Inf values among x[0..n).
 cudaError_t launch_count_nonfinite(const float* x, size_t n, unsigned int* count, cudaStream_t stream);
+// The column stage of stage A for 16 <= P <= 512 (columns.cu): `cnt` directions from `dir_begin` on, S to T.
+struct Workspace;
+cudaError_t launch_columns(const StageAConst& c, const Workspace& ws, int dir_begin, int cnt, cudaStream_t stream);
 // The row stage of stage A for 16 <= P <= 2048 (rows_inv.cu): `cnt` directions of T into the stack.
 cudaError_t launch_rows_inv(const StageAConst& c, const float2* T, void* stack, const float2* twp, int cnt,
                             cudaStream_t stream);

@@ -18,6 +18,7 @@
 
 #include <cmath>
 
+#include "columns.cuh"
 #include "density.cuh"
 #include "fft16.cuh"
 #include "fft_reg.cuh"
@@ -48,20 +49,6 @@ __device__ __forceinline__ float contrast_of(float x, int input_mode) {
 __device__ __forceinline__ float sin_from_turns(uint64_t x) {
   const int32_t hi = (int32_t)(x >> 32);
   return sinpif((float)hi * 4.656612873077393e-10f);  // hi * 2^-31 = chi / pi in [-1, 1)
-}
-
-// sin(pi t) for t = hi * 2^-31 in [-1, 1) (hi: the top 32 bits of chi / (2 pi) in
-// fixed point, so chi = pi t is already reduced to [-pi, pi) exactly by the integer
-// phase).  The hardware sine (__sinf, maximum absolute error 2^-21.4 on [-pi, pi])
-// measured faster than an odd polynomial after a quadrant fold, at 5.7e-7 instead of
-// 5.2e-7 rel-L2 against the FP64 oracle on the 256^3 / 360-view scan.
-__device__ __forceinline__ float sin_half_turns(int32_t hi) {
-  return __sinf((float)hi * 1.4629180792671596e-09f);  // hi * 2 pi / 2^32
-}
-
-// sin and cos of chi = pi t for t = hi * 2^-31 in [-1, 1) (hardware sine and cosine).
-__device__ __forceinline__ void sincos_half_turns(int32_t hi, float* sn, float* cs) {
-  __sincosf((float)hi * 1.4629180792671596e-09f, sn, cs);  // hi * 2 pi / 2^32
 }
 
 // The stack stores horizontal tap pairs: entry (row v + 1, column c) of a layer holds
@@ -114,177 +101,6 @@ __global__ void __launch_bounds__(kThreads) k_rows_fwd(const float* __restrict__
     // X1 = (Z[m] + conj Z[P-m]) / 2,  X2 = (Z[m] - conj Z[P-m]) / (2i)
     s1[m] = make_float2(0.5f * (zm.x + zc.x), 0.5f * (zm.y - zc.y));
     if (row2) s1[c.half + m] = make_float2(0.5f * (zm.y + zc.y), -0.5f * (zm.x - zc.x));
-  }
-}
-
-// Column stacks whose volume rows fall between two detector rows: row w is detector rows r_lo + w and
-// the next blended, zero outside the detector (the blend commutes with the row transform, so it
-// is done on the column's values, once per stack entry instead of once per voxel).
-template <class Idx>
-__device__ __forceinline__ void store_blended(const float2* buf, float2* out, const StageAConst& c, int j, int step,
-                                              Idx idx) {
-  for (int w = j; w < c.nw; w += step) {
-    const int r = w + c.r_lo;
-    const float2 a = r >= 0 && r < c.nv ? buf[idx(r)] : make_float2(0.f, 0.f);
-    const float2 b = r + 1 >= 0 && r + 1 < c.nv ? buf[idx(r + 1)] : make_float2(0.f, 0.f);
-    out[w] = make_float2(fmaf(c.b_frac, b.x - a.x, a.x), fmaf(c.b_frac, b.y - a.y, a.y));
-  }
-}
-
-// FILT: 0 ramp only (filter off), 1 Tikhonov eps, 2 learned eps table, 3 the opposite-pair
-// form of Eq. 10 / 11 (real part of the complex bracket at the image plane carried to the
-// layer depth); DENS: density
-// weighting (any geometry) instead of the ramp.  Compile-time, so that each variant keeps
-// only the registers it uses.
-// 3 resident CTAs per SM (80 registers) measured faster than 4 (64 registers) at P = 512.
-// BLEND: rows between two detector rows (c.b_frac != 0).
-template <int P, int FILT, bool DENS, bool BLEND>
-__global__ void __launch_bounds__(kThreads, 3) k_cols(const float2* __restrict__ S, float2* __restrict__ T,
-                                                    const float2* __restrict__ twg, const uint64_t* __restrict__ uA,
-                                                    const float* __restrict__ ramp, const DirParams* __restrict__ dirs,
-                                                    const float* __restrict__ dens,
-                                                    const double* __restrict__ band_sum,
-                                                    const float* __restrict__ eps_tab, int n_bins, int bin_width,
-                                                    StageAConst c, int dir_begin) {
-  constexpr int TT = P / 8, CB = groups_per_cta<P>(), L = fft::buffer_len(P, CB), NT = fft::pass_table_len(P);
-  __shared__ float2 tw[NT];
-  __shared__ float2 buf_all[CB * L];
-  const int g = threadIdx.x / TT, j = threadIdx.x % TT;
-  float2* buf = buf_all + g * L;
-  for (int i = threadIdx.x; i < NT; i += kThreads) tw[i] = twg[i];
-  const int n = blockIdx.y;
-  const int c0 = blockIdx.x * CB;
-  const int col = c0 + g;
-  const float2* Sn = S + (size_t)n * c.nv * c.half;
-  // coalesced fill of rows v < nv of the CTA's CB columns
-  for (int idx = threadIdx.x; idx < c.nv * CB; idx += kThreads) {
-    const int t = idx % CB, v = idx / CB;
-    buf_all[t * L + padded(v)] = (c0 + t < c.half) ? Sn[(size_t)v * c.half + c0 + t] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  float2 xg[8];
-#pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const int v = j + s * TT;
-    xg[s] = v < c.nv ? buf[padded(v)] : make_float2(0.f, 0.f);
-  }
-  // each group owns its exchange buffer from here on: barriers over the group only
-  const fft::GroupSync gsync{1 + g, TT};
-  fft::block_fft<P, false>(xg, buf, tw, j, gsync);  // G(col, m_v) at m_v = j + s*TT, kept for all layers
-
-  const bool ok = col < c.half;
-  const int colc = ok ? col : c.half - 1;
-  // ramp (single-axis scans) or sampling-density weight (any geometry), 1/P^2 included
-  float wgt[DENS ? 8 : 1];
-  if constexpr (DENS) {
-    const DirParams& dp = dirs[dir_begin + n];
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      const int m = j + s * TT;
-      const int mv = m < P / 2 ? m : m - P;
-      float wv = density_weight(c.dens, dens, band_sum, dp.af, dp.bf, (float)colc, (float)mv);
-      // the Nyquist bin is its own alias (+-P/2): mean over both, so that W stays even
-      const bool nyq_u = colc == P / 2, nyq_v = m == P / 2;
-      if (nyq_u || nyq_v) {
-        const float w2 = density_weight(c.dens, dens, band_sum, dp.af, dp.bf, nyq_u ? -(float)colc : (float)colc,
-                                        (nyq_v && !nyq_u) ? -(float)mv : (float)mv);
-        wv = 0.5f * (wv + w2);
-      }
-      wgt[s] = wv;
-    }
-  } else {
-    wgt[0] = ramp[colc];
-  }
-  // with a filter, the weight carries the filter's prefactor lambda / (4 pi sqrt(1+sigma^2))
-  if constexpr (FILT != 0) {
-#pragma unroll
-    for (int s = 0; s < (DENS ? 8 : 1); ++s) wgt[s] *= c.pref;
-  }
-  // chi/(2 pi) in 2^-32 turns needs only the top 32 bits of the 64-bit fixed-point
-  // sum: the per-layer product uA_k * m is formed as hi(uA) * m + umulhi(lo(uA), m), and
-  // the layer-independent part uC * m^2 - uW once per element (dropped low-word carries
-  // cost at most 2^-32 turns).
-  uint32_t msq[8], base_hi[8];
-#pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const int m = j + s * TT;
-    const int mv = m < P / 2 ? m : m - P;
-    msq[s] = (uint32_t)(colc * colc + mv * mv);
-    const uint64_t m64 = msq[s];
-    base_hi[s] = (uint32_t)((c.uC * (m64 * m64) - c.uW) >> 32);
-  }
-  // learned regulariser: the radial bin of each frequency (isqrt, exact integers)
-  int bin[FILT == 2 ? 8 : 1];
-  if constexpr (FILT == 2) {
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      int r = (int)sqrtf((float)msq[s]);
-      while ((uint32_t)r * (uint32_t)r > msq[s]) --r;
-      while ((uint32_t)(r + 1) * (uint32_t)(r + 1) <= msq[s]) ++r;
-      const int b = r / bin_width;
-      bin[s] = b < n_bins - 1 ? b : n_bins - 1;
-    }
-  }
-  // the opposite-pair filter (FILT 3) keeps one row more per direction: the image-plane
-  // phase constant after the Nz per-layer depth constants
-  const uint64_t* uAn = uA + (size_t)(dir_begin + n) * (c.nz_layers + (FILT == 3 ? 1 : 0));
-  float sp[FILT == 3 ? 8 : 1], cp[FILT == 3 ? 8 : 1];
-  if constexpr (FILT == 3) {  // image-plane sin chi / (sin^2 chi + eps), cos chi / (cos^2 chi + eps)
-    const uint64_t uR = uAn[c.nz_layers];
-    const uint32_t r_hi = (uint32_t)(uR >> 32), r_lo = (uint32_t)uR;
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      float sn, cs;
-      sincos_half_turns((int32_t)(r_hi * msq[s] + __umulhi(r_lo, msq[s]) + base_hi[s]), &sn, &cs);
-      sp[s] = c.pair_mode == 0 ? __fdividef(sn, fmaf(sn, sn, c.eps)) : (c.pair_mode == 1 ? 1.f : 0.f);
-      cp[s] = c.pair_mode == 0 ? __fdividef(cs, fmaf(cs, cs, c.eps)) : (c.pair_mode == 1 ? 0.f : -1.f);
-    }
-  }
-  // this thread's rows w = j + s TT - r_lo of T (s < 4: nv <= P/2), stored where 0 <= w < nw
-  float2* Tj = T + ((size_t)n * c.nz_layers * c.half + col) * c.tp + (BLEND ? 0 : j - c.r_lo);
-  bool keep[4];
-#pragma unroll
-  for (int s = 0; s < 4; ++s) keep[s] = ok && (unsigned)(j + s * TT - c.r_lo) < (unsigned)c.nw;
-  // this CTA's layers: group blockIdx.z of gridDim.z equal groups
-  const int lg = (c.nz_layers + gridDim.z - 1) / gridDim.z;
-  const int k_begin = blockIdx.z * lg;
-  const int k_end = min(c.nz_layers, k_begin + lg);
-  for (int k = k_begin; k < k_end; ++k) {
-    const uint64_t uAk = uAn[k];
-    const uint32_t a_hi = (uint32_t)(uAk >> 32), a_lo = (uint32_t)uAk;
-    const float* eps_k = eps_tab + ((size_t)n * c.nz_layers + k) * n_bins;
-    float2 x[8];
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      float f = wgt[DENS ? s : 0];
-      if constexpr (FILT == 3) {  // Re{bracket * exp(-i phi_k)}, phi_k = pi lambda z_k q^2
-        float sn, cs;
-        sincos_half_turns((int32_t)(a_hi * msq[s] + __umulhi(a_lo, msq[s])), &sn, &cs);
-        f *= fmaf(sp[s], cs, -cp[s] * sn);
-      } else if constexpr (FILT != 0) {
-        const uint32_t hi = a_hi * msq[s] + __umulhi(a_lo, msq[s]) + base_hi[s];
-        const float sn = sin_half_turns((int32_t)hi);
-        float e;
-        if constexpr (FILT == 2) e = __ldg(eps_k + bin[s]);  // learned eps
-        else e = c.eps;                                      // Tikhonov eps
-        f *= __fdividef(sn, fmaf(sn, sn, e));                // real part of the Eq. 11 bracket
-      }
-      x[s] = make_float2(xg[s].x * f, xg[s].y * f);
-    }
-    fft::block_fft<P, true>(x, buf, tw, j, gsync);
-    float2* out = Tj + (size_t)k * c.half * c.tp;
-    if constexpr (!BLEND) {
-      // elements s >= 4 (v >= P/2) are never kept (their last butterflies drop)
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-        if (keep[s]) out[s * TT] = x[s];
-    } else {
-      gsync();  // the transform's last reads of the buffer
-#pragma unroll
-      for (int s = 0; s < 4; ++s) buf[padded(j + s * TT)] = x[s];
-      gsync();
-      if (ok) store_blended(buf, out, c, j, TT, [](int v) { return padded(v); });
-    }
   }
 }
 
@@ -362,35 +178,33 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
       for (int s = 0; s < 16; ++s) xg[s] = make_float2(xg[s].x * wv, xg[s].y * wv);
     }
   }
-  // chi/(2 pi) in 2^-32 turns (top 32 bits of the 64-bit fixed-point phase): per layer
-  // hi(uA_k) m + umulhi(lo(uA_k), m), plus the layer-independent uC m^2 - uW
-  uint32_t msq[16], base_hi[16];
-#pragma unroll
-  for (int s = 0; s < 16; ++s) {
-    const int m = j + s * TT;
+  // chi/(2 pi) in 2^-32 turns, as in k_cols
+  const auto msq = [&](int s, int jj) {
+    const int m = jj + s * TT;
     const int mv = m < P / 2 ? m : m - P;
-    const uint32_t q2 = (uint32_t)(colc * colc + mv * mv);
-    const uint64_t m64 = q2;
-    base_hi[s] = (uint32_t)((c.uC * (m64 * m64) - c.uW) >> 32);
-    if constexpr (FILT == 2) {  // radial bin (exact isqrt) packed above the 22-bit m
+    return (uint32_t)(colc * colc + mv * mv);
+  };
+  const auto base_hi = [&](uint64_t m) { return (uint32_t)((c.uC * (m * m) - c.uW) >> 32); };
+  uint32_t bins[FILT == 2 ? 4 : 1];  // radial bins (exact isqrt, at most 256 of them), four to a word
+  if constexpr (FILT == 2) {
+#pragma unroll
+    for (int s = 0; s < 16; ++s) {
+      const uint32_t q2 = msq(s, j);
       int r = (int)sqrtf((float)q2);
       while ((uint32_t)r * (uint32_t)r > q2) --r;
       while ((uint32_t)(r + 1) * (uint32_t)(r + 1) <= q2) ++r;
-      const int b = min(r / bin_width, n_bins - 1);
-      msq[s] = q2 | ((uint32_t)b << 22);
-    } else {
-      msq[s] = q2;
+      const uint32_t b = (uint32_t)min(r / bin_width, n_bins - 1);
+      bins[s / 4] = s % 4 ? bins[s / 4] | b << 8 * (s % 4) : b;
     }
   }
   const uint64_t* uAn = uA + (size_t)(dir_begin + n) * (c.nz_layers + (FILT == 3 ? 1 : 0));
   float sp[FILT == 3 ? 16 : 1], cp[FILT == 3 ? 16 : 1];
   if constexpr (FILT == 3) {  // image-plane sin chi / (sin^2 chi + eps), cos chi / (cos^2 chi + eps)
     const uint64_t uR = uAn[c.nz_layers];
-    const uint32_t r_hi = (uint32_t)(uR >> 32), r_lo = (uint32_t)uR;
 #pragma unroll
     for (int s = 0; s < 16; ++s) {
       float sn, cs;
-      sincos_half_turns((int32_t)(r_hi * msq[s] + __umulhi(r_lo, msq[s]) + base_hi[s]), &sn, &cs);
+      sincos_half_turns((int32_t)(phase_of(uR, msq(s, j)) + base_hi(msq(s, j))), &sn, &cs);
       sp[s] = c.pair_mode == 0 ? __fdividef(sn, fmaf(sn, sn, c.eps)) : (c.pair_mode == 1 ? 1.f : 0.f);
       cp[s] = c.pair_mode == 0 ? __fdividef(cs, fmaf(cs, cs, c.eps)) : (c.pair_mode == 1 ? 0.f : -1.f);
     }
@@ -404,29 +218,41 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
   const int lg = (c.nz_layers + gridDim.z - 1) / gridDim.z;
   const int k_begin = blockIdx.z * lg;
   const int k_end = min(c.nz_layers, k_begin + lg);
-  for (int k = k_begin; k < k_end; ++k) {
-    const uint64_t uAk = uAn[k];
-    const uint32_t a_hi = (uint32_t)(uAk >> 32), a_lo = (uint32_t)uAk;
+  uint32_t hi[FILT != 0 ? 16 : 1], step[FILT != 0 ? 16 : 1];  // phase of the layer, per layer
+  const float eps0 = fmaxf(c.eps, FLT_MIN);                   // Tikhonov eps
+  for (int kr = k_begin, kr_end; kr < k_end; kr = kr_end) {  // runs of kPhaseRun layers
+  kr_end = min(k_end, kr - kr % kPhaseRun + kPhaseRun);
+  if constexpr (FILT != 0) {
+    const int k0 = kr - kr % kPhaseRun;
+    int jj = j;  // formed again for each run, not kept in registers over the layers
+    asm volatile("" : "+r"(jj));
+    const uint64_t uA0 = uAn[k0], dA = k0 + 1 < c.nz_layers ? uAn[k0 + 1] - uA0 : 0;
+#pragma unroll
+    for (int s = 0; s < 16; ++s) {
+      const uint32_t m = msq(s, jj);
+      step[s] = phase_step(dA, m);
+      hi[s] = phase_of(uA0, m) + (FILT == 3 ? 0 : base_hi(m)) + (uint32_t)(kr - k0) * step[s];
+    }
+  }
+  for (int k = kr; k < kr_end; ++k) {
     const float* eps_k = eps_tab + ((size_t)n * c.nz_layers + k) * n_bins;
     float2 x[16];
 #pragma unroll
     for (int s = 0; s < 16; ++s) {
-      if constexpr (FILT == 3) {  // Re{bracket * exp(-i phi_k)}, phi_k = pi lambda z_k q^2
-        float sn, cs;
-        sincos_half_turns((int32_t)(a_hi * msq[s] + __umulhi(a_lo, msq[s])), &sn, &cs);
-        const float f = fmaf(sp[s], cs, -cp[s] * sn);
-        x[s] = make_float2(xg[s].x * f, xg[s].y * f);
-      } else if constexpr (FILT != 0) {
-        const uint32_t q2 = FILT == 2 ? (msq[s] & 0x3FFFFFu) : msq[s];
-        const uint32_t hi = a_hi * q2 + __umulhi(a_lo, q2) + base_hi[s];
-        const float sn = sin_half_turns((int32_t)hi);
-        float e;
-        if constexpr (FILT == 2) e = __ldg(eps_k + (msq[s] >> 22));  // learned eps
-        else e = c.eps;                                             // Tikhonov eps
-        const float f = __fdividef(sn, fmaf(sn, sn, e));           // real part of the Eq. 11 bracket
-        x[s] = make_float2(xg[s].x * f, xg[s].y * f);
-      } else {
+      if constexpr (FILT == 0) {
         x[s] = xg[s];
+      } else {
+        float f;
+        if constexpr (FILT == 3) {  // Re{bracket * exp(-i phi_k)}, phi_k = pi lambda z_k q^2
+          float sn, cs;
+          sincos_half_turns((int32_t)hi[s], &sn, &cs);
+          f = fmaf(sp[s], cs, -cp[s] * sn);
+        } else {  // real part of the Eq. 11 bracket
+          const float e = FILT == 2 ? fmaxf(__ldg(eps_k + (bins[s / 4] >> 8 * (s % 4) & 255u)), FLT_MIN) : eps0;
+          f = inverse_ctf(sin_half_turns((int32_t)hi[s]), e);
+        }
+        hi[s] += step[s];
+        x[s] = make_float2(xg[s].x * f, xg[s].y * f);
       }
     }
     fft16::group_fft_db<P, true>(x, buf0, buf1, tw, j, gsync);
@@ -445,6 +271,7 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
       if (ok) store_blended(buf0, out, c, j, TT, [](int v) { return fft16::pad(v); });
       gsync();  // the next transform's first pass writes buf0
     }
+  }
   }
 }
 
@@ -608,25 +435,6 @@ __global__ void k_count_nonfinite(const float* __restrict__ x, size_t n, unsigne
 }
 
 // ------------------------------------------------------------------ launch
-// Layer groups of the column stage: the split of the Nz layers over CTAs that keeps the
-// last wave of `slots` resident CTAs fullest, counting the set-up each group repeats (the
-// column's forward FFT and weights, `setup` layers' worth of work) as extra work.
-int pick_layer_groups(int ctas_per_group, int nz_layers, int slots, double setup) {
-  int best = 1;
-  double best_eff = 0.0;
-  const int max_lg = nz_layers / 2 > 0 ? (nz_layers / 2 < 16 ? nz_layers / 2 : 16) : 1;
-  for (int lg = 1; lg <= max_lg; ++lg) {
-    const double waves = (double)ctas_per_group * lg / slots;
-    const double fill = waves / std::ceil(waves);
-    const double eff = fill * (double)nz_layers / (nz_layers + setup * lg);
-    if (eff > best_eff + 1e-9) {
-      best_eff = eff;
-      best = lg;
-    }
-  }
-  return best;
-}
-
 template <int P, int FILT, bool DENS, bool BLEND>
 cudaError_t launch_cols16(const StageAConst& c, const Workspace& ws, const float2* twq, int d0, int cnt, int sms,
                           cudaStream_t stream) {
@@ -664,7 +472,6 @@ cudaError_t launch_reg(const StageAConst& c, const Workspace& ws, const float* i
   // Sub-blocks of c.sub_block directions: S and T of one sub-block stay in L2 between the
   // column and the row kernels; each sub-block writes its part of the block's stack.
   const int sub = c.sub_block > 0 ? c.sub_block : dir_count;
-  const int col_groups = (c.half + G - 1) / G;
   const int sms = device_sm_count();
   for (int s0 = 0; s0 < dir_count; s0 += sub) {
     const int cnt = min(sub, dir_count - s0);
@@ -689,40 +496,13 @@ cudaError_t launch_reg(const StageAConst& c, const Workspace& ws, const float* i
                         : (c.filter == 3 ? RECON_K_COLS16(3) : (c.filter == 2 ? RECON_K_COLS16(2) : RECON_K_COLS16(1)));
 #undef RECON_K_COLS16
       if (e != cudaSuccess) return e;
-      if (rec) rec->mark(1, stream);
-      e = launch_rows(c, ws, s0, cnt, stream);
-      if (e != cudaSuccess) return e;
-      if (rec) rec->mark(2, stream);
-      continue;
-    }
-    // layer groups so that about 2 waves of CTAs run even for a small sub-block
-    const int target = 2 * sms * 4;
-    int lgroups = (target + col_groups * cnt - 1) / (col_groups * cnt);
-    lgroups = max(1, min(lgroups, c.nz_layers / 2 > 0 ? c.nz_layers / 2 : 1));
-    const dim3 gc(col_groups, cnt, lgroups);
-#define RECON_K_COLS3(F, D, B)                                                                                     \
-  k_cols<P, F, D, B><<<gc, kThreads, 0, stream>>>(ws.S, ws.T, ws.twp, ws.uA, ws.ramp, ws.dirs, ws.dens, ws.band_sum, \
-                                                  ws.eps, ws.n_bins, ws.bin_width, c, d0)
-#define RECON_K_COLS(F)                                                                             \
-  if (c.b_frac != 0.f) {                                                                            \
-    if (dens) RECON_K_COLS3(F, true, true); else RECON_K_COLS3(F, false, true);                     \
-  } else {                                                                                          \
-    if (dens) RECON_K_COLS3(F, true, false); else RECON_K_COLS3(F, false, false);                   \
-  }
-    if (c.filter == 0) {
-      RECON_K_COLS(0)
-    } else if (c.filter == 2) {
-      RECON_K_COLS(2)
-    } else if (c.filter == 3) {
-      RECON_K_COLS(3)
     } else {
-      RECON_K_COLS(1)
+      const cudaError_t e = launch_columns(c, ws, d0, cnt, stream);
+      if (e != cudaSuccess) return e;
     }
-#undef RECON_K_COLS3
-#undef RECON_K_COLS
     if (rec) rec->mark(1, stream);
-    const cudaError_t er = launch_rows(c, ws, s0, cnt, stream);
-    if (er != cudaSuccess) return er;
+    const cudaError_t e = launch_rows(c, ws, s0, cnt, stream);
+    if (e != cudaSuccess) return e;
     if (rec) rec->mark(2, stream);
   }
   return cudaGetLastError();

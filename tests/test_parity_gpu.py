@@ -96,6 +96,13 @@ def test_row_stage_edges_match_oracle(nu, nv):
     test_stage_a_layer_stack_matches_oracle((nu, nv, 2, "tikhonov", "intensity", 0.0, 0.1, 0.05, 1e-10, 1e-9, 60e-9))
 
 
+@pytest.mark.parametrize("nu,nv,nzl,filt", [(9, 5, 96, "tikhonov"), (20, 32, 67, "pair"), (60, 33, 65, "tikhonov"),
+                                            (100, 7, 70, "pair"), (200, 3, 96, "tikhonov"), (300, 2, 66, "pair")])
+def test_phase_runs_over_many_layers_match_oracle(nu, nv, nzl, filt):
+    """More layers than one run of the phase sum (64, of at most 96), a short last run, every size of column kernel."""
+    test_stage_a_layer_stack_matches_oracle((nu, nv, nzl, filt, "intensity", 1e-6, 0.1, 0.05, 1e-10, 1e-9, 60e-9))
+
+
 # ---------------------------------------------------------------- stage B
 def _stage_b_case(grid, nu, nv, nzl, D, seed, start=0.1, span=math.pi, axis=None, bp_kernel="auto",
                   interp="nearest", rot=None):
