@@ -766,7 +766,8 @@ recon::Workspace carve(recon_plan_t p, void* ws) {
   return w;
 }
 
-int upload_tables(recon_plan_t p, const recon::Workspace& w, cudaStream_t s) {
+// stage_a: whether the call filters images (a backprojection of ready stacks needs no sampling density).
+int upload_tables(recon_plan_t p, const recon::Workspace& w, cudaStream_t s, bool stage_a = true) {
   cudaError_t e = cudaSuccess;
   if (p->D > 0) {
     e = cudaMemcpyAsync(w.dirs, p->dirs.data(), sizeof(recon::DirParams) * p->D, cudaMemcpyHostToDevice, s);
@@ -788,7 +789,7 @@ int upload_tables(recon_plan_t p, const recon::Workspace& w, cudaStream_t s) {
   if (e == cudaSuccess && !p->x2.empty())
     e = cudaMemcpyAsync(base + p->off_x2, p->x2.data(), sizeof(float) * p->x2.size(), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return cuda_fail(e, "upload of plan tables");
-  if (p->ca.dens.enabled) {
+  if (stage_a && p->ca.dens.enabled) {
     e = recon::launch_density_setup(p->ca.dens, w.dirs, p->D, p->P, w.dens, w.band_sum, s);
     if (e != cudaSuccess) return cuda_fail(e, "sampling-density setup");
   }
@@ -1048,7 +1049,7 @@ int recon_backproject(recon_plan_t p, const void* stack, int dir_begin, int dir_
   int rc = check_ws(p, workspace, ws_bytes, "recon_backproject");
   if (rc) return rc;
   const recon::Workspace w = carve(p, workspace);
-  rc = upload_tables(p, w, s);
+  rc = upload_tables(p, w, s, false);
   if (rc) return rc;
   rc = tma_begin(p, workspace, s, "recon_backproject");
   if (rc) return rc;
