@@ -27,6 +27,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "recon_internal.h"
 #include "tma.cuh"
@@ -276,65 +277,72 @@ __global__ void __launch_bounds__(kThreads, RECON_TMA_MIN_CTAS) k_backproject_tm
     float2 A2 = make_float2(A, A + r.af2), B2 = make_float2(B, B + r.bf2);
     const float2 dA2 = make_float2(2.f * r.af2, 2.f * r.af2), dB2 = make_float2(2.f * r.bf2, 2.f * r.bf2);
     uint32_t t = r.t + r.ti * (uint32_t)tx + r.tj * (uint32_t)ty;
+    // one run of the tile's column where every layer lies inside the stack and one that clamps (a branch per item
+    // instead of one per pair of voxels: 1208 us instead of 1263 for 4 directions of a 1024 x 1024 x 256 slab)
+    const auto run = [&](auto clamp_layers) {
+      [[maybe_unused]] constexpr bool clamp = decltype(clamp_layers)::value;
 #pragma unroll
-    for (int q = 0; q < kMZ / 2; ++q) {
-      // voxels 2q and 2q + 1 of the thread's run, packed in the two halves of each float2
-      // the magic-number add rounded down holds floor(A) in its low mantissa bits; the
-      // box-local coordinate A is the pair index plus the weight on its right tap
-      const float2 tA = __fadd2_rd(A2, kM2), tB = __fadd2_rd(B2, kM2);
-      const float2 fA = __ffma2_rn(__fadd2_rn(tA, kMm2), kNeg, A2);  // A - floor(A)
-      const float2 fB = __ffma2_rn(__fadd2_rn(tB, kMm2), kNeg, B2);
-      const uint32_t rc0 = __float_as_uint(tA.x) * es + __float_as_uint(tB.x) * Wb + base;
-      const uint32_t rc1 = __float_as_uint(tA.y) * es + __float_as_uint(tB.y) * Wb + base;
-      const uint32_t t0 = t, t1 = t + r.tk;
-      if constexpr (LIN) {
-        float w[2];
-        uint32_t a0[2], a1[2];
+      for (int q = 0; q < kMZ / 2; ++q) {
+        // voxels 2q and 2q + 1 of the thread's run, packed in the two halves of each float2
+        // the magic-number add rounded down holds floor(A) in its low mantissa bits; the
+        // box-local coordinate A is the pair index plus the weight on its right tap
+        const float2 tA = __fadd2_rd(A2, kM2), tB = __fadd2_rd(B2, kM2);
+        const float2 fA = __ffma2_rn(__fadd2_rn(tA, kMm2), kNeg, A2);  // A - floor(A)
+        const float2 fB = __ffma2_rn(__fadd2_rn(tB, kMm2), kNeg, B2);
+        const uint32_t rc0 = __float_as_uint(tA.x) * es + __float_as_uint(tB.x) * Wb + base;
+        const uint32_t rc1 = __float_as_uint(tA.y) * es + __float_as_uint(tB.y) * Wb + base;
+        const uint32_t t0 = t, t1 = t + r.tk;
+        if constexpr (LIN) {
+          float w[2];
+          uint32_t a0[2], a1[2];
 #pragma unroll
-        for (int v = 0; v < 2; ++v) {
-          const int32_t tp = (int32_t)(v ? t1 : t0) - (1 << 23);
-          const int k0r = tp >> 24;
-          const bool outer = k0r < lo || k0r >= hi;
-          const int kk0 = min(max(k0r, lo), hi);
-          const int kk1 = min(kk0 + 1, hi);
-          w[v] = outer ? 0.f : (float)(tp & 0xFFFFFF) * 0x1p-24f;
-          a0[v] = (v ? rc1 : rc0) + (uint32_t)kk0 * HWb;
-          a1[v] = (v ? rc1 : rc0) + (uint32_t)kk1 * HWb;
+          for (int v = 0; v < 2; ++v) {
+            const int32_t tp = (int32_t)(v ? t1 : t0) - (1 << 23);
+            const int k0r = tp >> 24;
+            const bool outer = k0r < lo || k0r >= hi;
+            const int kk0 = min(max(k0r, lo), hi);
+            const int kk1 = min(kk0 + 1, hi);
+            w[v] = outer ? 0.f : (float)(tp & 0xFFFFFF) * 0x1p-24f;
+            a0[v] = (v ? rc1 : rc0) + (uint32_t)kk0 * HWb;
+            a1[v] = (v ? rc1 : rc0) + (uint32_t)kk1 * HWb;
+          }
+          const float2 p00 = pair_at<ST>(a0[0]), p01 = pair_at<ST>(a0[0] + Wb);
+          const float2 p10 = pair_at<ST>(a0[1]), p11 = pair_at<ST>(a0[1] + Wb);
+          const float2 s00 = pair_at<ST>(a1[0]), s01 = pair_at<ST>(a1[0] + Wb);
+          const float2 s10 = pair_at<ST>(a1[1]), s11 = pair_at<ST>(a1[1] + Wb);
+          const float2 X0 = make_float2(p00.x, p10.x), Y0 = make_float2(p00.y, p10.y);
+          const float2 X1 = make_float2(p01.x, p11.x), Y1 = make_float2(p01.y, p11.y);
+          const float2 U0 = make_float2(s00.x, s10.x), V0 = make_float2(s00.y, s10.y);
+          const float2 U1 = make_float2(s01.x, s11.x), V1 = make_float2(s01.y, s11.y);
+          const float2 top0 = __ffma2_rn(fA, __ffma2_rn(X0, kNeg, Y0), X0);
+          const float2 bot0 = __ffma2_rn(fA, __ffma2_rn(X1, kNeg, Y1), X1);
+          const float2 top1 = __ffma2_rn(fA, __ffma2_rn(U0, kNeg, V0), U0);
+          const float2 bot1 = __ffma2_rn(fA, __ffma2_rn(U1, kNeg, V1), U1);
+          const float2 v0 = __ffma2_rn(fB, __ffma2_rn(top0, kNeg, bot0), top0);
+          const float2 v1 = __ffma2_rn(fB, __ffma2_rn(top1, kNeg, bot1), top1);
+          acc[q] = __fadd2_rn(acc[q], __ffma2_rn(make_float2(w[0], w[1]), __ffma2_rn(v0, kNeg, v1), v0));
+        } else {
+          int l0 = (int32_t)t0 >> 24, l1 = (int32_t)t1 >> 24;
+          if (clamp) {
+            l0 = min(max(l0, lo), hi);
+            l1 = min(max(l1, lo), hi);
+          }
+          const uint32_t a0 = rc0 + (uint32_t)l0 * HWb, a1 = rc1 + (uint32_t)l1 * HWb;
+          const float2 p00 = pair_at<ST>(a0), p01 = pair_at<ST>(a0 + Wb);
+          const float2 p10 = pair_at<ST>(a1), p11 = pair_at<ST>(a1 + Wb);
+          const float2 X0 = make_float2(p00.x, p10.x), Y0 = make_float2(p00.y, p10.y);
+          const float2 X1 = make_float2(p01.x, p11.x), Y1 = make_float2(p01.y, p11.y);
+          const float2 top = __ffma2_rn(fA, __ffma2_rn(X0, kNeg, Y0), X0);
+          const float2 bot = __ffma2_rn(fA, __ffma2_rn(X1, kNeg, Y1), X1);
+          acc[q] = __fadd2_rn(acc[q], __ffma2_rn(fB, __ffma2_rn(top, kNeg, bot), top));
         }
-        const float2 p00 = pair_at<ST>(a0[0]), p01 = pair_at<ST>(a0[0] + Wb);
-        const float2 p10 = pair_at<ST>(a0[1]), p11 = pair_at<ST>(a0[1] + Wb);
-        const float2 s00 = pair_at<ST>(a1[0]), s01 = pair_at<ST>(a1[0] + Wb);
-        const float2 s10 = pair_at<ST>(a1[1]), s11 = pair_at<ST>(a1[1] + Wb);
-        const float2 X0 = make_float2(p00.x, p10.x), Y0 = make_float2(p00.y, p10.y);
-        const float2 X1 = make_float2(p01.x, p11.x), Y1 = make_float2(p01.y, p11.y);
-        const float2 U0 = make_float2(s00.x, s10.x), V0 = make_float2(s00.y, s10.y);
-        const float2 U1 = make_float2(s01.x, s11.x), V1 = make_float2(s01.y, s11.y);
-        const float2 top0 = __ffma2_rn(fA, __ffma2_rn(X0, kNeg, Y0), X0);
-        const float2 bot0 = __ffma2_rn(fA, __ffma2_rn(X1, kNeg, Y1), X1);
-        const float2 top1 = __ffma2_rn(fA, __ffma2_rn(U0, kNeg, V0), U0);
-        const float2 bot1 = __ffma2_rn(fA, __ffma2_rn(U1, kNeg, V1), U1);
-        const float2 v0 = __ffma2_rn(fB, __ffma2_rn(top0, kNeg, bot0), top0);
-        const float2 v1 = __ffma2_rn(fB, __ffma2_rn(top1, kNeg, bot1), top1);
-        acc[q] = __fadd2_rn(acc[q], __ffma2_rn(make_float2(w[0], w[1]), __ffma2_rn(v0, kNeg, v1), v0));
-      } else {
-        int l0 = (int32_t)t0 >> 24, l1 = (int32_t)t1 >> 24;
-        if (!inside) {
-          l0 = min(max(l0, lo), hi);
-          l1 = min(max(l1, lo), hi);
-        }
-        const uint32_t a0 = rc0 + (uint32_t)l0 * HWb, a1 = rc1 + (uint32_t)l1 * HWb;
-        const float2 p00 = pair_at<ST>(a0), p01 = pair_at<ST>(a0 + Wb);
-        const float2 p10 = pair_at<ST>(a1), p11 = pair_at<ST>(a1 + Wb);
-        const float2 X0 = make_float2(p00.x, p10.x), Y0 = make_float2(p00.y, p10.y);
-        const float2 X1 = make_float2(p01.x, p11.x), Y1 = make_float2(p01.y, p11.y);
-        const float2 top = __ffma2_rn(fA, __ffma2_rn(X0, kNeg, Y0), X0);
-        const float2 bot = __ffma2_rn(fA, __ffma2_rn(X1, kNeg, Y1), X1);
-        acc[q] = __fadd2_rn(acc[q], __ffma2_rn(fB, __ffma2_rn(top, kNeg, bot), top));
+        A2 = __fadd2_rn(A2, dA2);
+        B2 = __fadd2_rn(B2, dB2);
+        t += 2u * r.tk;
       }
-      A2 = __fadd2_rn(A2, dA2);
-      B2 = __fadd2_rn(B2, dB2);
-      t += 2u * r.tk;
-    }
+    };
+    if (LIN || inside) run(std::false_type{});  // the blend clamps its two layers by itself
+    else run(std::true_type{});
     __syncwarp();
     if (lane == 0) mbar_arrive(bar_empty + 8u * s);
     if (++s == S) {
