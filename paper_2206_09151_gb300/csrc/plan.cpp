@@ -374,11 +374,13 @@ static int plan_create(const recon_geometry* geom, double lambda, double delta, 
     // Ramp: (pi/D) delta DFT_P[Ram-Lak](m), m = 0..P/2, with the 1/P^2 of the inverse DFT.
     p->ramp.assign(p->half, 0.0f);
     if (D > 0) {
+      std::vector<double> cosines(P);
+      for (int j = 0; j < P; ++j) cosines[j] = std::cos(2.0 * M_PI * (long long)j / P);
       for (int m = 0; m < p->half; ++m) {
         double s = 1.0 / (4.0 * delta * delta);
         for (int nn = 1; nn < P / 2; nn += 2) {
           const long long ph = ((long long)m * nn) % P;
-          s += 2.0 * (-1.0 / ((double)nn * nn * M_PI * M_PI * delta * delta)) * std::cos(2.0 * M_PI * ph / P);
+          s += 2.0 * (-1.0 / ((double)nn * nn * M_PI * M_PI * delta * delta)) * cosines[ph];
         }
         if ((P / 2) % 2 == 1) {  // the unpaired tap n = -P/2 (odd only when P = 2)
           const double hn = (double)(P / 2);
@@ -453,15 +455,18 @@ static int plan_create(const recon_geometry* geom, double lambda, double delta, 
         p->theta.assign(recon::kMlpParams, 0.f);
         if (o.mlp_weights) std::memcpy(p->theta.data(), o.mlp_weights, sizeof(float) * recon::kMlpParams);
         p->cnt.assign(lc.n_bins, 0.f);
-        for (int a = -P / 2; a < P / 2; ++a)
-          for (int b = -P / 2; b < P / 2; ++b) {
+        // samples per radial bin, q = isqrt(a^2 + b^2) over -P/2 <= a, b < P/2: by |a| <= |b|, each for its signs
+        // and its transpose, q stepped along b (8 thousand short steps at P = 256 instead of 65 thousand roots)
+        const auto signs = [&](int a) { return a == 0 || a == P / 2 ? 1.f : 2.f; };
+        for (int a = 0; a <= P / 2; ++a) {
+          long long q = a;
+          for (int b = a; b <= P / 2; ++b) {
             const long long msq = (long long)a * a + (long long)b * b;
-            long long q = (long long)std::sqrt((double)msq);
-            while (q * q > msq) --q;
             while ((q + 1) * (q + 1) <= msq) ++q;
             const int bin = (int)(q / lc.bin_width);
-            p->cnt[bin < lc.n_bins - 1 ? bin : lc.n_bins - 1] += 1.f;
+            p->cnt[bin < lc.n_bins - 1 ? bin : lc.n_bins - 1] += signs(a) * signs(b) * (a == b ? 1.f : 2.f);
           }
+        }
         p->x2.assign((size_t)(D > 0 ? D : 1) * nz_layers, 0.f);
         for (int n = 0; n < D; ++n) {
           const double* R = geom->rot + 9 * (size_t)n;
