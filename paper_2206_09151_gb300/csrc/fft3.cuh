@@ -16,6 +16,8 @@
 // flight before its first shared-memory store.
 #pragma once
 
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 #include "fft16.cuh"
@@ -102,6 +104,18 @@ __device__ __forceinline__ void place(int k, int& t, int& v) {
   }
 }
 
+// Load functors with arithmetic behind their loads give them apart: fetch() returns what it read (Raw), finish() makes
+// the value of it, kBatch values at a time, so that the loads of a batch are in flight together (the
+// divisions and roots of finish() branch, and no load moves over a branch).
+template <class In, class = void>
+struct Batch {
+  static constexpr int N = 0;
+};
+template <class In>
+struct Batch<In, std::void_t<typename In::Raw>> {
+  static constexpr int N = In::kBatch;
+};
+
 template <int P, bool INV, class In, class Out>
 __global__ void __launch_bounds__(kThreads) k_lines(const In in_arg, const Out out, long long n_lines,
                                                     const float2* __restrict__ twg) {
@@ -116,11 +130,32 @@ __global__ void __launch_bounds__(kThreads) k_lines(const In in_arg, const Out o
   In in = in_arg;
   in.begin();
   float2 val[E::V];  // a CTA's CB lines of P elements are V per thread
+  if constexpr (Batch<In>::N > 0) {
+    constexpr int N = Batch<In>::N < E::V ? Batch<In>::N : E::V;
+    static_assert(E::V % N == 0, "whole batches");
 #pragma unroll
-  for (int k = 0; k < E::V; ++k) {
-    int t, v;
-    place<P, In::kAlong>(k, t, v);
-    val[k] = l0 + t < n_lines ? in.load(l0 + t, v) : make_float2(0.f, 0.f);
+    for (int k0 = 0; k0 < E::V; k0 += N) {
+      typename In::Raw raw[N];
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        int t, v;
+        place<P, In::kAlong>(k0 + k, t, v);
+        raw[k] = in.fetch(l0 + t < n_lines ? l0 + t : n_lines - 1, v);
+      }
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        int t, v;
+        place<P, In::kAlong>(k0 + k, t, v);
+        val[k0 + k] = l0 + t < n_lines ? in.finish(l0 + t, v, raw[k]) : make_float2(0.f, 0.f);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < E::V; ++k) {
+      int t, v;
+      place<P, In::kAlong>(k, t, v);
+      val[k] = l0 + t < n_lines ? in.load(l0 + t, v) : make_float2(0.f, 0.f);
+    }
   }
 #pragma unroll
   for (int k = 0; k < E::V; ++k) {
