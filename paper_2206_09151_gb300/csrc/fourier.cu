@@ -297,7 +297,10 @@ struct GridQuotient {
     const float inv = 1.f / (s + eps_s);
     float2 F = make_float2(a.x * inv, a.y * inv);
     if constexpr (RAW) {
-      const bool keep = s > 0.f && sqrtf(a.z * a.z + a.w * a.w) * inv >= nsr_m * rsqrtf(fmaxf(s, 1e-30f));
+            // squares fused in this order: the threshold of a cell must not hang on how a compiler contracts them (another
+      // order turned a few decisions in one volume out of three)
+      const float m2 = fmaf(a.w, a.w, a.z * a.z);
+      const bool keep = s > 0.f && sqrtf(m2) * inv >= nsr_m * rsqrtf(fmaxf(s, 1e-30f));
       if (!keep) return make_float2(0.f, 0.f);
     }
     // exp(-2 pi i sum_a m_a c_a / P3_a): the turns are T / (2 Pmax), T = sum_a m_a (2 c_a)
