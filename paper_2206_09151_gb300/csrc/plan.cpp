@@ -1375,19 +1375,26 @@ int run_in_scratch(recon_plan_t p, const float* images, float* volume, char* scr
   // Same table head as the caller-owned workspace, then the largest direction block
   // whose spectra, intermediates and stacks still fit the scratch.
   const size_t spec = (size_t)p->nv * p->half * 8;
-  const size_t inter = (size_t)p->t_rows * p->half * 8 * p->nzl;
   const bool mlp = p->ca.filter == RECON_FILTER_MLP;
   const size_t sub = (size_t)(p->ca.sub_block > 0 ? p->ca.sub_block : 1);
-  auto need = [&](size_t db) {
+  const auto need = [&](size_t db, size_t rows, size_t stack_dir) {
     const size_t sb = db < sub ? db : sub;
-    size_t b = p->table_bytes + align256(sb * spec) + align256(sb * inter) + align256(db * p->stack_dir_bytes);
+    size_t b = p->table_bytes + align256(sb * spec) + align256(sb * rows * p->half * 8 * p->nzl) + align256(db * stack_dir);
     if (mlp) b += align256(sizeof(float) * sb * p->lc.n_bins) + align256(sizeof(float) * sb * p->nzl * p->lc.n_bins);
     return b;
   };
-  if (need(1) > scratch_bytes)
-    return fail(RECON_E_UNSUPPORTED_SIZE, "recon_run_noalloc: this plan needs " + std::to_string(need(1)) +
+  // What one direction needs as tap pairs decides, whatever layout the plan runs with (column stacks need less).
+  const size_t value = p->ca.stack_bf16 ? 2 : 4, pairs_dir = 2 * value * p->nzl * p->ca.layer_elems;
+  if (need(1, p->nv, pairs_dir) > scratch_bytes)
+    return fail(RECON_E_UNSUPPORTED_SIZE, "recon_run_noalloc: this plan needs " +
+                                              std::to_string(need(1, p->nv, pairs_dir)) +
                                               " bytes of scratch for one direction; the static scratch holds " +
                                               std::to_string(scratch_bytes));
+  recon::StageAConst ca = p->ca;
+  const size_t stack_dir = ca.cols ? value * p->nzl * p->nu * ca.wp : pairs_dir;
+  if (need(1, ca.tp, stack_dir) > scratch_bytes) ca.tp = ca.nw;  // T without its rounded-up rows
+  if (need(1, ca.tp, stack_dir) > scratch_bytes)
+    return fail(RECON_E_UNSUPPORTED_SIZE, "recon_run_noalloc: one direction does not fit the static scratch");
   if (p->D == 0 || nvox == 0) {
     if (nvox > 0 && !p->opt.accumulate) {
       cudaError_t e = cudaMemsetAsync(volume, 0, nvox * sizeof(float), s);
@@ -1400,7 +1407,7 @@ int run_in_scratch(recon_plan_t p, const float* images, float* volume, char* scr
     if (rc) return rc;
   }
   size_t db = 1;
-  while ((int)db < p->db && need(db + 1) <= scratch_bytes) ++db;
+  while ((int)db < p->db && need(db + 1, ca.tp, stack_dir) <= scratch_bytes) ++db;
   recon::Workspace w;
   w.dirs = (recon::DirParams*)(scratch + p->off_dirs);
   w.uA = (uint64_t*)(scratch + p->off_uA);
@@ -1414,9 +1421,9 @@ int run_in_scratch(recon_plan_t p, const float* images, float* volume, char* scr
   w.S = (float2*)(scratch + off);
   off += align256(sb * spec);
   w.T = (float2*)(scratch + off);
-  off += align256(sb * inter);
+  off += align256(sb * ca.tp * p->half * 8 * p->nzl);
   w.stack = (void*)(scratch + off);
-  off += align256(db * p->stack_dir_bytes);
+  off += align256(db * stack_dir);
   float* pow = (float*)(scratch + off);
   if (mlp) off += align256(sizeof(float) * sb * p->lc.n_bins);
   w.eps = (float*)(scratch + off);
@@ -1426,7 +1433,6 @@ int run_in_scratch(recon_plan_t p, const float* images, float* volume, char* scr
   if (rc) return rc;
   MlpHookCtx hctx{p, scratch, pow, w.eps, w.S, w.twp};
   const recon::StageAHook hook{mlp_hook, &hctx};
-  recon::StageAConst ca = p->ca;
   if (p->P >= 16) ca.sub_block = (int)sb;
   const int n_blocks = (int)((p->D + db - 1) / db);
   for (int b = 0; b < n_blocks; ++b) {
@@ -1434,7 +1440,7 @@ int run_in_scratch(recon_plan_t p, const float* images, float* volume, char* scr
     const int cnt = (p->D - d0) < (int)db ? (p->D - d0) : (int)db;
     cudaError_t e = recon::launch_stage_a(ca, w, images, d0, cnt, s, nullptr, mlp ? &hook : nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "recon_run_noalloc: stage A launch");
-    // direct kernels only: no wait inside the GPU, so the call need not synchronise
+    // no kernel that reports through a status word, so the call need not synchronise
     e = p->cb.cols_j ? recon::launch_backproject_cols(p->cb, w.dirs, w.stack, d0, cnt, volume,
                                                       p->opt.accumulate || b > 0, s)
                      : recon::launch_backproject(p->cb, w.dirs, w.stack, d0, cnt, volume, p->opt.accumulate || b > 0, s);

@@ -74,7 +74,8 @@ struct StageAConst {
   // the stack hold rows w = 0 .. nw - 1, detector row r_lo + w (b_frac = 0; with tap pairs r_lo = 0,
   // nw = nv) or that row and the next blended with weight b_frac on the next.
   int cols, nw, r_lo, wp;
-  int tp;  // entries between the columns of T: nw rounded up to even, so that a row pair is 16-byte aligned
+  int tp;  // entries between the columns of T: nw rounded up to even, so that a row pair is 16-byte aligned (nw
+           // itself where a fixed scratch does not hold that)
   float b_frac;
   int sub_block;        // directions per stage-A sub-block (S and T sized for it), 0 = whole block
   int pair_mode;        // filter 3 only: 0 the opposite-pair bracket; 1 / 2 the depth factor

@@ -94,6 +94,12 @@ __host__ __device__ constexpr int last_radix() {
   return P / ns;
 }
 
+template <bool WIDE>
+__device__ __forceinline__ float4 row_pair(const float2* p, bool row2) {
+  if constexpr (WIDE) return *reinterpret_cast<const float4*>(p);
+  const float2 a = p[0], b = row2 ? p[1] : make_float2(0.f, 0.f);
+  return make_float4(a.x, a.y, b.x, b.y);
+}
 __device__ __forceinline__ void store_pair(float* out, float2 v) { *reinterpret_cast<float2*>(out) = v; }
 __device__ __forceinline__ void store_pair(__nv_bfloat16* out, float2 v) {
   *reinterpret_cast<__nv_bfloat162*>(out) = __floats2bfloat162_rn(v.x, v.y);
@@ -101,8 +107,9 @@ __device__ __forceinline__ void store_pair(__nv_bfloat16* out, float2 v) {
 __device__ __forceinline__ void store_taps(float2* out, float a, float b) { *out = make_float2(a, b); }
 __device__ __forceinline__ void store_taps(__nv_bfloat162* out, float a, float b) { *out = __floats2bfloat162_rn(a, b); }
 
-// Entry: the stack's, a tap pair (float2, bfloat162) or with COLS a single value.
-template <int P, typename Entry, bool COLS>
+// Entry: the stack's, a tap pair (float2, bfloat162) or with COLS a single value.  WIDE: c.tp is even, so that a row
+// pair of T is one 16-byte load (a scratch too small for the even pitch takes two 8-byte ones).
+template <int P, typename Entry, bool COLS, bool WIDE>
 __global__ void __launch_bounds__(RowsT<P>::NTH, RowsT<P>::MINB) k_rows_inv(const float2* __restrict__ T,
                                                                           Entry* __restrict__ stack,
                                                                           const float2* __restrict__ twg,
@@ -124,11 +131,11 @@ __global__ void __launch_bounds__(RowsT<P>::NTH, RowsT<P>::MINB) k_rows_inv(cons
     for (int s = 0; s < R / 2; ++s) {
       a[s] = b[s] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (row1) {
-        a[s] = *reinterpret_cast<const float4*>(Tk + (size_t)(j + s * B) * c.tp);
-        b[s] = *reinterpret_cast<const float4*>(Tk + (size_t)(jb + s * B) * c.tp);
+        a[s] = row_pair<WIDE>(Tk + (size_t)(j + s * B) * c.tp, row2);
+        b[s] = row_pair<WIDE>(Tk + (size_t)(jb + s * B) * c.tp, row2);
       }
     }
-    if (row1 && j == 0) ny = *reinterpret_cast<const float4*>(Tk + (size_t)(P / 2) * c.tp);
+    if (row1 && j == 0) ny = row_pair<WIDE>(Tk + (size_t)(P / 2) * c.tp, row2);
     for (int i = threadIdx.x; i < C::NT; i += C::NTH) tw[i] = twg[i];
     if (!row2) {
 #pragma unroll
@@ -207,7 +214,7 @@ __global__ void __launch_bounds__(RowsT<P>::NTH, RowsT<P>::MINB) k_rows_inv(cons
   }
 }
 
-template <int P, typename Entry, bool COLS>
+template <int P, typename Entry, bool COLS, bool WIDE>
 cudaError_t launch(const StageAConst& c, const float2* T, void* stack, const float2* twp, int cnt, cudaStream_t stream) {
   using C = RowsT<P>;
   static std::atomic<unsigned long long> attr_set{0};  // devices on which the shared-memory limit is raised
@@ -216,23 +223,27 @@ cudaError_t launch(const StageAConst& c, const float2* T, void* stack, const flo
     cudaGetDevice(&dev);
     if (dev >= 64 || !(attr_set.load() >> dev & 1ull)) {
       const cudaError_t e =
-          cudaFuncSetAttribute(k_rows_inv<P, Entry, COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
+          cudaFuncSetAttribute(k_rows_inv<P, Entry, COLS, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
       if (e != cudaSuccess) return e;
       if (dev < 64) attr_set.fetch_or(1ull << dev);
     }
   }
   const float2* tw = twp + (P >= 1024 ? P - 8 : 0);  // the 16-value table follows the 8-value one
   const dim3 grid((c.nw + 2 * C::G - 1) / (2 * C::G), c.nz_layers, cnt);
-  k_rows_inv<P, Entry, COLS><<<grid, C::NTH, C::smem, stream>>>(T, (Entry*)stack, tw, c);
+  k_rows_inv<P, Entry, COLS, WIDE><<<grid, C::NTH, C::smem, stream>>>(T, (Entry*)stack, tw, c);
   return cudaGetLastError();
+}
+template <int P, bool WIDE>
+cudaError_t launch(const StageAConst& c, const float2* T, void* stack, const float2* twp, int cnt, cudaStream_t s) {
+  if (c.cols)
+    return c.stack_bf16 ? launch<P, __nv_bfloat16, true, WIDE>(c, T, stack, twp, cnt, s)
+                        : launch<P, float, true, WIDE>(c, T, stack, twp, cnt, s);
+  return c.stack_bf16 ? launch<P, __nv_bfloat162, false, WIDE>(c, T, stack, twp, cnt, s)
+                      : launch<P, float2, false, WIDE>(c, T, stack, twp, cnt, s);
 }
 template <int P>
 cudaError_t launch(const StageAConst& c, const float2* T, void* stack, const float2* twp, int cnt, cudaStream_t s) {
-  if (c.cols)
-    return c.stack_bf16 ? launch<P, __nv_bfloat16, true>(c, T, stack, twp, cnt, s)
-                        : launch<P, float, true>(c, T, stack, twp, cnt, s);
-  return c.stack_bf16 ? launch<P, __nv_bfloat162, false>(c, T, stack, twp, cnt, s)
-                      : launch<P, float2, false>(c, T, stack, twp, cnt, s);
+  return c.tp & 1 ? launch<P, false>(c, T, stack, twp, cnt, s) : launch<P, true>(c, T, stack, twp, cnt, s);
 }
 
 }  // namespace

@@ -102,3 +102,24 @@ def test_noalloc_refuses_a_plan_beyond_its_scratch():
     assert e.value.code == _abi.RECON_E_UNSUPPORTED_SIZE
     assert "scratch" in str(e.value)
     _abi.recon_destroy(plan)
+
+
+def test_noalloc_at_the_edge_of_its_scratch_matches_recon_run():
+    """Odd image rows and 60 layers of tap pairs: 65 024 bytes less than the scratch as long as the spectra's rows are
+    not rounded up to even, 58 368 more if they are."""
+    nu, nv, nzl, grid, rot = 200, 149, 60, (16, 24, 16), ph.single_axis_rotations(3)
+    opts = _abi.recon_default_options()
+    opts.bp_kernel = _abi.RECON_BP_DIRECT
+    rng = np.random.default_rng(149)
+    img = torch.from_numpy((1.0 + 1e-2 * rng.standard_normal((3, nv, nu))).astype(np.float32)).cuda()
+    plan = _abi.recon_plan(rot, nu, nv, 1e-10, 1e-9, np.zeros(3), nzl, grid, opts)
+    ws_bytes = _abi.recon_workspace_size(plan)
+    ws = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    ref = torch.empty(grid[::-1], device="cuda")
+    vol = torch.full(grid[::-1], float("nan"), device="cuda")
+    _abi.recon_run(plan, img.data_ptr(), ref.data_ptr(), ws.data_ptr(), ws_bytes, stream)
+    _abi.recon_run_noalloc(plan, img.data_ptr(), vol.data_ptr(), stream)
+    _abi.recon_sync(stream)
+    assert rel_l2(vol, ref) <= TOL_F32
+    _abi.recon_destroy(plan)
