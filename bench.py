@@ -54,37 +54,15 @@ WORKLOAD_TEXT = {
 DEFAULT_STACK = {"mid": "f32", "small": "f32", "learned": "bf16", "slab": "bf16", "batch": "bf16"}
 
 # DRAM traffic per launch (bytes) from ncu captures, keyed by kernel and workload and
-# valid only for the kernel source they were taken on (sha256 of the .cu file).  The column
-# kernels' entries were re-stamped once, after a change to stage_a.cu that touched only the row
-# kernel (its FFT call now asks the engine for twiddle powers, a template branch the column
-# kernels do not take): their code is the captured code.
+# valid only for the kernel source they were taken on (sha256 of the file).
 NCU_TRAFFIC: dict = {
-    # mid (float32): one 40-direction launch each, scaled by 120/40 to the bench's blocks (the
-    # backprojection's volume read-modify-write does not scale; its figure overstates it)
-    ("k_cols", "mid", "f32"): {"bytes_per_launch": (21.171456e6 + 612.15744e6) * 3, "l2_hit_pct": 3.8,
-                               "src": "12ea9f939a270171"},
-    ("k_backproject", "mid", "f32"): {"bytes_per_launch": (617.094656e6 + 59.883008e6) * 3, "l2_hit_pct": 51.1,
-                                      # 171.8 M warp instructions for 40 x 256^3 updates
-                                      "warp_inst_per_update": 171823104 / (40 * 256 ** 3),
-                                      "src": "b7ee0b8780a4373d"},
-    # slab (bf16 stack): the column kernel from one 3-direction sub-block launch (the bench's
-    # launch size); the TMA-staged backprojection from a 6-direction launch, its reads scaled
-    # by 56/6 to the bench's 56-direction blocks (the stack boxes grow with the directions),
-    # plus the volume read of an accumulating block and the volume write (1.07 GB each)
-    ("k_cols", "slab", "bf16"): {"bytes_per_launch": 55.945984e6 + 1.550934e9, "l2_hit_pct": 8.4,
-                                 "src": "12ea9f939a270171"},
-    ("k_backproject", "slab", "bf16"): {"bytes_per_launch": 3.059654e9 * 56 / 6 + 1.073742e9 + 1.055155e9,
-                                        "l2_hit_pct": 56.2,
-                                        # 1.553 G warp instructions for 6 x 1024^2 x 256 updates
-                                        "warp_inst_per_update": 1553227094 / (6 * 1024 * 1024 * 256),
-                                        "src": "f76a56888e3e5455"},
 }
 
 
 # The roof that binds each stage-A kernel (ncu evidence in profiles/): FP32 arithmetic for the
 # column FFT and filter, the L1 / shared-memory pipe for the row stage; the forward row FFTs
 # are small and memory-bound.  The backprojection's depends on the kernel that ran.
-KERNEL_BOUND = {"k_rows_fwd": "hbm", "k_cols": "alu (FP32)", "k_rows_inv": "l1/shared-memory pipe"}
+KERNEL_BOUND = {"k_rows_fwd": "hbm", "k_cols": "alu (FP32)", "k_rows_inv": "hbm, l1/shared-memory pipe"}
 ISSUE_PEAK = 152 * 4 * 2.07e9  # warp instructions per second
 
 
@@ -462,19 +440,20 @@ def run_ours(args):
     counts = [min(db, D - b * db) for b in range(nb)]
     algo = algorithmic_bytes(cfg, r, 2 if args.stack == "bf16" else 4, counts)
     kernels = {}
-    bp_src = "backproject_tma.cu" if r.bp_kernel_used == "tma" else "backproject.cu"
+    bp_src = ("backproject_tma.cu" if r.bp_kernel_used == "tma" else
+              "backproject_cols.cuh" if args.bp_kernel == "auto" else "backproject.cu")
+    kernel_src = ["stage_a.cu", "columns.cu" if r.padded <= 512 else "stage_a.cu", "rows_inv.cu", bp_src]
     for q, name in enumerate(KERNELS):
         per_launch_ms = kern_ms[q] / max(kern_n[q], 1)
         gbs = algo[q] / (kern_ms[q] / args.steps / 1e3) / 1e9 if kern_ms[q] > 0 else None
         tr = ncu_traffic(name, args.workload, args.stack, args.filter)
-        src = bp_src if q == 3 else "stage_a.cu"
-        valid = tr is not None and tr["src"] == _src_hash(src)
+        valid = tr is not None and tr["src"] == _src_hash(kernel_src[q])
         kernels[name] = {"launches": kern_n[q], "ms_per_launch": per_launch_ms,
                          "share": kern_ms[q] / max(sum(kern_ms), 1e-12), "algorithmic_GBps": gbs,
                          "algorithmic_bytes_per_launch": algo[q] * args.steps / max(kern_n[q], 1),
                          "ncu_dram_bytes_per_launch": tr["bytes_per_launch"] if valid else None,
                          "bound": KERNEL_BOUND[name] if q < 3 else
-                         ("issue (FMA/ALU pipes)" if r.bp_kernel_used == "tma" else "l1 (gathers)")}
+                         ("issue (FMA/ALU pipes)" if r.bp_kernel_used == "tma" else "l1 / shared-memory loads")}
         if valid and per_launch_ms > 0:
             # the captured bytes at the bench's launch time, against the measured HBM peak
             kernels[name]["ncu_dram_frac"] = tr["bytes_per_launch"] / (per_launch_ms / 1e3) / 1e9 / peaks["hbm_gbs"]
@@ -489,9 +468,8 @@ def run_ours(args):
                                                if kern_ms[1] > 0 else None)
     dom = max(range(4), key=lambda q: kern_ms[q])
     dom_name = KERNELS[dom]
-    src = bp_src if dom == 3 else "stage_a.cu"
     tr = ncu_traffic(dom_name, args.workload, args.stack, args.filter)
-    traffic = tr["bytes_per_launch"] if tr and tr["src"] == _src_hash(src) else None
+    traffic = tr["bytes_per_launch"] if tr and tr["src"] == _src_hash(kernel_src[dom]) else None
     launches = max(kern_n[dom], 1)
     common = {"kernel": dom_name, "traffic": traffic,
               "algorithmic_bytes_per_launch": algo[dom] * args.steps / launches, "launches": kern_n[dom],
