@@ -362,22 +362,26 @@ struct RealCall {
   }
 };
 
-// The inverse passes after the producing load `in` of axis 2: P, n, off per axis (0 fastest in the
-// half spectrum H [n2][P1 / 2 + 1][P0]), the cropped real volume to vol.
-template <bool ROWS0, class In>
-cudaError_t inverse_real(const In& in, float2* H, float* vol, const int P[3], const int n[3], const int off[3],
-                         const float2* const tw[3], cudaStream_t s) {
-  const long long half = P[1] / 2 + 1, plane = half * P[0];
+// The inverse passes: the first one, along axis 2, from the producing load `in` into the half spectrum H [n2][P1 / 2
+// + 1][P0] (P, n, off per axis, 0 fastest), and the others, the cropped real volume to vol.
+template <class In>
+cudaError_t inverse_first(const In& in, float2* H, const int P[3], const int n[3], const int off[3],
+                          const float2* const tw[3], cudaStream_t s) {
+  const long long plane = (long long)(P[1] / 2 + 1) * P[0];
   const Columns z{H - (long long)off[2] * plane, 62, 0, plane, off[2], off[2] + n[2]};
-  cudaError_t e = launch_lines<true>(P[2], in, z, plane, tw[2], s);
+  return launch_lines<true>(P[2], in, z, plane, tw[2], s);
+}
+template <bool ROWS0>
+cudaError_t inverse_rest(float2* H, float* vol, const int P[3], const int n[3], const int off[3],
+                         const float2* const tw[3], cudaStream_t s) {
   const Rows x{H, P[0], 0, P[0]}, xc{H, P[0], off[0], off[0] + n[0]};
-  if (e == cudaSuccess) e = launch_lines<true>(P[0], x, xc, (long long)n[2] * half, tw[0], s);
+  cudaError_t e = launch_lines<true>(P[0], x, xc, (long long)n[2] * (P[1] / 2 + 1), tw[0], s);
   const RealOut o{H, vol, n[0], n[1], n[2], off[0], off[1], P[0], (float)(1.0 / ((double)P[0] * P[1] * P[2]))};
   if (e == cudaSuccess) e = with_length(P[1], RealCall<ROWS0>{o, tw[1], s});
   return e;
 }
 
-// Complex cells of the half spectrum that inverse_real works in.
+// Complex cells of the half spectrum that the inverse passes work in.
 inline size_t half_cells(const int P[3], int n2) { return (size_t)n2 * (P[1] / 2 + 1) * P[0]; }
 
 }  // namespace fft3

@@ -151,6 +151,24 @@ __device__ __forceinline__ void cell_add(float2* p, float w, float2 z, float2) {
   asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(w * z.x), "f"(w * z.y) : "memory");
 }
 
+// A sample's arithmetic in a written-out order of its fused products, since k_grid_resum forms the same terms again:
+// its point (q_u, q_v, q_z) in DFT bins of each grid axis, ...
+__device__ __forceinline__ void sample_point(const GridDir& d, const Fourier3Const& f, int mu, int mv, float qz,
+                                             float (&g)[3]) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    g[a] = fmaf(qz, d.r[6 + a], fmaf((float)mu, d.r[a], (float)mv * d.r[3 + a])) * f.scale[a];
+}
+// ... and its contrast about the detector centre: G0 (for the mirrored half conj G0) times
+// exp(i pi (mu (nu - 1) + mv (nv - 1)) / P), exact phase.
+__device__ __forceinline__ float2 centred(float2 G0, bool mirror, const StageAConst& c, int mu, int mv) {
+  const int k = (mu * (c.nu - 1) + mv * (c.nv - 1)) % (2 * c.P);
+  float ps, pc;
+  sincospif((float)k / (float)c.P, &ps, &pc);
+  return mirror ? make_float2(fmaf(G0.y, ps, G0.x * pc), fmaf(G0.x, ps, -(G0.y * pc)))
+                : make_float2(fmaf(G0.x, pc, -(G0.y * ps)), fmaf(G0.x, ps, G0.y * pc));
+}
+
 template <typename CellT>
 __device__ __forceinline__ void splat(CellT* acc, float* S, const Fourier3Const& f, const float g[3], float2 z,
                                       float2 gc) {
@@ -194,11 +212,7 @@ __global__ void k_grid_splat(const float2* __restrict__ G, const GridDir* __rest
     const int mu = col == P / 2 ? -P / 2 : col;  // the Nyquist column is bin -P/2 of the full grid
     const int mv = signed_bin(mvi, P);
     const float2 G0 = G[((long long)n * half + col) * P + mvi];
-    // about the detector centre: times exp(i pi (mu (nu - 1) + mv (nv - 1)) / P), exact phase
-    const int k = (mu * (c.nu - 1) + mv * (c.nv - 1)) % (2 * P);
-    float ps, pc;
-    sincospif((float)k / (float)P, &ps, &pc);
-    const float2 gc = make_float2(G0.x * pc - G0.y * ps, G0.x * ps + G0.y * pc);
+    const float2 gc = centred(G0, false, c, mu, mv);
     // Eq. 11's bracket at this view's R_n: chi / (2 pi) in 2^-64 turns, exact modulo 1
     const uint32_t m2 = (uint32_t)(mu * mu + mv * mv);
     const uint64_t m64 = m2;
@@ -211,20 +225,15 @@ __global__ void k_grid_splat(const float2* __restrict__ G, const GridDir* __rest
     // the point (q_u, q_v, -lambda q^2 / 2) in DFT bins of each grid axis
     const float qz = -d.qz_coef * (float)m2;  // in units of 1 / (P delta)
     float g[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) g[a] = ((float)mu * d.r[a] + (float)mv * d.r[3 + a] + qz * d.r[6 + a]) * f.scale[a];
+    sample_point(d, f, mu, mv, qz, g);
     splat(acc, S, f, g, z, gc);
     if (col >= 1 && col < P / 2) {  // the mirror (-mu, -mv): conjugate contrast, same bracket
       // its own bin (-P/2 stays -P/2 on the Nyquist row) and its own centring phase
       const int mvm = mv == -P / 2 ? mv : -mv;
-      const int km = (-mu * (c.nu - 1) + mvm * (c.nv - 1)) % (2 * P);
-      float qs, qc;
-      sincospif((float)km / (float)P, &qs, &qc);
-      const float2 gm = make_float2(G0.x * qc + G0.y * qs, G0.x * qs - G0.y * qc);  // conj(G0) e^{i pi km / P}
+      const float2 gm = centred(G0, true, c, -mu, mvm);
       const float2 zm = make_float2(c.pref * (gm.x * sp + gm.y * cp), c.pref * (gm.y * sp - gm.x * cp));
       float h[3];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) h[a] = ((float)(-mu) * d.r[a] + (float)mvm * d.r[3 + a] + qz * d.r[6 + a]) * f.scale[a];
+      sample_point(d, f, -mu, mvm, qz, h);
       splat(acc, S, f, h, zm, gm);
     }
   }
@@ -253,6 +262,27 @@ __global__ void k_grid_stats(const float* __restrict__ S, long long n, double* _
   }
 }
 
+// The noise filter keeps or drops whole cells by comparing float sums of atomics with a threshold, so for a cell
+// next to it the order in which the atomics land would decide, and the volume change by a plane wave (1e-4 of its
+// norm) from call to call.  Cells within kNearBand of the threshold (far more than the sums' rounding; some thousand
+// of 79 million for 192^3, 180 views) are noted by the pass that takes the decision, summed again in 64 bits in a
+// fixed order (k_grid_resum), and where the sums so rounded decide otherwise, the cell is added to or
+// taken out of the pass's result (k_grid_settle).  A note list that is full leaves its other cells as they were taken.
+// 192^3, 180 views: the call 2.71 ms, 2.66 without.
+constexpr float kNearBand = 0x1p-15f;
+
+// The two sides of the filter's comparison, |contrast| against its noise at a cell of weight s, inv = 1 / (s + eps_S).
+__device__ __forceinline__ void noise_sides(float s, float inv, float x, float y, float nsr_m, float* signal,
+                                            float* noise) {
+  // squares fused in this order: the decision must not hang on how a compiler contracts them
+  *signal = sqrtf(fmaf(y, y, x * x)) * inv;
+  *noise = nsr_m * rsqrtf(fmaxf(s, 1e-30f));
+}
+
+__device__ __forceinline__ float grid_eps(const double* stats) {
+  return stats[1] > 0.0 ? (float)(1e-3 * stats[0] / stats[1]) : 1.f;
+}
+
 // Load functor of the first inverse pass (along z) of the gridding: the Hermitian part, (F(q) +
 // conj F(-q)) / 2, of the quotient F = acc / (S + eps_S) with the noise filter and the phase from
 // the volume centre to the frame origin.  Line l = ix P3y + iy with ix <= P3x / 2.
@@ -266,7 +296,8 @@ struct GridQuotient {
   int kx, ky, kz;             // 2 c_a Pmax / P3_a, c_a = off_a + (n_a - 1) / 2 the volume's centre
   int turn;                   // 2 Pmax
   float inv_pmax, inv_delta, nsr_m, eps_s;
-  __device__ __forceinline__ void begin() { eps_s = stats[1] > 0.0 ? (float)(1e-3 * stats[0] / stats[1]) : 1.f; }
+  NearCells near;
+  __device__ __forceinline__ void begin() { eps_s = grid_eps(stats); }
   using Acc = typename Cell<RAW>::type;
   struct Raw {
     float s, sm;  // the cells at q and -q: weight,
@@ -292,17 +323,26 @@ struct GridQuotient {
     r.am = sums(r.sm, m);
     return r;
   }
-  __device__ __forceinline__ float2 quotient(int ix, int iy, int iz, float s, const Acc& a) const {
+  __device__ __forceinline__ float2 quotient(int ix, int iy, int iz, float s, const Acc& a, bool note) const {
     if (s == 0.f) return make_float2(0.f, 0.f);
     const float inv = 1.f / (s + eps_s);
-    float2 F = make_float2(a.x * inv, a.y * inv);
     if constexpr (RAW) {
-            // squares fused in this order: the threshold of a cell must not hang on how a compiler contracts them (another
-      // order turned a few decisions in one volume out of three)
-      const float m2 = fmaf(a.w, a.w, a.z * a.z);
-      const bool keep = s > 0.f && sqrtf(m2) * inv >= nsr_m * rsqrtf(fmaxf(s, 1e-30f));
+      float signal, noise;
+      noise_sides(s, inv, a.z, a.w, nsr_m, &signal, &noise);
+      const bool keep = s > 0.f && signal >= noise;
+      if (note && fabsf(signal - noise) < kNearBand * noise) {
+        const unsigned int at = atomicAdd(near.count, 1u);
+        if (at < near.cap) {
+          near.cells[at] = 2 * (unsigned long long)cell(ix, iy, iz) + (keep ? 1 : 0);
+          for (int q = 0; q < 3; ++q) near.sums[3 * (size_t)at + q] = 0.0;
+        }
+      }
       if (!keep) return make_float2(0.f, 0.f);
     }
+    return placed(ix, iy, iz, make_float2(a.x * inv, a.y * inv));
+  }
+  // F with the phase from the volume centre to the frame origin, over Delta.
+  __device__ __forceinline__ float2 placed(int ix, int iy, int iz, float2 F) const {
     // exp(-2 pi i sum_a m_a c_a / P3_a): the turns are T / (2 Pmax), T = sum_a m_a (2 c_a)
     // (Pmax / P3_a) an exact integer, reduced modulo 2 Pmax (a power of two)
     const int T = (signed_bin(ix, P3x) * kx + signed_bin(iy, P3y) * ky + signed_bin(iz, P3z) * kz) & (turn - 1);
@@ -312,11 +352,121 @@ struct GridQuotient {
   }
   __device__ __forceinline__ float2 finish(long long l, int iz, const Raw& r) const {
     const int iy = (int)(l & (P3y - 1)), ix = (int)(l >> ly);
-    const float2 a = quotient(ix, iy, iz, r.s, r.a);
-    const float2 b = quotient((P3x - ix) & (P3x - 1), (P3y - iy) & (P3y - 1), (P3z - iz) & (P3z - 1), r.sm, r.am);
+    // every cell is noted once: where it is q itself, the cells beyond the half where they are -q
+    const float2 a = quotient(ix, iy, iz, r.s, r.a, true);
+    const float2 b = quotient((P3x - ix) & (P3x - 1), (P3y - iy) & (P3y - 1), (P3z - iz) & (P3z - 1), r.sm, r.am,
+                              ix > 0 && ix < P3x / 2);
     return make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
   }
 };
+
+// The noted cells' sums over `n_dirs` views in 64 bits: a warp per cell, its lanes over the views, in a fixed order.  A
+// view's samples that reach the cell lie around the cell's projection onto the view's axes, so a few are tried.
+__global__ void k_grid_resum(const float2* __restrict__ G, const GridDir* __restrict__ dirs, int dir_begin, int n_dirs,
+                             StageAConst c, Fourier3Const f, int lx, int ly, int reach, NearCells near) {
+  const int P = c.P, lane = threadIdx.x & 31;
+  const unsigned int n = min(*near.count, near.cap);
+  for (unsigned int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < n; e += (gridDim.x * blockDim.x) >> 5) {
+    const long long cell = (long long)(near.cells[e] >> 1);
+    const int at[3] = {signed_bin((int)(cell >> ly) & (f.P3[0] - 1), f.P3[0]), signed_bin((int)cell & (f.P3[1] - 1), f.P3[1]),
+                       signed_bin((int)(cell >> (lx + ly)), f.P3[2])};
+    double s = 0.0, x = 0.0, y = 0.0;
+    for (int v = lane; v < n_dirs; v += 32) {
+      const GridDir& d = dirs[dir_begin + v];
+      // half widths, in samples, of the cell's reach along the view's axes
+      float h[3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        h[q] = 1.f + fabsf(d.r[3 * q]) / f.scale[0] + fabsf(d.r[3 * q + 1]) / f.scale[1] + fabsf(d.r[3 * q + 2]) / f.scale[2];
+      // the grid is periodic: samples land on a cell's images up to `reach` periods further too
+      const int side = 2 * reach + 1;
+      for (int image = 0; image < side * side * side; ++image) {
+        const int b[3] = {at[0] + (image % side - reach) * f.P3[0], at[1] + (image / side % side - reach) * f.P3[1],
+                          at[2] + (image / (side * side) - reach) * f.P3[2]};
+        float p[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          p[q] = (float)b[0] / f.scale[0] * d.r[3 * q] + (float)b[1] / f.scale[1] * d.r[3 * q + 1] +
+                 (float)b[2] / f.scale[2] * d.r[3 * q + 2];
+        // q_z at the projection, and how far it varies over the window
+        const float qz0 = -d.qz_coef * (p[0] * p[0] + p[1] * p[1]);
+        const float vary = d.qz_coef * (2.f * (fabsf(p[0]) * h[0] + fabsf(p[1]) * h[1]) + h[0] * h[0] + h[1] * h[1]);
+        if (fabsf(p[2] - qz0) > h[2] + vary) continue;
+        const int u1 = min(P / 2 - 1, (int)floorf(p[0] + h[0])), v1 = min(P / 2 - 1, (int)floorf(p[1] + h[1]));
+        for (int mu = max(-P / 2, (int)ceilf(p[0] - h[0])); mu <= u1; ++mu)
+          for (int mv = max(-P / 2, (int)ceilf(p[1] - h[1])); mv <= v1; ++mv) {
+            float g[3], w[3];
+            sample_point(d, f, mu, mv, -d.qz_coef * (float)(uint32_t)(mu * mu + mv * mv), g);
+            bool hit = true;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+              const float fl = floorf(g[a]);
+              const int to = b[a] - (int)fl;  // 0 or 1: the cell is a corner of the sample's
+              hit &= to == 0 || to == 1;
+              w[a] = to ? g[a] - fl : 1.f - (g[a] - fl);
+            }
+            const float wt = w[0] * w[1] * w[2];
+            if (!hit || wt == 0.f) continue;
+            const bool mirror = mu < 0 && mu > -P / 2;  // from column -mu, whose row -P/2 stays
+            const int col = abs(mu), row = mirror && mv > -P / 2 ? -mv : mv;
+            const float2 gc = centred(G[((long long)v * c.half + col) * P + (row & (P - 1))], mirror, c, mu, mv);
+            s += (double)wt;
+            x += (double)__fmul_rn(wt, gc.x);
+            y += (double)__fmul_rn(wt, gc.y);
+          }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s += __shfl_down_sync(0xffffffffu, s, o);
+      x += __shfl_down_sync(0xffffffffu, x, o);
+      y += __shfl_down_sync(0xffffffffu, y, o);
+    }
+    if (lane == 0) {
+      double* t = near.sums + 3 * (size_t)e;
+      t[0] += s;
+      t[1] += x;
+      t[2] += y;
+    }
+  }
+}
+
+// A warp per noted cell: where the 64-bit sums, rounded, decide otherwise, the cell's share of its z lines (transformed
+// already, planes off .. off + n of H) is added or taken out.
+__global__ void k_grid_settle(const GridQuotient<true> in, float2* __restrict__ H, int off, int n) {
+  const int lane = threadIdx.x & 31;
+  const unsigned int noted = min(*in.near.count, in.near.cap);
+  const float eps_s = grid_eps(in.stats);
+  const long long plane = (long long)(in.P3x / 2 + 1) * in.P3y;
+  for (unsigned int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < noted; e += (gridDim.x * blockDim.x) >> 5) {
+    const long long cell = (long long)(in.near.cells[e] >> 1);
+    const bool kept = in.near.cells[e] & 1;
+    const double* t = in.near.sums + 3 * (size_t)e;
+    const float sum = (float)t[0];
+    float signal, noise;
+    noise_sides(sum, 1.f / (sum + eps_s), (float)t[1], (float)t[2], in.nsr_m, &signal, &noise);
+    const bool keep = signal >= noise;
+    if (!(sum > 0.f) || keep == kept) continue;
+    const int iy = (int)cell & (in.P3y - 1), ix = (int)(cell >> in.ly) & (in.P3x - 1), iz = (int)(cell >> (in.lx + in.ly));
+    const float inv = (keep ? 0.5f : -0.5f) / (in.S[cell] + eps_s);  // half: of the Hermitian part
+    const float4 a = in.acc[cell];
+    const float2 F = in.placed(ix, iy, iz, make_float2(a.x * inv, a.y * inv));
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {  // as q, and conjugate as -q
+      const int jx = m ? (in.P3x - ix) & (in.P3x - 1) : ix, jy = m ? (in.P3y - iy) & (in.P3y - 1) : iy;
+      const int jz = m ? (in.P3z - iz) & (in.P3z - 1) : iz;
+      if (jx > in.P3x / 2) continue;
+      const float Fy = m ? -F.y : F.y;
+      for (int z = lane; z < n; z += 32) {
+        float ps, pc;
+        sincospif(2.f * (float)((jz * (z + off)) & (in.P3z - 1)) / (float)in.P3z, &ps, &pc);
+        float2* h = H + z * plane + (long long)jx * in.P3y + jy;
+        atomicAdd(&h->x, F.x * pc - Fy * ps);
+        atomicAdd(&h->y, F.x * ps + Fy * pc);
+      }
+    }
+  }
+}
 
 // frac(t) in 2^-64 turns (t >= 0)
 uint64_t turns_fixed(double t) {
@@ -396,7 +546,8 @@ cudaError_t launch_swap_phase(const float2* Z, float2* H, float* vol, const Four
   k.sy = (Pmax / f.P3[1]) * (Pmax / f.P3[1]);
   k.sz = (Pmax / f.P3[2]) * (Pmax / f.P3[2]);
   const SwapPhase in{Z, f.P3[0], f.P3[1], f.P3[2], k};
-  return fft3::inverse_real<true>(in, H, vol, f.P3, f.n, f.off, tw, s);
+  const cudaError_t e = fft3::inverse_first(in, H, f.P3, f.n, f.off, tw, s);
+  return e == cudaSuccess ? fft3::inverse_rest<true>(H, vol, f.P3, f.n, f.off, tw, s) : e;
 }
 
 cudaError_t launch_grid_splat(const float2* G, const GridDir* dirs, int dir_begin, int n_dirs, const StageAConst& c,
@@ -410,14 +561,18 @@ cudaError_t launch_grid_splat(const float2* G, const GridDir* dirs, int dir_begi
   return cudaGetLastError();
 }
 
+unsigned int grid_near_cap(const Fourier3Const& f) {
+  const long long cells = (long long)f.P3[0] * f.P3[1] * f.P3[2];
+  return (unsigned int)std::min<long long>(1 << 18, std::max<long long>(1024, cells / 64));
+}
+
 template <bool RAW>
-static cudaError_t grid_inverse(const void* acc, const float* S, const double* stats, float2* H, float* vol,
-                                const Fourier3Const& f, float nsr_m, const float2* const tw[3], cudaStream_t s) {
+static GridQuotient<RAW> grid_quotient(const GridSums& g, const Fourier3Const& f) {
   const int Pmax = std::max(f.P3[0], std::max(f.P3[1], f.P3[2]));
   GridQuotient<RAW> in;
-  in.acc = (const typename Cell<RAW>::type*)acc;
-  in.S = S;
-  in.stats = stats;
+  in.acc = (const typename Cell<RAW>::type*)g.acc;
+  in.S = g.S;
+  in.stats = g.stats;
   in.P3x = f.P3[0];
   in.P3y = f.P3[1];
   in.P3z = f.P3[2];
@@ -429,24 +584,49 @@ static cudaError_t grid_inverse(const void* acc, const float* S, const double* s
   in.turn = 2 * Pmax;
   in.inv_pmax = 1.f / (float)Pmax;  // a power of two: exact
   in.inv_delta = (float)(1.0 / f.delta);
-  in.nsr_m = nsr_m;
+  in.nsr_m = g.nsr_m;
   in.eps_s = 0.f;  // set on the device from stats
+  in.near = g.near;
+  return in;
+}
+
+cudaError_t launch_grid_quotient(const GridSums& g, const Fourier3Const& f, const float2* const tw[3], cudaStream_t s) {
+  const long long nb = (long long)f.P3[0] * f.P3[1] * f.P3[2];
+  cudaError_t e = cudaMemsetAsync(g.stats, 0, 2 * sizeof(double), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(g.near.count, 0, sizeof(unsigned int), s);
+  if (e != cudaSuccess) return e;
+  k_grid_stats<<<grid_blocks(nb), 256, 0, s>>>(g.S, nb, g.stats);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   int P[3], n[3], off[3];
   grid_axes(f, P, n, off);
   const float2* const twp[3] = {tw[1], tw[0], tw[2]};
-  return fft3::inverse_real<false>(in, H, vol, P, n, off, twp, s);
+  return g.nsr_m > 0.f ? fft3::inverse_first(grid_quotient<true>(g, f), g.H, P, n, off, twp, s)
+                       : fft3::inverse_first(grid_quotient<false>(g, f), g.H, P, n, off, twp, s);
 }
 
-cudaError_t launch_grid_finish(const void* acc, const float* S, double* stats, float2* H, float* vol,
-                               const Fourier3Const& f, float nsr_m, const float2* const tw[3], cudaStream_t s) {
-  const long long nb = (long long)f.P3[0] * f.P3[1] * f.P3[2];
-  cudaError_t e = cudaMemsetAsync(stats, 0, 2 * sizeof(double), s);
-  if (e != cudaSuccess) return e;
-  k_grid_stats<<<grid_blocks(nb), 256, 0, s>>>(S, nb, stats);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return nsr_m > 0.f ? grid_inverse<true>(acc, S, stats, H, vol, f, nsr_m, tw, s)
-                     : grid_inverse<false>(acc, S, stats, H, vol, f, nsr_m, tw, s);
+cudaError_t launch_grid_resum(const GridSums& g, const float2* G, const GridDir* dirs, int dir_begin, int n_dirs,
+                              const StageAConst& c, const Fourier3Const& f, cudaStream_t s) {
+  // samples reach sqrt(2) P / 2 in the image plane and lambda / (4 Delta) P along the beam.  Beyond 8 pixels of
+  // wavelength (no image resolves that) the images of a cell are too many to try: its sums stay 0 and settle nothing
+  const double reach = 0.7072 + f.lam / (4.0 * f.delta);
+  if (reach > 2.8) return cudaSuccess;
+  k_grid_resum<<<device_sm_count() * 4, 128, 0, s>>>(G, dirs, dir_begin, n_dirs, c, f, log2_int(f.P3[0]),
+                                                     log2_int(f.P3[1]), (int)(reach + 1.0), g.near);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_grid_finish(const GridSums& g, float* vol, const Fourier3Const& f, const float2* const tw[3],
+                               cudaStream_t s) {
+  if (g.nsr_m > 0.f) {
+    k_grid_settle<<<device_sm_count(), 128, 0, s>>>(grid_quotient<true>(g, f), g.H, f.off[2], f.n[2]);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  int P[3], n[3], off[3];
+  grid_axes(f, P, n, off);
+  const float2* const twp[3] = {tw[1], tw[0], tw[2]};
+  return fft3::inverse_rest<false>(g.H, vol, P, n, off, twp, s);
 }
 
 }  // namespace recon

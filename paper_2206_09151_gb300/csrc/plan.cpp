@@ -1158,7 +1158,7 @@ SwapLayout swap_layout(recon_plan_t p) {
 }
 
 struct GridLayout {
-  size_t Srows, G, dirs, acc, S, H, stats, tw[3], total;
+  size_t Srows, G, dirs, near_cells, near_sums, near_count, acc, S, H, stats, tw[3], total;
   int sub;
 };
 
@@ -1173,6 +1173,13 @@ GridLayout grid_layout(recon_plan_t p) {
   off = align256(off + (size_t)L.sub * p->half * p->P * sizeof(float2));
   L.dirs = off;
   off = align256(off + p->gdirs.size() * sizeof(recon::GridDir));
+  const size_t cap = recon::grid_near_cap(p->f3);
+  L.near_cells = off;
+  off = align256(off + cap * sizeof(unsigned long long));
+  L.near_sums = off;
+  off = align256(off + cap * 3 * sizeof(double));
+  L.near_count = off;
+  off = align256(off + sizeof(unsigned int));
   L.acc = off;
   off = align256(off + grid3_cells(p) * sizeof(float4));
   L.S = off;
@@ -1327,6 +1334,7 @@ int recon_grid_run(recon_plan_t p, const float* images, float* volume, double ns
   recon::GridDir* gd = (recon::GridDir*)(b + L.dirs);
   void* acc = b + L.acc;
   float* S = (float*)(b + L.S);
+  const float nsr_m = (float)(nsr * std::sqrt((double)p->nu * p->nv));
   const size_t cells = grid3_cells(p);
   cudaError_t e = cudaMemcpyAsync(gd, p->gdirs.data(), sizeof(recon::GridDir) * p->gdirs.size(),
                                   cudaMemcpyHostToDevice, s);
@@ -1334,16 +1342,26 @@ int recon_grid_run(recon_plan_t p, const float* images, float* volume, double ns
   if (e == cudaSuccess) e = cudaMemsetAsync(S, 0, cells * sizeof(float), s);
   float2* Srows = (float2*)(b + L.Srows);
   float2* G = (float2*)(b + L.G);
+  const auto spectra = [&](int d0, int cnt) {
+    const cudaError_t er = recon::launch_rows_fwd(p->ca, Srows, w.twp, images, d0, cnt, s);
+    return er == cudaSuccess ? recon::launch_cols_forward(p->ca, p->lc, Srows, G, nullptr, w.twp, cnt, s) : er;
+  };
   for (int d0 = 0; d0 < p->D && e == cudaSuccess; d0 += L.sub) {
     const int cnt = std::min(L.sub, p->D - d0);
-    e = recon::launch_rows_fwd(p->ca, Srows, w.twp, images, d0, cnt, s);
-    if (e == cudaSuccess) e = recon::launch_cols_forward(p->ca, p->lc, Srows, G, nullptr, w.twp, cnt, s);
+    e = spectra(d0, cnt);
     if (e == cudaSuccess) e = recon::launch_grid_splat(G, gd, d0, cnt, p->ca, p->f3, acc, S, nsr > 0.0, s);
   }
-  const float nsr_m = (float)(nsr * std::sqrt((double)p->nu * p->nv));
+  const recon::GridSums sums{acc, S, (double*)(b + L.stats), (float2*)(b + L.H),
+                             {(unsigned long long*)(b + L.near_cells), (double*)(b + L.near_sums),
+                              (unsigned int*)(b + L.near_count), recon::grid_near_cap(p->f3)}, nsr_m};
   const float2* twa[3] = {axis_tw(p, tw[0], 0), axis_tw(p, tw[1], 1), axis_tw(p, tw[2], 2)};
-  if (e == cudaSuccess)
-    e = recon::launch_grid_finish(acc, S, (double*)(b + L.stats), (float2*)(b + L.H), volume, p->f3, nsr_m, twa, s);
+  if (e == cudaSuccess) e = recon::launch_grid_quotient(sums, p->f3, twa, s);
+  for (int d0 = 0; nsr_m > 0.f && d0 < p->D && e == cudaSuccess; d0 += L.sub) {
+    const int cnt = std::min(L.sub, p->D - d0);
+    if (L.sub < p->D) e = spectra(d0, cnt);  // else G still holds every view's
+    if (e == cudaSuccess) e = recon::launch_grid_resum(sums, G, gd, d0, cnt, p->ca, p->f3, s);
+  }
+  if (e == cudaSuccess) e = recon::launch_grid_finish(sums, volume, p->f3, twa, s);
   if (e != cudaSuccess) return cuda_fail(e, "recon_grid_run");
   return RECON_OK;
 }

@@ -238,9 +238,29 @@ size_t swap_half_cells(const Fourier3Const& f);
 // contrast; with_raw) or a float2 (the first alone), S its weight; H: grid_half_cells complex cells.
 cudaError_t launch_grid_splat(const float2* G, const GridDir* dirs, int dir_begin, int n_dirs, const StageAConst& c,
                               const Fourier3Const& f, void* acc, float* S, bool with_raw, cudaStream_t s);
-cudaError_t launch_grid_finish(const void* acc, const float* S, double* stats, float2* H, float* vol,
-                               const Fourier3Const& f, float nsr_m, const float2* const tw[3], cudaStream_t s);
 size_t grid_half_cells(const Fourier3Const& f);
+// The inverse of the gridded sums: launch_grid_quotient (eps_S, the quotient and the first transform pass), with the
+// noise filter (nsr_m > 0) launch_grid_resum for every block of views, launch_grid_finish.
+struct NearCells {            // cells next to the noise filter's threshold
+  unsigned long long* cells;  // 2 cell + (1: kept)
+  double* sums;               // [cap][3]: weight and contrast in 64 bits
+  unsigned int* count;
+  unsigned int cap;
+};
+unsigned int grid_near_cap(const Fourier3Const& f);
+struct GridSums {
+  const void* acc;
+  const float* S;
+  double* stats;
+  float2* H;
+  NearCells near;
+  float nsr_m;
+};
+cudaError_t launch_grid_quotient(const GridSums& g, const Fourier3Const& f, const float2* const tw[3], cudaStream_t s);
+cudaError_t launch_grid_resum(const GridSums& g, const float2* G, const GridDir* dirs, int dir_begin, int n_dirs,
+                              const StageAConst& c, const Fourier3Const& f, cudaStream_t s);
+cudaError_t launch_grid_finish(const GridSums& g, float* vol, const Fourier3Const& f, const float2* const tw[3],
+                               cudaStream_t s);
 
 // Whole-operator run with its workspace carved from `scratch` (tables first, then
 // the largest direction block that fits); used by recon_run_noalloc.
