@@ -1334,11 +1334,11 @@ int recon_grid_run(recon_plan_t p, const float* images, float* volume, double ns
   recon::GridDir* gd = (recon::GridDir*)(b + L.dirs);
   void* acc = b + L.acc;
   float* S = (float*)(b + L.S);
-  const float nsr_m = (float)(nsr * std::sqrt((double)p->nu * p->nv));
+  const float nsr_m = (float)(nsr * std::sqrt((double)p->nu * p->nv));  // 0: no filter, and the sums' other layout
   const size_t cells = grid3_cells(p);
   cudaError_t e = cudaMemcpyAsync(gd, p->gdirs.data(), sizeof(recon::GridDir) * p->gdirs.size(),
                                   cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, cells * (nsr > 0.0 ? sizeof(float4) : sizeof(float2)), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, cells * (nsr_m > 0.f ? sizeof(float4) : sizeof(float2)), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(S, 0, cells * sizeof(float), s);
   float2* Srows = (float2*)(b + L.Srows);
   float2* G = (float2*)(b + L.G);
@@ -1349,7 +1349,7 @@ int recon_grid_run(recon_plan_t p, const float* images, float* volume, double ns
   for (int d0 = 0; d0 < p->D && e == cudaSuccess; d0 += L.sub) {
     const int cnt = std::min(L.sub, p->D - d0);
     e = spectra(d0, cnt);
-    if (e == cudaSuccess) e = recon::launch_grid_splat(G, gd, d0, cnt, p->ca, p->f3, acc, S, nsr > 0.0, s);
+    if (e == cudaSuccess) e = recon::launch_grid_splat(G, gd, d0, cnt, p->ca, p->f3, acc, S, nsr_m > 0.f, s);
   }
   const recon::GridSums sums{acc, S, (double*)(b + L.stats), (float2*)(b + L.H),
                              {(unsigned long long*)(b + L.near_cells), (double*)(b + L.near_sums),

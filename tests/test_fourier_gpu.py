@@ -143,3 +143,14 @@ def test_noise_filter_decides_alike_in_whatever_order_its_sums_are_added():
             first = vol(bits)
             assert all(same(vol(bits), first) for _ in range(15)), (t, bits - lo)
     r.close()
+
+
+def test_gridding_with_a_noise_ratio_below_float32_is_the_one_without_the_filter():
+    from paper_2206_09151_gb300.recon import Reconstructor
+    grid, D = (20, 24, 16), 12
+    img, rot, Rs = _scan(grid, 24, 24, D, 2 * math.pi, 4e-10, 20e-9)
+    r = Reconstructor(rot, 24, 24, grid, lam=4e-10, delta=1e-9, defocus=Rs, nz_layers=4, sigma=0.3, eps=1e-2)
+    im = torch.from_numpy(img).cuda()
+    ref, got = (r.grid_run(im, nsr).cpu().numpy() for nsr in (0.0, 1e-50))
+    r.close()
+    assert rel_l2(got, ref) <= TOL_F32, rel_l2(got, ref)
