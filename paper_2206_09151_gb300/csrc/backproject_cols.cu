@@ -99,8 +99,11 @@ __global__ void __launch_bounds__(cols::kThreads, 2) k_backproject_cols_persiste
   __shared__ unsigned long long s_bars[2 * cols::kStages];
   const cols::Ring ring = cols::init_ring(s_bars, smem_cols, cols::fixed_bytes<J>(), stage_bytes);
   uint32_t uses = 0;
+  const BatchBp* fenced = nullptr;
   for (unsigned n = blockIdx.x; n < total && uses != cols::kFailed; n += gridDim.x) {
     const Item it = batch_item(desc, n_desc, n);
+    if (it.d != fenced) acquire_map(&it.d->map);  // by every warp: each issues loads
+    fenced = it.d;
     uses = it.d->c.stack_bf16 ? cols_item<__nv_bfloat16, J>(it, smem_cols, ring, uses)
                               : cols_item<float, J>(it, smem_cols, ring, uses);
   }

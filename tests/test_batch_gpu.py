@@ -213,3 +213,40 @@ def test_batch_with_host_images_matches_the_device_image_run():
     b.close()
     for r in recons:
         r.close()
+
+
+def test_two_batches_one_after_the_other_in_one_workspace():
+    """Batches of single-axis scans of other sizes, layers and stack types whose descriptors and
+    stacks take the same places of one workspace, in turn and without a pause: every volume
+    is the one of its plan run alone."""
+    from paper_2206_09151_gb300 import _abi
+    from paper_2206_09151_gb300.recon import Batch, Reconstructor
+    rng = np.random.default_rng(11)
+    batches = []
+    for specs in (((40, 44, 1, "f32", 33), (64, 64, 4, "f32", 12)), ((64, 50, 3, "bf16", 40), (24, 90, 6, "f32", 9)),
+                  ((33, 37, 2, "f32", 20),)):
+        recons, images, ref = [], [], []
+        for n, nu, layers, stack, D in specs:
+            rot = ph.single_axis_rotations(D, start=0.2)
+            kw = dict(lam=1e-10, delta=1e-9, defocus=rng.uniform(50e-9, 80e-9, D), nz_layers=layers, sigma=0.05, eps=0.02,
+                      stack_dtype=stack)
+            img = torch.from_numpy((1.0 + 1e-2 * rng.standard_normal((D, n, nu))).astype(np.float32)).cuda()
+            r = Reconstructor(rot, nu, n, (n, n, n), **kw)
+            recons.append(r)
+            images.append(img)
+            ref.append(r.run(img))
+        batches.append((Batch(recons, dir_block=16), images, ref))
+    ws = torch.empty(max(b.ws_bytes for b, _, _ in batches), dtype=torch.uint8, device="cuda")
+    s = torch.cuda.current_stream().cuda_stream
+    got = []
+    for _ in range(4):
+        for b, images, ref in batches:
+            vols = [torch.full_like(v, float("nan")) for v in ref]
+            _abi.recon_batch_run(b.batch, [im.data_ptr() for im in images], [v.data_ptr() for v in vols], ws.data_ptr(),
+                                 ws.numel(), s, False)
+            got.append((vols, ref))
+    for vols, ref in got:
+        for v, a in zip(vols, ref):
+            assert rel_l2(v.cpu(), a.cpu()) <= 1e-5
+    for b, _, _ in batches:
+        b.close()
