@@ -234,13 +234,14 @@ int recon_filter_stage(recon_plan_t plan, const float* images, int dir_begin, in
 int recon_backproject(recon_plan_t plan, const void* stack, int dir_begin, int dir_count, float* volume,
                       int accumulate, void* workspace, size_t ws_bytes, void* stream);
 
-/* Self-test of the failure detection of the TMA-staged backprojection: launches it on
- * one voxel tile whose producer issues no copy, so every consumer's wait on its
- * stage runs out after the 2 s limit; the kernel then sets its status bit and returns
- * without touching the GPU's state.  Allocates and frees 16 KB of device memory and
- * synchronises `stream`.  RECON_OK when the kernel reported the run-out wait (the
- * expected outcome, after about 2 s), RECON_E_DEVICE_CHECK if it did not, RECON_E_CUDA
- * on a CUDA error. */
+/* Self-test of the failure detection of the two backprojection kernels with bounded waits.
+ * The TMA-staged one runs on one voxel tile whose producer issues no copy, so every
+ * consumer's wait on its stage runs out after the 2 s limit; the kernel then sets its
+ * status bit and returns without touching the GPU's state.  The column-stack one runs in its
+ * three forms (a CTA per tile, a cluster, the batch's persistent kernel) with no copy and a
+ * limit of 10 ms, and must leave NaN in every voxel that it owes.  Allocates and frees 4 MB
+ * of device memory and synchronises `stream`.  RECON_OK when both behaved so (the expected
+ * outcome, after about 2 s), RECON_E_DEVICE_CHECK if not, RECON_E_CUDA on a CUDA error. */
 int recon_selftest_wait_limit(void* stream);
 
 /* ---------------------------------------------------------------- batches

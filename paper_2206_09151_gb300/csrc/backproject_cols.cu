@@ -83,8 +83,11 @@ template <typename ST, int J>
 __device__ __noinline__ uint32_t cols_item(const Item& it, unsigned char* smem, const cols::Ring& ring, uint32_t uses) {
   const BackprojConst& c = it.d->c;
   cols::Pair acc[cols::kB * cols::kB][2];
-  uses = cols::tile_sums<ST, J, true>(it.bx, it.by, it.bz, it.d->dirs, &it.d->map, c, it.d->dir_begin, 0, it.d->dir_count,
-                                smem, ring, uses, acc);
+  if (uses != cols::kFailed)
+    uses = cols::tile_sums<ST, J, true>(it.bx, it.by, it.bz, it.d->dirs, &it.d->map, c, it.d->dir_begin, 0,
+                                        it.d->dir_count, smem, ring, uses, acc);
+  else  // a wait of an earlier item ran out: the warp is out of step with the ring and leaves no voxel unwritten
+    cols::nan_sums(acc);
   cols::write_tile<J>(it.bx, it.by, it.bz, c, it.d->vol, it.d->accumulate != 0, acc);
   if (it.bz == 0 && c.nw < c.ny && !it.d->accumulate) cols::clear_beside<J>(it.bx, it.by, c, it.d->vol);
   return uses;
@@ -100,7 +103,7 @@ __global__ void __launch_bounds__(cols::kThreads, 2) k_backproject_cols_persiste
   const cols::Ring ring = cols::init_ring(s_bars, smem_cols, cols::fixed_bytes<J>(), stage_bytes);
   uint32_t uses = 0;
   const BatchBp* fenced = nullptr;
-  for (unsigned n = blockIdx.x; n < total && uses != cols::kFailed; n += gridDim.x) {
+  for (unsigned n = blockIdx.x; n < total; n += gridDim.x) {
     const Item it = batch_item(desc, n_desc, n);
     if (it.d != fenced) acquire_map(&it.d->map);  // by every warp: each issues loads
     fenced = it.d;

@@ -27,7 +27,7 @@
 // direction two ahead and otherwise advance on their own (a barrier per direction for the whole
 // CTA cost a seventh of the time, as warps differ in the lines that span layers; a ninth warp for
 // the preparation costs the others 24 registers).  Every wait is bounded; one that runs out leaves NaN
-// in the tile's voxels.  A cluster of CTAs may share a tile's directions; their sums are
+// in the warp's voxels, in the batch's persistent form in those of its later items too.  A cluster of CTAs may share a tile's directions; their sums are
 // added in rank order through distributed shared memory, so the result does not depend on timing.
 #pragma once
 
@@ -244,6 +244,10 @@ struct Ring {
   uint32_t stage_bytes;
 };
 
+__device__ __forceinline__ unsigned long long wait_limit(const BackprojConst& c) {
+  return c.cols_probe_ns ? (unsigned long long)c.cols_probe_ns : kWaitNs;
+}
+
 // One warp: the records of a tile for one direction (d of the block that `map` describes) and the load of its
 // box, into stage `use` mod kStages; false if the wait for the stage ran out.
 template <typename ST, int J>
@@ -253,7 +257,7 @@ __device__ __forceinline__ bool prepare(int bz, const Info& f, const CUtensorMap
   constexpr int ROWB = J * (int)sizeof(ST);
   const int lane = threadIdx.x & 31, W = c.cols_w;
   const uint32_t s = use % kStages;
-  if (!__all_sync(0xffffffffu, mbar_wait(ring.empty + 8 * s, ((use / kStages) & 1u) ^ 1u))) return false;
+  if (!__all_sync(0xffffffffu, mbar_wait(ring.empty + 8 * s, ((use / kStages) & 1u) ^ 1u, wait_limit(c)))) return false;
   Stage<J>& st = reinterpret_cast<Stage<J>*>(smem)[s];
 #pragma unroll
   for (int q = 0; q < T::LINES / 32; ++q) {
@@ -276,9 +280,15 @@ __device__ __forceinline__ bool prepare(int bz, const Info& f, const CUtensorMap
   __syncwarp();
   if (lane == 0) {
     mbar_expect_tx(ring.full + 8 * s, (uint32_t)(W * c.cols_l * ROWB));  // releases the records above
-    tma_load_4d(ring.boxes + s * ring.stage_bytes, map, bz * J, f.c0, f.L0, d, ring.full + 8 * s);
+    if (!c.cols_probe_ns) tma_load_4d(ring.boxes + s * ring.stage_bytes, map, bz * J, f.c0, f.L0, d, ring.full + 8 * s);
   }
   return true;
+}
+
+__device__ __forceinline__ void nan_sums(Pair (&acc)[kB * kB][2]) {
+  const float nan = __int_as_float(0x7FC00000);
+#pragma unroll
+  for (int v = 0; v < kB * kB; ++v) acc[v][0] = acc[v][1] = pack(nan, nan);
 }
 
 // The sums of tile (bx, by, bz) over the directions [d0, d1) of a block.  Returns the new count; a warp whose
@@ -310,7 +320,7 @@ __device__ __forceinline__ uint32_t tile_sums(int bx, int by, int bz, const DirP
   if (warp < kStages - 1 && warp < count) ok = ready(warp);
   uint32_t s = uses % kStages, parity = (uses / kStages) & 1u;
   for (int n = 0; ok && n < count; ++n) {
-    ok = __all_sync(0xffffffffu, mbar_wait(ring.full + 8 * s, parity));
+    ok = __all_sync(0xffffffffu, mbar_wait(ring.full + 8 * s, parity, wait_limit(c)));
     if (!ok) break;
     const Stage<J>& st = stages[s];
     const uint32_t box = ring.boxes + s * ring.stage_bytes + (uint32_t)(jl * 4 * (int)sizeof(ST));
@@ -334,12 +344,10 @@ __device__ __forceinline__ uint32_t tile_sums(int bx, int by, int bz, const DirP
   if ((tid & 31) == 0) {
     const uint32_t end = uses + (uint32_t)count;
     for (uint32_t m = end - uses > kStages ? end - kStages : uses; m < end; ++m)
-      mbar_wait(ring.full + 8 * (m % kStages), (m / kStages) & 1u);
+      mbar_wait(ring.full + 8 * (m % kStages), (m / kStages) & 1u, wait_limit(c));
   }
   __syncwarp();
-  const float nan = __int_as_float(0x7FC00000);
-#pragma unroll
-  for (int v = 0; v < kB * kB; ++v) acc[v][0] = acc[v][1] = pack(nan, nan);
+  nan_sums(acc);
   return kFailed;
 }
 

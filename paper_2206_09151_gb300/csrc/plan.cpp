@@ -1066,6 +1066,88 @@ int recon_backproject(recon_plan_t p, const void* stack, int dir_begin, int dir_
   return tma_end(p, workspace, s, "recon_backproject");
 }
 
+// The column-stack kernel with waits that run out (no box is loaded; limit 10 ms): one CTA per tile, a cluster,
+// and the batch's persistent form, where the CTA of the first item also has later ones.  NaN, and nothing
+// unwritten, is what it must leave.
+static int cols_wait_probe(cudaStream_t s) {
+  constexpr int kDirs = 12, kSide = 800;
+  double rot[9 * kDirs], defocus[kDirs] = {};
+  for (int n = 0; n < kDirs; ++n) {
+    const double c = std::cos(0.2 * n), si = std::sin(0.2 * n), r[9] = {c, 0, si, 0, 1, 0, -si, 0, c};
+    std::copy(r, r + 9, rot + 9 * n);
+  }
+  const recon_geometry geom{kDirs, 16, 16, rot};
+  recon_options o;
+  recon_default_options(&o);
+  struct Plans {
+    recon_plan_t p[2] = {nullptr, nullptr};
+    void* buf = nullptr;
+    ~Plans() {
+      for (recon_plan_t q : p) recon_destroy(q);
+      if (buf) cudaFree(buf);
+    }
+  } own;
+  const recon_grid grids[2] = {{16, 16, 16}, {kSide, 1, kSide}};
+  for (int q = 0; q < 2; ++q) {
+    const int rc = plan_create(&geom, 1e-10, 1e-9, defocus, 1, &grids[q], &o, &own.p[q], false);
+    if (rc) return rc;
+  }
+  const recon_plan_t small = own.p[0], wide = own.p[1];
+  if (small->cb.cols_j == 0 || small->cb.cols_j != wide->cb.cols_j)
+    return fail(RECON_E_DEVICE_CHECK, "recon_selftest_wait_limit: the probe's plans are not of one column-stack class");
+  const size_t n_small = 16 * 16 * 16, n_wide = (size_t)kSide * kSide, n_all = n_small + n_wide;
+  const size_t off_vol = align256(sizeof(recon::DirParams) * 2 * kDirs), off_desc = align256(off_vol + 4 * n_all);
+  const size_t off_stack = align256(off_desc + 2 * sizeof(recon::BatchBp));
+  const size_t stack = kDirs * std::max(small->stack_dir_bytes, wide->stack_dir_bytes), bytes = off_stack + stack;
+  cudaError_t e = cudaMalloc(&own.buf, bytes);
+  if (e != cudaSuccess) return cuda_fail(e, "recon_selftest_wait_limit: allocation");
+  char* b = (char*)own.buf;
+  auto* dirs = (recon::DirParams*)b;
+  float* vol = (float*)(b + off_vol);
+  recon::BackprojConst held = small->cb;
+  held.cols_probe_ns = 10000000;
+  std::vector<float> got(n_all);
+  for (int form = 0; form < 3 && e == cudaSuccess; ++form) {
+    e = cudaMemsetAsync(b, 0, bytes, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(dirs, small->dirs.data(), sizeof(recon::DirParams) * kDirs, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(dirs + kDirs, wide->dirs.data(), sizeof(recon::DirParams) * kDirs, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(vol, 0x40, 4 * n_all, s);  // 3.0039 everywhere
+    size_t n = n_small;
+    if (form < 2) {
+      if (e == cudaSuccess) e = recon::launch_backproject_cols(held, dirs, b + off_stack, 0, form ? kDirs : 1, vol, 0, s);
+    } else {
+      n = n_all;
+      recon::BatchBp desc[2];
+      if (e == cudaSuccess) e = recon::describe_backproject(held, dirs, b + off_stack, 0, 1, vol, 0, &desc[0]);
+      if (e == cudaSuccess)
+        e = recon::describe_backproject(wide->cb, dirs + kDirs, b + off_stack, 0, 1, vol + n_small, 0, &desc[1]);
+      desc[0].first_item = 0;
+      desc[1].first_item = (unsigned long long)desc[0].gx * desc[0].gy * desc[0].gz;
+      if (e == cudaSuccess) e = cudaMemcpyAsync(b + off_desc, desc, sizeof desc, cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess)
+        e = recon::launch_backproject_cols_persistent(
+            (const recon::BatchBp*)(b + off_desc), 2,
+            desc[1].first_item + (unsigned long long)desc[1].gx * desc[1].gy * desc[1].gz, held.cols_j,
+            std::max(recon::cols_smem_bytes(held), recon::cols_smem_bytes(wide->cb)), s);
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(got.data(), vol, 4 * n, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) break;
+    size_t nan = 0, unwritten = 0;
+    for (size_t i = 0; i < n; ++i) {
+      nan += std::isnan(got[i]) && i >= (form < 2 ? 0 : n_small);
+      unwritten += i < n_small ? !std::isnan(got[i]) : !(std::isnan(got[i]) || got[i] == 0.f);
+    }
+    if (unwritten != 0 || nan == 0)
+      return fail(RECON_E_DEVICE_CHECK, "recon_selftest_wait_limit: the column-stack kernel (form " + std::to_string(form) +
+                                            ") left " + std::to_string(unwritten) + " voxels without NaN after a run-out wait, " +
+                                            std::to_string(nan) + " with");
+  }
+  return e == cudaSuccess ? RECON_OK : cuda_fail(e, "recon_selftest_wait_limit: column stacks");
+}
+
 int recon_selftest_wait_limit(void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   void* buf = nullptr;
@@ -1082,7 +1164,7 @@ int recon_selftest_wait_limit(void* stream) {
   if (e != cudaSuccess) return cuda_fail(e, "recon_selftest_wait_limit");
   if ((h & 1u) == 0)
     return fail(RECON_E_DEVICE_CHECK, "recon_selftest_wait_limit: the kernel did not report its run-out wait");
-  return RECON_OK;
+  return cols_wait_probe(s);
 }
 
 int recon_profile_enable(recon_plan_t p, int enable) {

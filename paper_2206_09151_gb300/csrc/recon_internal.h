@@ -155,6 +155,7 @@ struct BackprojConst {
   // column stack (backproject_cols.cuh): cols_j rows per tile (0: not used), the staged box of cols_w
   // columns x cols_l layers in stages of cols_stage bytes; nw rows from volume row j_lo, wp entries apart
   int cols_j, cols_w, cols_l, cols_stage, nw, j_lo, wp;
+  int cols_probe_ns;  // 0, or (self-test) the limit of its waits, with no box ever loaded
   int warp_cols;     // general kernel: a warp's patch of voxel columns is warp_cols x 32/warp_cols
 };
 

@@ -149,3 +149,27 @@ def test_tile_depths_agree_and_the_tuner_picks_one():
     assert rel_l2(vols[8], vols[16]) <= TOL_F32
     out = tune_bp_tile(rot, nu, nu, grid, img, nz_layers=7, candidates=(8, 16), repeats=2, **kw)
     assert out["bp_tile_z"] in (8, 16) and set(out["ms"]) == {"8", "16"}
+
+
+def test_column_stack_waits_that_run_out_leave_nan_and_a_usable_context():
+    """The self-test also holds the column-stack kernel's boxes back, in its single, clustered and
+    persistent forms, and refuses if any voxel is left unwritten (the persistent CTA's later items among
+    them); single-axis runs and a batch afterwards still match the direct kernel."""
+    from paper_2206_09151_gb300.recon import Batch, Reconstructor
+    s = torch.cuda.current_stream()
+    assert _abi.recon_selftest_wait_limit(int(s.cuda_stream)) == _abi.RECON_OK, _abi.recon_last_error()
+    rng = np.random.default_rng(2)
+    rot = ph.single_axis_rotations(9, start=0.1)
+    img = torch.from_numpy((1.0 + 1e-2 * rng.standard_normal((9, 20, 24))).astype(np.float32)).cuda()
+    kw = dict(lam=1e-10, delta=1e-9, defocus=np.full(9, 60e-9), nz_layers=3, sigma=0.05, eps=0.02)
+    vols = {}
+    for k in ("direct", "auto"):
+        r = Reconstructor(rot, 24, 20, (40, 24, 30), bp_kernel=k, **kw)
+        vols[k] = r.run(img).cpu().numpy()
+        if k == "auto":
+            b = Batch([r])
+            vols["batch"] = b.run([img])[0].cpu().numpy()
+            b.close()
+        r.close()
+    assert rel_l2(vols["auto"], vols["direct"]) <= TOL_F32
+    assert rel_l2(vols["batch"], vols["direct"]) <= TOL_F32
