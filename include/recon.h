@@ -59,7 +59,8 @@ extern "C" {
 #define RECON_E_NO_WEIGHTS (-7)       /* RECON_FILTER_MLP without its network parameters */
 #define RECON_E_DEVICE_CHECK (-8)     /* a kernel's own check failed: a bounded wait ran out
                                          (2 s) or a footprint left its staging box; the call
-                                         synchronised its stream and the output is incomplete */
+                                         (recon_sync for the asynchronous ones) synchronised
+                                         its stream and the output is incomplete              */
 
 /* ---------------------------------------------------------------- option values */
 #define RECON_FILTER_OFF 0       /* H = 1: ramp-filtered backprojection of g (Eq. 15)   */
@@ -100,8 +101,9 @@ extern "C" {
                                     of the first kind (recon_run and its forms, the batch)
                                     keep single values along the detector columns instead
                                     of tap pairs between the two stages where that layout
-                                    fits; its kernel's bounded waits leave NaN if one runs
-                                    out, and the call stays asynchronous                  */
+                                    fits; the call stays asynchronous, and if one of its
+                                    kernel's bounded waits runs out, the voxels concerned
+                                    are NaN and recon_sync says so                        */
 #define RECON_BP_DIRECT 1        /* bilinear gathers straight from the stack (single-axis
                                     kernel, or the general kernel)                       */
 #define RECON_BP_STAGED 2        /* single-axis: footprint staged in shared memory        */
@@ -239,7 +241,7 @@ int recon_backproject(recon_plan_t plan, const void* stack, int dir_begin, int d
  * consumer's wait on its stage runs out after the 2 s limit; the kernel then sets its
  * status bit and returns without touching the GPU's state.  The column-stack one runs in its
  * three forms (a CTA per tile, a cluster, the batch's persistent kernel) with no copy and a
- * limit of 10 ms, and must leave NaN in every voxel that it owes.  Allocates and frees 4 MB
+ * limit of 10 ms, must leave NaN in every voxel that it owes and have recon_sync report it.  Allocates and frees 4 MB
  * of device memory and synchronises `stream`.  RECON_OK when both behaved so (the expected
  * outcome, after about 2 s), RECON_E_DEVICE_CHECK if not, RECON_E_CUDA on a CUDA error. */
 int recon_selftest_wait_limit(void* stream);
@@ -422,7 +424,9 @@ int recon_profile_read(recon_plan_t plan, double* ms, int* launches);
  * Calls no cudaMalloc, cudaFree or allocating library routine. */
 int recon_run_noalloc(recon_plan_t plan, const float* images, float* volume, void* stream);
 
-/* Waits for `stream` and reports a CUDA error raised by earlier kernels. */
+/* Waits for `stream` and reports a CUDA error raised by earlier kernels, or
+ * (RECON_E_DEVICE_CHECK, once) that since the last call a bounded wait of the column-stack
+ * backprojection ran out on the current device, in whichever stream. */
 int recon_sync(void* stream);
 
 /* Frees the plan.  NULL is a no-op. */

@@ -180,6 +180,16 @@ cudaError_t launch_cols_t(const BackprojConst& c, const DirParams* dirs, const v
 
 }  // namespace
 
+cudaError_t take_wait_failures(unsigned int* n, cudaStream_t stream) {
+  void* count = nullptr;
+  cudaError_t e = cudaGetSymbolAddress(&count, cols::wait_failures);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(n, count, sizeof *n, cudaMemcpyDeviceToHost, stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  if (e == cudaSuccess && *n) e = cudaMemsetAsync(count, 0, sizeof *n, stream);
+  if (e == cudaSuccess && *n) e = cudaStreamSynchronize(stream);
+  return e;
+}
+
 size_t cols_smem_bytes(const BackprojConst& c) {
   const size_t fixed = c.cols_j == 64 ? cols::fixed_bytes<64>() : cols::fixed_bytes<32>();
   const size_t dump = c.cols_j == 64 ? cols::Tile<64>::kDumpBytes : cols::Tile<32>::kDumpBytes;

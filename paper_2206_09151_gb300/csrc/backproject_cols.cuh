@@ -27,7 +27,7 @@
 // direction two ahead and otherwise advance on their own (a barrier per direction for the whole
 // CTA cost a seventh of the time, as warps differ in the lines that span layers; a ninth warp for
 // the preparation costs the others 24 registers).  Every wait is bounded; one that runs out leaves NaN
-// in the warp's voxels, in the batch's persistent form in those of its later items too.  A cluster of CTAs may share a tile's directions; their sums are
+// in the warp's voxels, in the batch's persistent form in those of its later items too, and is counted for recon_sync.  A cluster of CTAs may share a tile's directions; their sums are
 // added in rank order through distributed shared memory, so the result does not depend on timing.
 #pragma once
 
@@ -84,6 +84,8 @@ template <int J>
 __host__ __device__ constexpr size_t fixed_bytes() {
   return (kStages * sizeof(Stage<J>) + kWarps * kOwn * sizeof(Info) + 127) / 128 * 128;
 }
+
+__device__ unsigned int wait_failures;  // warps whose wait ran out, since recon_sync last took it
 
 constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: x + kMagic, rounded down, holds floor(x) in its low mantissa bits
 constexpr int kMagicBits = 0x4B400000;
@@ -347,6 +349,7 @@ __device__ __forceinline__ uint32_t tile_sums(int bx, int by, int bz, const DirP
       mbar_wait(ring.full + 8 * (m % kStages), (m / kStages) & 1u, wait_limit(c));
   }
   __syncwarp();
+  if ((tid & 31) == 0) atomicAdd(&wait_failures, 1u);
   nan_sums(acc);
   return kFailed;
 }

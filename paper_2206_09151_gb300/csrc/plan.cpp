@@ -1144,6 +1144,10 @@ static int cols_wait_probe(cudaStream_t s) {
       return fail(RECON_E_DEVICE_CHECK, "recon_selftest_wait_limit: the column-stack kernel (form " + std::to_string(form) +
                                             ") left " + std::to_string(unwritten) + " voxels without NaN after a run-out wait, " +
                                             std::to_string(nan) + " with");
+    if (recon_sync(s) != RECON_E_DEVICE_CHECK)
+      return fail(RECON_E_DEVICE_CHECK, "recon_selftest_wait_limit: recon_sync did not report the run-out wait");
+    const int rc = recon_sync(s);
+    if (rc) return rc;
   }
   return e == cudaSuccess ? RECON_OK : cuda_fail(e, "recon_selftest_wait_limit: column stacks");
 }
@@ -1457,6 +1461,12 @@ int recon_sync(void* stream) {
   if (e != cudaSuccess) return cuda_fail(e, "recon_sync");
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "recon_sync");
+  unsigned int failed = 0;
+  e = recon::take_wait_failures(&failed, (cudaStream_t)stream);
+  if (e != cudaSuccess) return cuda_fail(e, "recon_sync");
+  if (failed)
+    return fail(RECON_E_DEVICE_CHECK, "recon_sync: a bounded wait of the column-stack backprojection ran out (" +
+                                          std::to_string(failed) + " warps); voxels of a run on this device hold NaN");
   return RECON_OK;
 }
 

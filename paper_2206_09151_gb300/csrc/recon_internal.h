@@ -166,6 +166,8 @@ cudaError_t launch_backproject(const BackprojConst& c, const DirParams* dirs, co
 // cols_w, cols_l, cols_stage, nw, j_lo and wp (cols_j = 0 where the scan does not fit it).
 void cols_setup(BackprojConst& c, const DirParams* dirs, int n_dirs);
 size_t cols_smem_bytes(const BackprojConst& c);
+// Waits for `stream` and takes the current device's count of its run-out waits (then 0 again).
+cudaError_t take_wait_failures(unsigned int* n, cudaStream_t stream);
 cudaError_t launch_backproject_cols(const BackprojConst& c, const DirParams* dirs, const void* stack, int dir_begin,
                                     int dir_count, float* volume, int accumulate, cudaStream_t stream);
 
