@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(ColsT<P>::NTH, P >= 256 ? 2 : 4)
           if constexpr (FILT == 3) {
             f[i] = amp[i] * cos_half_turns((int32_t)hi[i]);
           } else {  // real part of the Eq. 11 bracket
-            const float e = FILT == 2 ? fmaxf(__ldg(eps_k + bin[i]), FLT_MIN) : eps0;
+            const float e = FILT == 2 ? positive_eps(__ldg(eps_k + bin[i])) : eps0;
             f[i] = inverse_ctf(sin_half_turns((int32_t)hi[i]), e);
           }
           hi[i] += step[i];

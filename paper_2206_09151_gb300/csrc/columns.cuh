@@ -37,6 +37,13 @@ __device__ __forceinline__ uint32_t phase_step(uint64_t dA, uint32_t m) {
   return (uint32_t)((dA * m + 0x80000000ull) >> 32);
 }
 
+// The learned eps, at least FLT_MIN; a NaN (of the network's weights) stays one, which fmaxf would hide.
+__device__ __forceinline__ float positive_eps(float eps) {
+  float e;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(e) : "f"(eps), "f"(FLT_MIN));
+  return e;
+}
+
 // sn / (sn^2 + eps), eps >= FLT_MIN: one reciprocal (the general divide also scales for subnormal divisors).
 __device__ __forceinline__ float inverse_ctf(float sn, float eps) {
   float r;

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
           sincos_half_turns((int32_t)hi[s], &sn, &cs);
           f = fmaf(sp[s], cs, -cp[s] * sn);
         } else {  // real part of the Eq. 11 bracket
-          const float e = FILT == 2 ? fmaxf(__ldg(eps_k + (bins[s / 4] >> 8 * (s % 4) & 255u)), FLT_MIN) : eps0;
+          const float e = FILT == 2 ? positive_eps(__ldg(eps_k + (bins[s / 4] >> 8 * (s % 4) & 255u))) : eps0;
           f = inverse_ctf(sin_half_turns((int32_t)hi[s]), e);
         }
         hi[s] += step[s];

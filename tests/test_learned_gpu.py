@@ -220,3 +220,19 @@ def test_training_gradient_at_the_edges_of_its_tiles(n, views, nzl):
                                            r_eff=r_eff, nsr=1e-2, **PHYS)
     assert abs(loss[0] - ref_loss) <= 1e-5 * ref_loss, (loss[0], ref_loss)
     assert rel_l2(grad, ref_grad) <= 1e-4, rel_l2(grad, ref_grad)
+
+
+@pytest.mark.parametrize("nu,nv", [(8, 3), (24, 20), (300, 5), (600, 3)])
+def test_a_nan_of_the_network_reaches_the_layers(nu, nv):
+    """A NaN bias of the output unit makes every eps NaN: every layer value is NaN, in every column kernel (the transform
+    lengths 16, 64, 1024 and 2048), and not the finite layers of the smallest eps."""
+    from paper_2206_09151_gb300.recon import Reconstructor
+    w = _weights(3).astype(np.float32)
+    w[-1] = np.nan
+    rot = ph.single_axis_rotations(2)
+    r = Reconstructor(rot, nu, nv, (8, 8, 8), defocus=np.full(2, 60e-9), nz_layers=3, filter="mlp", mlp_weights=w, nsr=1e-2,
+                      lam=PHYS["lam"], delta=PHYS["delta"], sigma=PHYS["sigma"])
+    img = torch.from_numpy((1.0 + 0.05 * np.random.default_rng(1).standard_normal((2, nv, nu))).astype(np.float32)).cuda()
+    layers = r.filter_stage(img, 0, 2)[:, :, 1:nv + 1, 1:, 0]
+    assert bool(torch.isnan(layers).all())
+    r.close()
