@@ -107,14 +107,16 @@ __device__ __forceinline__ Info make_info(const DirParams& p, const BackprojCons
   f.du = fabsf(du);
   f.dt = dt;
   // u is a chain of FMAs, monotone in the voxel indices, and the depth an exact integer sum: the
-  // extremes are at the tile's corners
+  // extremes are at the tile's corners (for the depth at those of its part inside the volume: 32 bits hold no
+  // depth from 128 layers on)
+  const int x_in = min(ti_n, c.nx - i0) - 1, z_in = min(kTK, c.nz - k0) - 1;
   float umin = 1e30f;
   int lmin = INT32_MAX;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int x = q & 1 ? ti_n - 1 : 0, z = q & 2 ? kTK - 1 : 0;
     umin = fminf(umin, fmaf(f.af0, (float)x, fmaf(f.af2, (float)z, f.fa)));
-    lmin = min(lmin, (int32_t)(f.t + f.ti * (uint32_t)x + f.tk * (uint32_t)z) >> 24);
+    lmin = min(lmin, (int32_t)(f.t + f.ti * (uint32_t)(q & 1 ? x_in : 0) + f.tk * (uint32_t)(q & 2 ? z_in : 0)) >> 24);
   }
   // where u falls along the lines, their 5 columns end at the tap above the first u, up to one column
   // below the tile's least u

@@ -377,3 +377,21 @@ def test_column_stack_runs_match_oracle_and_the_tap_pair_kernel(grid, nu, nv, nz
         r.close()
     assert rel_l2(out["auto"], ref) <= (TOL_F32 if stack == "f32" else TOL_BF16)
     assert rel_l2(out["auto"], out["direct"]) <= TOL_F32
+
+
+def test_column_stack_depths_beyond_the_volume_do_not_move_the_box():
+    """96 layers over 66 voxels along the beam: the last tile reaches 29 voxels past the volume, to a depth
+    of 138 layers, which 32 bits do not hold."""
+    rng = np.random.default_rng(66)
+    grid, nu, nv, nzl = (66, 32, 20), 70, 32, 96
+    img = (1.0 + 0.05 * rng.standard_normal((1, nv, nu))).astype(np.float32)
+    rot = ph.single_axis_rotations(1, start=-0.5 * math.pi)
+    kw = dict(lam=1e-10, delta=1e-9, defocus=np.full(1, 60e-9), nz_layers=nzl, sigma=0.05, eps=0.02)
+    ref = O.recon(img, rot, grid=grid, filt=O.FILTER_TIKHONOV, **kw)
+    out = {}
+    for kernel in ("auto", "direct"):
+        r = make(rot, nu, nv, grid, filter="tikhonov", stack_dtype="bf16", bp_kernel=kernel, **kw)
+        out[kernel] = r.run(torch.from_numpy(img).cuda()).cpu().numpy()
+        r.close()
+    assert rel_l2(out["auto"], ref) <= TOL_BF16
+    assert rel_l2(out["auto"], out["direct"]) <= TOL_F32
