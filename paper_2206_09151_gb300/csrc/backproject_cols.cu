@@ -112,6 +112,8 @@ __global__ void __launch_bounds__(cols::kThreads, 2) k_backproject_cols_persiste
   }
 }
 
+constexpr int kMaxSmem = 220 * 1024;  // what a plan's boxes may take
+
 // CTAs that share a tile's directions: the split whose last wave is fullest, each CTA's prologue,
 // first loads and write-out counted as 5 directions' work.
 int pick_split(long long tiles, int slots, int dirs) {
@@ -152,7 +154,8 @@ cudaError_t launch_cols_t(const BackprojConst& c, const DirParams* dirs, const v
   using T = cols::Tile<J>;
   auto* kernel = k_backproject_cols<ST, J, LAYERS>;
   const size_t smem = cols_smem_bytes(c);
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static std::atomic<unsigned long long> raised{0};
+  cudaError_t e = raise_smem_limit(raised, (const void*)kernel, kMaxSmem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, cols::kThreads, smem);
@@ -232,7 +235,7 @@ void cols_setup(BackprojConst& c, const DirParams* dirs, int n_dirs) {
     c.cols_w = (int)W;
     c.cols_l = (int)L;
     c.cols_stage = (int)((W * L * J * (c.stack_bf16 ? 2 : 4) + 127) / 128 * 128);
-    if (cols_smem_bytes(c) <= 220 * 1024) return;
+    if (cols_smem_bytes(c) <= (size_t)kMaxSmem) return;
     c.cols_j = 0;
   }
 }
@@ -250,7 +253,8 @@ cudaError_t describe_backproject_cols(const BackprojConst& c, BatchBp* out) {
 template <int J>
 static cudaError_t launch_persistent_t(const BatchBp* desc, int n_desc, unsigned total, size_t smem, cudaStream_t stream) {
   auto* kernel = k_backproject_cols_persistent<J>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static std::atomic<unsigned long long> raised{0};
+  cudaError_t e = raise_smem_limit(raised, (const void*)kernel, kMaxSmem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, cols::kThreads, smem);

@@ -49,6 +49,7 @@ namespace {
 // The tile is 16 x 16 x TZ voxels, TZ (voxels along z per thread) a run-time choice of
 // the plan: 16 (the default, measured faster on the slab) or 8.
 constexpr int kMX = 16, kMY = 16;
+constexpr int kMaxSmem = 200 * 1024;  // what a plan's boxes may take
 constexpr int kConsumerWarps = 8;
 constexpr int kThreads = (kConsumerWarps + 1) * 32;
 constexpr long long kMargin = 1LL << 30;               // 2^-10 pixel in 2^-40 pixel units
@@ -416,8 +417,8 @@ cudaError_t launch_tma_t(const BackprojConst& c, const TmaBox& box, const DirPar
   g.box_bytes = (uint32_t)((size_t)box.W * box.H * box.L * es);
   g.stall = stall;
   const size_t smem = (size_t)box.stages * (box.stage_bytes + 16 + sizeof(Rec));
-  cudaError_t e = cudaFuncSetAttribute(k_backproject_tma<ST, LIN, kMZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  static std::atomic<unsigned long long> raised{0};
+  cudaError_t e = raise_smem_limit(raised, (const void*)k_backproject_tma<ST, LIN, kMZ>, kMaxSmem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_backproject_tma<ST, LIN, kMZ>, kThreads, smem);
@@ -485,7 +486,7 @@ TmaBox tma_box_for(const BackprojConst& c, const DirParams* dirs, int n_dirs, in
   b.stages = (int)std::min<size_t>(RECON_TMA_MAX_STAGES, st);
   if (b.stages < 2) b.stages = 2 * (b.stage_bytes + 16 + sizeof(Rec)) <= (size_t)200 * 1024 ? 2 : 1;
   const size_t smem = (size_t)b.stages * (b.stage_bytes + 16 + sizeof(Rec));
-  b.ok = W <= 256 && H <= 256 && L <= 256 && smem <= 200 * 1024;
+  b.ok = W <= 256 && H <= 256 && L <= 256 && smem <= (size_t)kMaxSmem;
   return b;
 }
 

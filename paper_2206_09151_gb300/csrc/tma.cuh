@@ -6,6 +6,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 #include <mutex>
 
@@ -73,6 +74,17 @@ inline PFN_cuTensorMapEncodeTiled_v12000 encode_tiled() {
       fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
   });
   return fn;
+}
+
+// Lets `kernel` take up to `bytes` of dynamic shared memory, once per device (a bit each in `raised`) and always the
+// same: a limit set for one launch's own size could be lowered by another thread's before the launch.
+inline cudaError_t raise_smem_limit(std::atomic<unsigned long long>& raised, const void* kernel, int bytes) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || (dev < 64 && (raised.load() >> dev & 1ull))) return e;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && dev < 64) raised.fetch_or(1ull << dev);
+  return e;
 }
 
 }  // namespace recon

@@ -395,3 +395,39 @@ def test_column_stack_depths_beyond_the_volume_do_not_move_the_box():
         r.close()
     assert rel_l2(out["auto"], ref) <= TOL_BF16
     assert rel_l2(out["auto"], out["direct"]) <= TOL_F32
+
+
+@pytest.mark.parametrize("bp_kernel", ["auto", "tma"])
+def test_plans_of_other_box_sizes_run_from_several_threads(bp_kernel):
+    """Plans that launch one kernel with small and with large boxes of shared memory, from threads of their own on
+    streams of their own."""
+    import threading
+    jobs, errors = [], []
+    for nzl in (2, 12, 2, 12):
+        n, D = 16, 1
+        rot = ph.single_axis_rotations(D, start=0.7)
+        img = torch.from_numpy((1.0 + 0.05 * np.random.default_rng(nzl).standard_normal((D, n, n))).astype(np.float32)).cuda()
+        kw = dict(lam=1e-10, delta=1e-9, defocus=np.full(D, 60e-9), nz_layers=nzl, sigma=0.05, eps=0.02)
+        r = make(rot, n, n, (n, 64, n), bp_kernel=bp_kernel, **kw)
+        jobs.append((r, img, r.run(img), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+
+    def work(r, img, ref, stream):
+        try:
+            with torch.cuda.stream(stream):
+                vol = torch.empty_like(ref)
+                for _ in range(4000):
+                    r.run(img, vol)
+                stream.synchronize()
+                assert torch.equal(vol, ref)
+        except Exception as e:  # reported by the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for j in jobs:
+        j[0].close()
