@@ -33,6 +33,7 @@
 
 #include <cuda_bf16.h>
 
+#include "recon.h"
 #include "recon_internal.h"
 #include "tma.cuh"
 
@@ -107,16 +108,18 @@ __device__ __forceinline__ Info make_info(const DirParams& p, const BackprojCons
   f.du = fabsf(du);
   f.dt = dt;
   // u is a chain of FMAs, monotone in the voxel indices, and the depth an exact integer sum: the
-  // extremes are at the tile's corners (for the depth at those of its part inside the volume: 32 bits hold no
-  // depth from 128 layers on)
-  const int x_in = min(ti_n, c.nx - i0) - 1, z_in = min(kTK, c.nz - k0) - 1;
+  // extremes are at the tile's corners.  Corners beyond the volume lie up to 58 layers (the deepest box) off the
+  // stack's at most 96: counted from its middle, so that 32 bits hold the depth (clamping the corners to the
+  // volume instead cost the kernel 8 %: 442 us against 410 for 320^3, 60 directions)
+  constexpr int kMiddle = RECON_MAX_LAYERS / 2;
+  const uint32_t tm = f.t - ((uint32_t)kMiddle << 24);
   float umin = 1e30f;
   int lmin = INT32_MAX;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int x = q & 1 ? ti_n - 1 : 0, z = q & 2 ? kTK - 1 : 0;
     umin = fminf(umin, fmaf(f.af0, (float)x, fmaf(f.af2, (float)z, f.fa)));
-    lmin = min(lmin, (int32_t)(f.t + f.ti * (uint32_t)(q & 1 ? x_in : 0) + f.tk * (uint32_t)(q & 2 ? z_in : 0)) >> 24);
+    lmin = min(lmin, (int32_t)(tm + f.ti * (uint32_t)x + f.tk * (uint32_t)z) >> 24);
   }
   // where u falls along the lines, their 5 columns end at the tap above the first u, up to one column
   // below the tile's least u
@@ -124,7 +127,7 @@ __device__ __forceinline__ Info make_info(const DirParams& p, const BackprojCons
   f.c0 = ia + cmin;
   f.shift = -cmin;
   // the box's layers: clamped to the stack's, as the voxels' are
-  f.L0 = max(min(lmin, c.nz_layers - c.cols_l), 0);
+  f.L0 = max(min(lmin + kMiddle, c.nz_layers - c.cols_l), 0);
   f.t -= (uint32_t)f.L0 << 24;
   f.top = c.cols_l - 1;
   return f;
