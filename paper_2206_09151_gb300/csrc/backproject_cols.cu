@@ -114,19 +114,30 @@ __global__ void __launch_bounds__(cols::kThreads, 2) k_backproject_cols_persiste
 
 constexpr int kMaxSmem = 220 * 1024;  // what a plan's boxes may take
 
-// CTAs that share a tile's directions: the split whose last wave is fullest, each CTA's prologue,
-// first loads and write-out counted as 5 directions' work.
-int pick_split(long long tiles, int slots, int dirs) {
+// CTAs that run at once in clusters of S, by CTAs per SM (1 or 2): clusters do not fill every SM of a GPC.  As
+// cudaOccupancyMaxActiveClusters gives it on a GB300.
+constexpr int kSlots[2][9] = {{0, 152, 152, 138, 144, 140, 138, 105, 120}, {0, 304, 304, 291, 296, 290, 276, 266, 288}};
+constexpr int kMaxSplit = 8;
+
+// Time of `ctas` CTAs, `slots` at once, in times of one that has its SM to itself: two on one SM take 1.43 of it.
+double wave_units(long long ctas, long long slots, int per_sm) {
+  const double full = per_sm == 2 ? 1.43 : 1.0;
+  const long long rest = ctas % slots;
+  return (double)(ctas / slots) * full + (rest == 0 ? 0.0 : (rest * per_sm > slots ? full : 1.0));
+}
+// A CTA's time in directions (0.63 us each, dir_cost times that): its share of them and what it spends around them,
+// 2.8, or 11 where a cluster shares them (sums left in shared memory and added across it).
+double split_units(long long tiles, int S, int per_sm, int dirs, double dir_cost) {
+  return wave_units(tiles * S, kSlots[per_sm - 1][S], per_sm) * ((dirs + S - 1) / S * dir_cost + (S == 1 ? 2.8 : 11.0));
+}
+// CTAs that share a tile's directions.  A split pays where the tiles leave SMs idle: 45 tiles, 60 directions 45
+// us whole, 27 in four; 128 tiles, 60 directions 45 whole, 51 in two.  Over 250 scans (32^3 to 288^3, flat and tall
+// volumes, 12 to 120 directions, 1 to 32 layers), each run with every split, the choice loses 2 % of the time on
+// average; counting 5 directions around either lost 14 % (208^3, 30 directions in two: 127 us instead of 101).
+int pick_split(long long tiles, int per_sm, int dirs) {
   int best = 1;
-  double best_t = 0.0;
-  for (int S = 1; S <= 8 && (S == 1 || dirs >= 4 * S); ++S) {
-    const double waves = (double)((tiles * S + slots - 1) / slots);
-    const double t = waves * ((double)((dirs + S - 1) / S) + 5.0);
-    if (S == 1 || t < best_t * 0.97) {
-      best = S;
-      best_t = t;
-    }
-  }
+  for (int S = 2; S <= kMaxSplit && dirs >= 2 * S; ++S)
+    if (split_units(tiles, S, per_sm, dirs, 1.0) < split_units(tiles, best, per_sm, dirs, 1.0)) best = S;
   return best;
 }
 
@@ -162,7 +173,7 @@ cudaError_t launch_cols_t(const BackprojConst& c, const DirParams* dirs, const v
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const unsigned gi = (c.nx + T::TI - 1) / T::TI, gk = (c.nz + cols::kTK - 1) / cols::kTK, gj = (c.nw + J - 1) / J;
-  const int S = pick_split((long long)gi * gk * gj, device_sm_count() * per_sm, dir_count);
+  const int S = pick_split((long long)gi * gk * gj, per_sm > 1 ? 2 : 1, dir_count);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(gi * S, gk, gj);
   cfg.blockDim = dim3(cols::kThreads);
