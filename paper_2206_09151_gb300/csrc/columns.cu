@@ -12,7 +12,9 @@
 //   - The phase is a 32-bit sum per layer (columns.cuh).
 // 120 directions x 32 layers of 256 x 256 (P = 512): 970 us with 8 values per thread, a filter value for each
 // and groups of two warps; 885 with the phase sums and 2 CTAs of up to 128 registers per SM instead of 3 of 80 (937
-// with 3); 805 with the mirrored parts.  The pair filter's layers (swapped order, 60 directions x 32): 1085, 881, 856.
+// with 3); 805 with the mirrored parts.  The pair filter's layers (swapped order, 60 directions x 32): 561, 470; two
+// layers (200 directions of 200 x 200): 225, 218, but 257 with an amplitude and an angle per frequency, one cosine
+// per layer, in place of the sine and the cosine (32 layers 461).
 // Forming the exchange addresses again per layer, or reading one part after the other, trades the 27 registers that
 // spill per layer for as many instructions: 1 to 9 % slower.
 // The CTA's columns are consecutive in (direction, column), so that the last column (Nyquist) of a direction
@@ -192,20 +194,16 @@ __global__ void __launch_bounds__(ColsT<P>::NTH, P >= 256 ? 2 : 4)
   // Nz per-layer depth constants
   const uint64_t* uAn = uA + (size_t)(dir_begin + n) * (c.nz_layers + (FILT == 3 ? 1 : 0));
   // The pair filter at a layer is Re{bracket exp(-i phi_k)} = sp cos phi_k - cp sin phi_k, phi_k = pi lambda z_k
-  // q^2, of the image-plane sp = sin chi / (sin^2 chi + eps) and cp = cos chi / (cos^2 chi + eps): kept as an
-  // amplitude and an angle that joins the phase, one cosine per layer.
-  float amp[FILT == 3 ? 9 : 1];
-  uint32_t angle[FILT == 3 ? 9 : 1];
+  // q^2, of the image-plane sp = sin chi / (sin^2 chi + eps) and cp = cos chi / (cos^2 chi + eps).
+  float sp[FILT == 3 ? 9 : 1], cp[FILT == 3 ? 9 : 1];
   if constexpr (FILT == 3) {
     const uint64_t uR = uAn[c.nz_layers];
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
       float sn, cs;
       sincos_half_turns((int32_t)(phase_of(uR, msq(i, j)) + base_hi(msq(i, j))), &sn, &cs);
-      const float sp = c.pair_mode == 0 ? __fdividef(sn, fmaf(sn, sn, c.eps)) : (c.pair_mode == 1 ? 1.f : 0.f);
-      const float cp = c.pair_mode == 0 ? __fdividef(cs, fmaf(cs, cs, c.eps)) : (c.pair_mode == 1 ? 0.f : -1.f);
-      amp[i] = sqrtf(fmaf(sp, sp, cp * cp));
-      angle[i] = (uint32_t)__float2ll_rn(atan2f(cp, sp) * 683565275.5764316f);  // 2^32 / (2 pi)
+      sp[i] = c.pair_mode == 0 ? __fdividef(sn, fmaf(sn, sn, c.eps)) : (c.pair_mode == 1 ? 1.f : 0.f);
+      cp[i] = c.pair_mode == 0 ? __fdividef(cs, fmaf(cs, cs, c.eps)) : (c.pair_mode == 1 ? 0.f : -1.f);
     }
   }
   // this thread's rows w = v - r_lo of T, v = j + s TT (nv <= P/2: s < 8), stored where 0 <= w < nw
@@ -218,19 +216,23 @@ __global__ void __launch_bounds__(ColsT<P>::NTH, P >= 256 ? 2 : 4)
   const int k_begin = blockIdx.y * lg;
   const int k_end = min(c.nz_layers, k_begin + lg);
   const float eps0 = fmaxf(c.eps, FLT_MIN);  // Tikhonov eps
-  uint32_t hi[NF], step[NF];                 // phase of the layer, per layer
+  uint32_t hi[NF], step[NF] = {};            // phase of the layer, per layer
+  if (FILT != 0 && c.nz_layers > 1) {
+    const uint64_t dA = uAn[1] - uAn[0];
+#pragma unroll
+    for (int i = 0; i < NF; ++i) step[i] = phase_step(dA, msq(i, j));
+  }
   for (int kr = k_begin, kr_end; kr < k_end; kr = kr_end) {  // runs of kPhaseRun layers
     kr_end = min(k_end, kr - kr % kPhaseRun + kPhaseRun);
     if constexpr (FILT != 0) {
       const int k0 = kr - kr % kPhaseRun;
       int jj = j;  // formed again for each run, not kept in registers over the layers
       asm volatile("" : "+r"(jj));
-      const uint64_t uA0 = uAn[k0], dA = k0 + 1 < c.nz_layers ? uAn[k0 + 1] - uA0 : 0;
+      const uint64_t uA0 = uAn[k0];
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
         const uint32_t m = msq(i, jj);
-        step[i] = phase_step(dA, m);
-        hi[i] = phase_of(uA0, m) + (FILT == 3 ? angle[FILT == 3 ? i : 0] : base_hi(m)) + (uint32_t)(kr - k0) * step[i];
+        hi[i] = phase_of(uA0, m) + (FILT == 3 ? 0u : base_hi(m)) + (uint32_t)(kr - k0) * step[i];
       }
     }
     for (int k = kr; k < kr_end; ++k) {
@@ -247,7 +249,9 @@ __global__ void __launch_bounds__(ColsT<P>::NTH, P >= 256 ? 2 : 4)
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
           if constexpr (FILT == 3) {
-            f[i] = amp[i] * cos_half_turns((int32_t)hi[i]);
+            float sn, cs;
+            sincos_half_turns((int32_t)hi[i], &sn, &cs);
+            f[i] = fmaf(sp[i], cs, -cp[i] * sn);
           } else {  // real part of the Eq. 11 bracket
             const float e = FILT == 2 ? positive_eps(__ldg(eps_k + bin[i])) : eps0;
             f[i] = inverse_ctf(sin_half_turns((int32_t)hi[i]), e);
