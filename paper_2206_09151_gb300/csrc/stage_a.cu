@@ -119,8 +119,9 @@ __host__ __device__ constexpr int cols16_per_cta() {
 // Column stage: a group of P/16 threads per spectrum column, cols16_per_cta columns per CTA.
 // The forward FFT along v stays in registers, multiplied once by the column's weight (ramp
 // or density weight, with the filter prefactor and 1/P^2); per layer: the CTF filter,
-// inverse FFT, store v < nv.
-template <int P, int FILT, bool DENS, bool BLEND>
+// inverse FFT, store v < nv.  ONE: one filtered layer, its phases formed where they are used: the sums' registers
+// cost 8 % there (200 directions of 512 x 16: 481 us, 447 without, 436 before there were sums).
+template <int P, int FILT, bool DENS, bool BLEND, bool ONE>
 __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const float2* __restrict__ S, float2* __restrict__ T,
                                                           const float2* __restrict__ twg,
                                                           const uint64_t* __restrict__ uA,
@@ -218,11 +219,12 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
   const int lg = (c.nz_layers + gridDim.z - 1) / gridDim.z;
   const int k_begin = blockIdx.z * lg;
   const int k_end = min(c.nz_layers, k_begin + lg);
-  uint32_t hi[FILT != 0 ? 16 : 1], step[FILT != 0 ? 16 : 1];  // phase of the layer, per layer
+  constexpr int NF = FILT != 0 && !ONE ? 16 : 1;
+  uint32_t hi[NF], step[NF];  // phase of the layer, per layer
   const float eps0 = fmaxf(c.eps, FLT_MIN);                   // Tikhonov eps
   for (int kr = k_begin, kr_end; kr < k_end; kr = kr_end) {  // runs of kPhaseRun layers
   kr_end = min(k_end, kr - kr % kPhaseRun + kPhaseRun);
-  if constexpr (FILT != 0) {
+  if constexpr (FILT != 0 && !ONE) {
     const int k0 = kr - kr % kPhaseRun;
     int jj = j;  // formed again for each run, not kept in registers over the layers
     asm volatile("" : "+r"(jj));
@@ -243,15 +245,21 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
         x[s] = xg[s];
       } else {
         float f;
+        uint32_t h;
+        if constexpr (ONE) {
+          h = phase_of(uAn[0], msq(s, j)) + (FILT == 3 ? 0 : base_hi(msq(s, j)));
+        } else {
+          h = hi[s];
+          hi[s] += step[s];
+        }
         if constexpr (FILT == 3) {  // Re{bracket * exp(-i phi_k)}, phi_k = pi lambda z_k q^2
           float sn, cs;
-          sincos_half_turns((int32_t)hi[s], &sn, &cs);
+          sincos_half_turns((int32_t)h, &sn, &cs);
           f = fmaf(sp[s], cs, -cp[s] * sn);
         } else {  // real part of the Eq. 11 bracket
           const float e = FILT == 2 ? positive_eps(__ldg(eps_k + (bins[s / 4] >> 8 * (s % 4) & 255u))) : eps0;
-          f = inverse_ctf(sin_half_turns((int32_t)hi[s]), e);
+          f = inverse_ctf(sin_half_turns((int32_t)h), e);
         }
-        hi[s] += step[s];
         x[s] = make_float2(xg[s].x * f, xg[s].y * f);
       }
     }
@@ -435,8 +443,8 @@ __global__ void k_count_nonfinite(const float* __restrict__ x, size_t n, unsigne
 }
 
 // ------------------------------------------------------------------ launch
-template <int P, int FILT, bool DENS, bool BLEND>
-cudaError_t launch_cols16(const StageAConst& c, const Workspace& ws, const float2* twq, int d0, int cnt, int sms,
+template <int P, int FILT, bool DENS, bool BLEND, bool ONE>
+cudaError_t launch_cols16_t(const StageAConst& c, const Workspace& ws, const float2* twq, int d0, int cnt, int sms,
                           cudaStream_t stream) {
   constexpr size_t smem = cols16_smem<P>();
   static unsigned long long attr_set = 0;  // devices on which the shared-memory limit is raised
@@ -444,7 +452,7 @@ cudaError_t launch_cols16(const StageAConst& c, const Workspace& ws, const float
   cudaGetDevice(&dev);
   if (dev >= 64 || !(attr_set >> dev & 1ull)) {
     const cudaError_t e =
-        cudaFuncSetAttribute(k_cols16<P, FILT, DENS, BLEND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_cols16<P, FILT, DENS, BLEND, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (dev < 64) attr_set |= 1ull << dev;
   }
@@ -453,9 +461,17 @@ cudaError_t launch_cols16(const StageAConst& c, const Workspace& ws, const float
   // set-up per group: the forward FFT (about one layer's work), and with the density
   // weighting about one more for the weights' trilinear lookups
   const int lg = pick_layer_groups(col_groups * cnt, c.nz_layers, (FILT == 3 ? 1 : 2) * sms, DENS ? 2.2 : 1.2);
-  k_cols16<P, FILT, DENS, BLEND><<<dim3(col_groups, cnt, lg), kThreads16, smem, stream>>>(
+  k_cols16<P, FILT, DENS, BLEND, ONE><<<dim3(col_groups, cnt, lg), kThreads16, smem, stream>>>(
       ws.S, ws.T, twq, ws.uA, ws.ramp, ws.dirs, ws.dens, ws.band_sum, ws.eps, ws.n_bins, ws.bin_width, c, d0);
   return cudaGetLastError();
+}
+
+template <int P, int FILT, bool DENS, bool BLEND>
+cudaError_t launch_cols16(const StageAConst& c, const Workspace& ws, const float2* twq, int d0, int cnt, int sms,
+                          cudaStream_t stream) {
+  if constexpr (FILT != 0 && !DENS)
+    if (c.nz_layers == 1) return launch_cols16_t<P, FILT, DENS, BLEND, true>(c, ws, twq, d0, cnt, sms, stream);
+  return launch_cols16_t<P, FILT, DENS, BLEND, false>(c, ws, twq, d0, cnt, sms, stream);
 }
 
 // The row stage of one sub-block into the stacks from direction s0 of the block on.

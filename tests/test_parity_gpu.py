@@ -431,3 +431,39 @@ def test_plans_of_other_box_sizes_run_from_several_threads(bp_kernel):
     assert not errors, errors
     for j in jobs:
         j[0].close()
+
+
+@pytest.mark.parametrize("nu,nv,filt", [(300, 5, "tikhonov"), (300, 6, "pair"), (1000, 3, "tikhonov"), (600, 2, "pair"),
+                                        (257, 1, "mlp"), (1024, 3, "mlp"), (200, 9, "pair"), (9, 4, "tikhonov")])
+def test_one_layer_column_stage_matches_oracle(nu, nv, filt):
+    """One filtered layer, which the 16-value column kernels take without phase sums.  The learned filter with a network
+    that gives one eps (only its output bias) is the Tikhonov filter of that eps."""
+    if filt != "mlp":
+        test_stage_a_layer_stack_matches_oracle((nu, nv, 1, filt, "intensity", 1e-6, 0.1, 0.05, 1e-10, 1e-9, 60e-9))
+        return
+    D, bias = 2, -1.5
+    rot = ph.single_axis_rotations(D, start=0.3)
+    img = torch.from_numpy((1.0 + 1e-2 * np.random.default_rng(nu).standard_normal((D, nv, nu))).astype(np.float32)).cuda()
+    kw = dict(lam=1e-10, delta=1e-9, defocus=np.full(D, 60e-9), nz_layers=1, sigma=0.1, cs=1e-6)
+    w = np.zeros(4481, np.float32)
+    w[-1] = bias
+    a = make(rot, nu, nv, (16, 8, 16), filter="mlp", mlp_weights=w, nsr=1e-2, **kw)
+    b = make(rot, nu, nv, (16, 8, 16), filter="tikhonov", eps=math.log1p(math.exp(bias)), **kw)
+    assert rel_l2(a.filter_stage(img, 0, D).cpu(), b.filter_stage(img, 0, D).cpu()) <= TOL_F32
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("nu,filt", [(300, "tikhonov"), (600, "pair")])
+def test_one_layer_between_two_detector_rows(nu, filt):
+    """... and its rows blended on the column stage, against the tap-pair kernel."""
+    rng = np.random.default_rng(nu)
+    img = torch.from_numpy((1.0 + 0.05 * rng.standard_normal((20, 24, nu))).astype(np.float32)).cuda()
+    rot = ph.single_axis_rotations(20, span=2 * math.pi, start=0.3)
+    kw = dict(lam=1e-10, delta=1e-9, defocus=rng.uniform(50e-9, 80e-9, 20), nz_layers=1, sigma=0.05, eps=0.02, filter=filt)
+    out = {}
+    for kernel in ("auto", "direct"):
+        r = make(rot, nu, 24, (40, 23, 40), bp_kernel=kernel, **kw)
+        out[kernel] = r.run(img).cpu().numpy()
+        r.close()
+    assert rel_l2(out["auto"], out["direct"]) <= TOL_F32
