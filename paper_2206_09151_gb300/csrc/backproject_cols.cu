@@ -251,6 +251,15 @@ void cols_setup(BackprojConst& c, const DirParams* dirs, int n_dirs) {
   }
 }
 
+// Not for flat volumes whose rows fill half of a tile's 32 or less, where the single-axis kernel, 16 rows per CTA, finds
+// them all on the detector and the tiles fill the SMs by themselves: 300 x 16 x 300 voxels, 60 directions 64 us,
+// the pairs 42; 256 x 16 x 256 (128 tiles) 45, 38.  With fewer tiles the split makes up for it (100 x 20 x 100: 20, 55).
+bool cols_pay(const BackprojConst& c) {
+  const long long tiles = (long long)((c.nx + cols::Tile<32>::TI - 1) / cols::Tile<32>::TI) * ((c.nz + cols::kTK - 1) / cols::kTK);
+  const bool flat = c.ny <= 16 && c.b_frac == 0.f && c.b_int >= -1 && c.b_int + 15 <= c.nv;
+  return !flat || tiles < 120;
+}
+
 cudaError_t describe_backproject_cols(const BackprojConst& c, BatchBp* out) {
   const int TI = c.cols_j == 64 ? cols::Tile<64>::TI : cols::Tile<32>::TI;
   out->kind = 8 + (c.stack_bf16 ? 2 : 0) + (c.cols_j == 64 ? 0 : 1);

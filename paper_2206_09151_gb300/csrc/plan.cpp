@@ -91,8 +91,10 @@ struct recon_plan_s {
   std::vector<float> theta, cnt, x2;  // learned regulariser: weights, bin counts, defocus feature
   recon::LearnConst lc;
   bool training = false;
-  recon::StageAConst ca;       // of whole runs (column stacks where the scan takes them)
+  recon::StageAConst ca;       // of whole runs: ca_cols or ca_pair
   recon::StageAConst ca_pair;  // of recon_filter_stage, whose layout is the tap pairs
+  recon::StageAConst ca_cols;  // of the batch: column stacks where the scan takes them
+  bool run_cols = false;       // whole runs use the column stacks
   recon::BackprojConst cb;
   int t_rows = 0;              // rows of T: nv, or the column stack's where those are more, rounded up to even
   recon::TmaBox tma{};   // footprint box of the TMA-staged backprojection
@@ -507,10 +509,8 @@ static int plan_create(const recon_geometry* geom, double lambda, double delta, 
   cb.staged = o.bp_kernel == RECON_BP_STAGED;
   cb.layer_linear = o.layer_interp == RECON_LAYER_LINEAR;
   cb.warp_cols = o.bp_warp ? o.bp_warp : 8;
-  // Column stacks (backproject_cols.cuh) where AUTO would run the single-axis kernel on tap pairs and
-  // the scan fits them, measured against the pairs per whole run: 64^3 / 90 views 78 us (106), 151 x 133 x 141 /
-  // 151 views between detector rows 1051 (1564), 512 x 256 x 512 / 360 views / 1 layer 5459 (8177), 256^3 / 360
-  // views / 32 layers 7.9 ms (the same: most lines span layers there).  An explicit DIRECT or STAGED keeps the pairs.
+  // Column stacks (backproject_cols.cuh) where AUTO would run the single-axis kernel on tap pairs, the
+  // scan fits them and (single runs) they pay, by cols_pay below.  An explicit DIRECT or STAGED keeps the pairs.
   ca.cols = 0;
   ca.nw = p->nv;
   ca.tp = (p->nv + 1) & ~1;
@@ -662,6 +662,9 @@ static int plan_create(const recon_geometry* geom, double lambda, double delta, 
   }
   p->ws_bytes = off;
   p->ca_pair.sub_block = ca.sub_block;
+  p->ca_cols = ca;
+  p->run_cols = cb.cols_j != 0 && recon::cols_pay(cb);
+  if (!p->run_cols) ca = p->ca_pair;
   if (o.filter == RECON_FILTER_MLP && !training && P < 16) {
     delete p;
     return fail(RECON_E_UNSUPPORTED_SIZE, "recon_plan: the learned filter needs images of more than 4 pixels");
@@ -823,7 +826,7 @@ unsigned int* tma_status(recon_plan_t p, void* ws) { return (unsigned int*)((cha
 // Stage B of one direction block through the plan's backprojection kernel.
 cudaError_t backproject_block(recon_plan_t p, const recon::DirParams* dirs, const void* stack, int d0, int cnt,
                               float* vol, int accumulate, void* ws, cudaStream_t s) {
-  if (p->cb.cols_j) return recon::launch_backproject_cols(p->cb, dirs, stack, d0, cnt, vol, accumulate, s);
+  if (p->run_cols) return recon::launch_backproject_cols(p->cb, dirs, stack, d0, cnt, vol, accumulate, s);
   if (p->use_tma)
     return recon::launch_backproject_tma(p->cb, p->tma, dirs, stack, d0, cnt, vol, accumulate, tma_status(p, ws), s);
   return recon::launch_backproject(p->cb, dirs, stack, d0, cnt, vol, accumulate, s);
@@ -1059,7 +1062,7 @@ int recon_backproject(recon_plan_t p, const void* stack, int dir_begin, int dir_
   rc = tma_begin(p, workspace, s, "recon_backproject");
   if (rc) return rc;
   // the caller's stack holds tap pairs (recon_filter_stage's layout)
-  cudaError_t e = p->cb.cols_j
+  cudaError_t e = p->run_cols
                       ? recon::launch_backproject(p->cb, w.dirs, stack, dir_begin, dir_count, volume, accumulate, s)
                       : backproject_block(p, w.dirs, stack, dir_begin, dir_count, volume, accumulate, workspace, s);
   if (e != cudaSuccess) return cuda_fail(e, "recon_backproject: launch");
@@ -1551,9 +1554,9 @@ int run_in_scratch(recon_plan_t p, const float* images, float* volume, char* scr
     cudaError_t e = recon::launch_stage_a(ca, w, images, d0, cnt, s, nullptr, mlp ? &hook : nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "recon_run_noalloc: stage A launch");
     // no kernel that reports through a status word, so the call need not synchronise
-    e = p->cb.cols_j ? recon::launch_backproject_cols(p->cb, w.dirs, w.stack, d0, cnt, volume,
-                                                      p->opt.accumulate || b > 0, s)
-                     : recon::launch_backproject(p->cb, w.dirs, w.stack, d0, cnt, volume, p->opt.accumulate || b > 0, s);
+    e = p->run_cols ? recon::launch_backproject_cols(p->cb, w.dirs, w.stack, d0, cnt, volume,
+                                                     p->opt.accumulate || b > 0, s)
+                    : recon::launch_backproject(p->cb, w.dirs, w.stack, d0, cnt, volume, p->opt.accumulate || b > 0, s);
     if (e != cudaSuccess) return cuda_fail(e, "recon_run_noalloc: backprojection launch");
   }
   return RECON_OK;
@@ -1869,7 +1872,7 @@ int batch_launch(recon_batch_t bt, const float* const* images, float* const* vol
       w.eps = (float*)(base + bt->off_eps);
       MlpHookCtx hctx{p, base + bt->off_tables[q], (float*)(base + bt->off_pow), w.eps, w.S, w.twp};
       const recon::StageAHook hook{mlp_hook, &hctx};
-      recon::StageAConst ca = p->ca;
+      recon::StageAConst ca = p->ca_cols;
       if (p->P >= 16) ca.sub_block = std::min(bt->dbb, p->ca.sub_block > 0 ? p->ca.sub_block : 1);
       e = recon::launch_stage_a(ca, w, img_q, d0, cnt, s, nullptr,
                                 p->ca.filter == RECON_FILTER_MLP ? &hook : nullptr);

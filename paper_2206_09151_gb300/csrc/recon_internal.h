@@ -165,6 +165,8 @@ cudaError_t launch_backproject(const BackprojConst& c, const DirParams* dirs, co
 // The column-stack backprojection of single-axis scans about y.  cols_setup fills c.cols_j,
 // cols_w, cols_l, cols_stage, nw, j_lo and wp (cols_j = 0 where the scan does not fit it).
 void cols_setup(BackprojConst& c, const DirParams* dirs, int n_dirs);
+// Whether single runs of a plan that cols_setup took use the column stacks (else tap pairs, the single-axis kernel).
+bool cols_pay(const BackprojConst& c);
 size_t cols_smem_bytes(const BackprojConst& c);
 // Waits for `stream` and takes the current device's count of its run-out waits (then 0 again).
 cudaError_t take_wait_failures(unsigned int* n, cudaStream_t stream);

@@ -467,3 +467,28 @@ def test_one_layer_between_two_detector_rows(nu, filt):
         out[kernel] = r.run(img).cpu().numpy()
         r.close()
     assert rel_l2(out["auto"], out["direct"]) <= TOL_F32
+
+
+@pytest.mark.parametrize("ny,nv,kernel_is_direct", [(16, 16, True), (17, 16, False), (16, 15, False), (9, 31, True), (9, 30, False)])
+def test_flat_single_axis_volumes_match_oracle(ny, nv, kernel_is_direct):
+    """Volumes of up to 16 rows over enough tiles keep the tap pairs in single runs (the same bits as bp_kernel="direct"),
+    others take the column stacks; a batch takes the column stacks for all."""
+    from paper_2206_09151_gb300.recon import Batch
+    rng = np.random.default_rng(ny * nv)
+    grid, nu, D = (330, ny, 180), 330, 4
+    img = (1.0 + 0.05 * rng.standard_normal((D, nv, nu))).astype(np.float32)
+    rot = ph.single_axis_rotations(D, start=0.3)
+    kw = dict(lam=1e-10, delta=1e-9, defocus=rng.uniform(50e-9, 80e-9, D), nz_layers=2, sigma=0.05, eps=0.02)
+    ref = O.recon(img, rot, grid=grid, filt=O.FILTER_TIKHONOV, **kw)
+    dimg, out = torch.from_numpy(img).cuda(), {}
+    for kernel in ("direct", "auto"):
+        r = make(rot, nu, nv, grid, filter="tikhonov", bp_kernel=kernel, **kw)
+        out[kernel] = r.run(dimg)
+        if kernel == "auto":
+            b = Batch([r])
+            out["batch"] = b.run([dimg])[0]
+            b.close()
+        r.close()
+    for v in out.values():
+        assert rel_l2(v.cpu(), ref) <= TOL_F32
+    assert torch.equal(out["auto"], out["direct"]) == kernel_is_direct
