@@ -204,6 +204,8 @@ struct TwoSum {
     e += (s - (t - b)) + (v - b);
     s = t;
   }
+  // an overflowed sum is infinite, its rounding error not a number
+  __device__ __forceinline__ double value() const { return isinf(s) ? (double)s : (double)s + e; }
 };
 
 template <int P>
@@ -294,7 +296,7 @@ __global__ void __launch_bounds__(kThreads) k_train_loss(const float2* __restric
     }
     __syncthreads();
   }
-  double a = (double)num.s + num.e, d = (double)den.s + den.e;
+  double a = num.value(), d = den.value();
   for (int o = 16; o > 0; o >>= 1) {
     a += __shfl_down_sync(0xffffffffu, a, o);
     d += __shfl_down_sync(0xffffffffu, d, o);

@@ -236,3 +236,19 @@ def test_a_nan_of_the_network_reaches_the_layers(nu, nv):
     layers = r.filter_stage(img, 0, 2)[:, :, 1:nv + 1, 1:, 0]
     assert bool(torch.isnan(layers).all())
     r.close()
+
+
+def test_training_loss_beyond_float32_is_infinite():
+    """Contrasts so large that a frequency's residual overflows: the loss is infinite, not NaN."""
+    from paper_2206_09151_gb300.recon import train_mlp
+    n, nzl = 16, 2
+    rng = np.random.default_rng(5)
+    img = torch.from_numpy((1e33 * rng.standard_normal((2, n, n))).astype(np.float32)).cuda()
+    tgt = torch.from_numpy((1e-9 * rng.standard_normal((2, nzl, n, n))).astype(np.float32)).cuda()
+    rot = ph.single_axis_rotations(2)
+    kw = {k: v for k, v in PHYS.items() if k != "input_mode"}
+    w = np.zeros(4481, np.float32)
+    w[-1] = -1.0  # one eps for all
+    _, loss, _ = train_mlp(w, img, tgt, rot, np.full(2, 50e-9), (n, n, n), nz_layers=nzl, nsr=1e-2, steps=0,
+                           input_mode="contrast", **kw)
+    assert np.isposinf(loss[0]), loss
