@@ -154,3 +154,23 @@ def test_gridding_with_a_noise_ratio_below_float32_is_the_one_without_the_filter
     ref, got = (r.grid_run(im, nsr).cpu().numpy() for nsr in (0.0, 1e-50))
     r.close()
     assert rel_l2(got, ref) <= TOL_F32, rel_l2(got, ref)
+
+
+@pytest.mark.parametrize("grid,n", [((300, 2, 3), 300), ((3, 270, 2), 270), ((2, 3, 511), 511), ((520, 2, 1), 520),
+                                    ((1, 600, 2), 600), ((2, 1, 700), 700)])
+def test_gridding_on_long_axes_matches_oracle(grid, n):
+    """Padded sides of 1024 and 2048 along each axis in turn, with images of that length.  The splat forms its coordinates
+    (up to P3 / 2 cells) in three float32 roundings, d = 1.5 2^-24 P3 / 2 cells off at most; a weight changes by d per
+    axis and a cell by its difference from its neighbours, so the volume is within 2 sqrt(3) d."""
+    from paper_2206_09151_gb300.recon import Reconstructor
+    rng = np.random.default_rng(n)
+    D, lam = 2, 1e-10
+    nu, nv = (n, 24) if grid[1] < n else (24, n)
+    img = (1.0 + 0.05 * rng.standard_normal((D, nv, nu))).astype(np.float32)
+    rot, Rs = ph.single_axis_rotations(D, start=0.2), rng.uniform(15e-9, 25e-9, D)
+    r = Reconstructor(rot, nu, nv, grid, lam=lam, delta=1e-9, defocus=Rs, nz_layers=2, sigma=0.3, eps=1e-2)
+    got = r.grid_run(torch.from_numpy(img).cuda()).cpu().numpy()
+    r.close()
+    ref = F.recon_gridding(img, rot, lam=lam, delta=1e-9, defocus=Rs, grid=grid, sigma=0.3, eps=1e-2)
+    P3 = 2 << (max(grid) - 1).bit_length()
+    assert rel_l2(got, ref) <= 2 * math.sqrt(3) * 1.5 * 2.0 ** -24 * P3 / 2, rel_l2(got, ref)
