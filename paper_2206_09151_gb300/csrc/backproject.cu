@@ -671,7 +671,7 @@ cudaError_t launch_backproject(const BackprojConst& c, const DirParams* dirs, co
 }
 
 cudaError_t describe_backproject(const BackprojConst& c, const DirParams* dirs, const void* stack, int dir_begin,
-                          int dir_count, float* volume, int accumulate, BatchBp* out) {
+                                 int dir_count, float* volume, int accumulate, BatchBp* out) {
   out->c = c;
   out->dirs = dirs;
   out->stack = stack;
@@ -679,9 +679,7 @@ cudaError_t describe_backproject(const BackprojConst& c, const DirParams* dirs, 
   out->dir_begin = dir_begin;
   out->dir_count = dir_count;
   out->accumulate = accumulate;
-  if (c.cols_j) {
-    return describe_backproject_cols(c, out);
-  }
+  if (c.cols_j) return describe_backproject_cols(c, out);
   const bool axis = c.axis_y && !c.layer_linear;
   if (axis) {
     out->kind = 2 + (c.stack_bf16 ? 2 : 0) + (c.b_frac != 0.f ? 1 : 0);
@@ -694,7 +692,6 @@ cudaError_t describe_backproject(const BackprojConst& c, const DirParams* dirs, 
     out->gy = (c.ny + kTY - 1) / kTY;
     out->gz = (c.nz + kTZ - 1) / kTZ;
   }
-  out->smem = (size_t)dir_count * (axis ? sizeof(AxisDir) : sizeof(TileDir));
   return cudaSuccess;
 }
 

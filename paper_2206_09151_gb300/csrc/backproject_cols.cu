@@ -262,11 +262,9 @@ bool cols_pay(const BackprojConst& c) {
 
 cudaError_t describe_backproject_cols(const BackprojConst& c, BatchBp* out) {
   const int TI = c.cols_j == 64 ? cols::Tile<64>::TI : cols::Tile<32>::TI;
-  out->kind = 8 + (c.stack_bf16 ? 2 : 0) + (c.cols_j == 64 ? 0 : 1);
   out->gx = (c.nx + TI - 1) / TI;
   out->gy = (c.nz + cols::kTK - 1) / cols::kTK;
   out->gz = (c.nw + c.cols_j - 1) / c.cols_j;
-  out->smem = cols_smem_bytes(c);
   return encode_cols(c, out->stack, out->dir_count, &out->map);
 }
 

@@ -27,8 +27,9 @@ __device__ __forceinline__ void sincos_half_turns(int32_t hi, float* sn, float* 
 // The phase of a frequency m runs linearly over the layers (their depths are equidistant), so the
 // layer loops add a 32-bit step per layer instead of forming uA_k m (a 32 x 64-bit product) each time:
 // hi(k) = hi(k0) + (k - k0) step, k0 the multiple of kPhaseRun below k, whose hi is exact to 2^-32 turns.  The step is
-// rounded to the nearest 2^-32 turns: at most kPhaseRun 2^-33 = 2^-27 turns of drift, less than the rounding of
-// the phase to float.  hi is a function of k alone, however the layers are split.
+// rounded to the nearest 2^-32 turns: at most kPhaseRun 2^-33 = 2^-27 turns of drift, 4.7e-8 rad, below the hardware
+// sine's error of 2^-21.4 (runs of 8, 16 and 64 layers leave the same error against 64 bits, 1.5e-6 for a batch of
+// uneven tomograms; 8 cost 3 to 5 % more time).  hi is a function of k alone, however the layers are split.
 constexpr int kPhaseRun = 64;
 __device__ __forceinline__ uint32_t phase_of(uint64_t uA, uint32_t m) {
   return (uint32_t)(uA >> 32) * m + __umulhi((uint32_t)uA, m);

@@ -191,10 +191,9 @@ cudaError_t launch_backproject_tma(const BackprojConst& c, const TmaBox& box, co
 // its 2 s limit) and sets bit 0 of *status; buf: >= 10 KB of device memory, 256-byte aligned.
 cudaError_t launch_tma_wait_probe(void* buf, size_t buf_bytes, unsigned int* status, cudaStream_t stream);
 
-// One tomogram's share of a persistent batched backprojection: its constants, pointers,
-// kernel kind (general 0/1, single-axis 2..5 (float32 / bfloat16 stack, one or two detector
-// rows), general with the layer blend 6/7, column stack 8..11 (float32 / bfloat16, 64 or 32 rows per
-// tile)), tile grid and the index of its first work item.
+// One tomogram's share of a persistent batched backprojection: its constants, pointers, tile grid and the index of
+// its first work item.  Tomograms on tap pairs: their kernel kind (general 0/1, single-axis 2..5 (float32 / bfloat16
+// stack, one or two detector rows), general with the layer blend 6/7); on column stacks: the round's tensor map.
 struct BatchBp {
   BackprojConst c;
   const DirParams* dirs;
@@ -203,14 +202,13 @@ struct BatchBp {
   int dir_begin, dir_count, accumulate, kind;
   int gx, gy, gz;
   unsigned long long first_item;
-  size_t smem;      // shared bytes its tiles need
-  alignas(64) CUtensorMap map;  // kinds 8..11: the round's column stacks
+  CUtensorMap map;
 };
 cudaError_t describe_backproject(const BackprojConst& c, const DirParams* dirs, const void* stack, int dir_begin,
-                          int dir_count, float* volume, int accumulate, BatchBp* out);
+                                 int dir_count, float* volume, int accumulate, BatchBp* out);
 cudaError_t launch_backproject_persistent(const BatchBp* desc_dev, int n_desc, unsigned long long total,
                                           unsigned long long* counter, size_t smem, cudaStream_t stream);
-// The tomograms of kinds 8..11 run in kernels of their own, one for 64-row and one for 32-row tiles (`rows`).
+// The tomograms on column stacks run in kernels of their own, one for 64-row and one for 32-row tiles (`rows`).
 cudaError_t describe_backproject_cols(const BackprojConst& c, BatchBp* out);
 cudaError_t launch_backproject_cols_persistent(const BatchBp* desc_dev, int n_desc, unsigned long long total, int rows,
                                                size_t smem, cudaStream_t stream);

@@ -4,9 +4,9 @@
 // Three kernels per block of directions:
 //   k_rows_fwd  two image rows packed as one complex row (real + i real), forward FFT,
 //               split into the two half spectra                    -> S[n][v][0..P/2]
-//   k_cols      one spectrum column per group of P/8 threads: forward FFT along v (rows
-//               >= nv are the zero padding), kept in registers; then for every layer
-//               k: multiply by H_k(q) W(q_u), inverse FFT along v, store v < nv
+//   k_cols      (columns.cu for P <= 512, P/16 threads per spectrum column; k_cols16 here for the larger ones) the
+//               forward FFT along v (rows >= nv are the zero padding), kept in registers; then for every
+//               layer k: multiply by H_k(q) W(q_u), inverse FFT along v, store the stack's rows
 //                                                                   -> T[n][k][col][v]
 //   k_rows_inv  (rows_inv.cu) two rows of one layer: Hermitian-extend both half spectra, pack
 //               as real + i real, inverse FFT, crop u < nu         -> the stack
@@ -223,63 +223,63 @@ __global__ void __launch_bounds__(kThreads16, FILT == 3 ? 1 : 2) k_cols16(const 
   uint32_t hi[NF], step[NF];  // phase of the layer, per layer
   const float eps0 = fmaxf(c.eps, FLT_MIN);                   // Tikhonov eps
   for (int kr = k_begin, kr_end; kr < k_end; kr = kr_end) {  // runs of kPhaseRun layers
-  kr_end = min(k_end, kr - kr % kPhaseRun + kPhaseRun);
-  if constexpr (FILT != 0 && !ONE) {
-    const int k0 = kr - kr % kPhaseRun;
-    int jj = j;  // formed again for each run, not kept in registers over the layers
-    asm volatile("" : "+r"(jj));
-    const uint64_t uA0 = uAn[k0], dA = k0 + 1 < c.nz_layers ? uAn[k0 + 1] - uA0 : 0;
+    kr_end = min(k_end, kr - kr % kPhaseRun + kPhaseRun);
+    if constexpr (FILT != 0 && !ONE) {
+      const int k0 = kr - kr % kPhaseRun;
+      int jj = j;  // formed again for each run, not kept in registers over the layers
+      asm volatile("" : "+r"(jj));
+      const uint64_t uA0 = uAn[k0], dA = k0 + 1 < c.nz_layers ? uAn[k0 + 1] - uA0 : 0;
 #pragma unroll
-    for (int s = 0; s < 16; ++s) {
-      const uint32_t m = msq(s, jj);
-      step[s] = phase_step(dA, m);
-      hi[s] = phase_of(uA0, m) + (FILT == 3 ? 0 : base_hi(m)) + (uint32_t)(kr - k0) * step[s];
-    }
-  }
-  for (int k = kr; k < kr_end; ++k) {
-    const float* eps_k = eps_tab + ((size_t)n * c.nz_layers + k) * n_bins;
-    float2 x[16];
-#pragma unroll
-    for (int s = 0; s < 16; ++s) {
-      if constexpr (FILT == 0) {
-        x[s] = xg[s];
-      } else {
-        float f;
-        uint32_t h;
-        if constexpr (ONE) {
-          h = phase_of(uAn[0], msq(s, j)) + (FILT == 3 ? 0 : base_hi(msq(s, j)));
-        } else {
-          h = hi[s];
-          hi[s] += step[s];
-        }
-        if constexpr (FILT == 3) {  // Re{bracket * exp(-i phi_k)}, phi_k = pi lambda z_k q^2
-          float sn, cs;
-          sincos_half_turns((int32_t)h, &sn, &cs);
-          f = fmaf(sp[s], cs, -cp[s] * sn);
-        } else {  // real part of the Eq. 11 bracket
-          const float e = FILT == 2 ? positive_eps(__ldg(eps_k + (bins[s / 4] >> 8 * (s % 4) & 255u))) : eps0;
-          f = inverse_ctf(sin_half_turns((int32_t)h), e);
-        }
-        x[s] = make_float2(xg[s].x * f, xg[s].y * f);
+      for (int s = 0; s < 16; ++s) {
+        const uint32_t m = msq(s, jj);
+        step[s] = phase_step(dA, m);
+        hi[s] = phase_of(uA0, m) + (FILT == 3 ? 0 : base_hi(m)) + (uint32_t)(kr - k0) * step[s];
       }
     }
-    fft16::group_fft_db<P, true>(x, buf0, buf1, tw, j, gsync);
-    float2* out = Tj + (size_t)k * c.half * c.tp;
-    if constexpr (!BLEND) {
-      // elements s >= 8 (v >= P/2) are never kept, so the last pass's butterflies that only feed them are
-      // dropped
+    for (int k = kr; k < kr_end; ++k) {
+      const float* eps_k = eps_tab + ((size_t)n * c.nz_layers + k) * n_bins;
+      float2 x[16];
 #pragma unroll
-      for (int s = 0; s < 8; ++s)
-        if (keep[s]) out[s * TT] = x[s];
-    } else {
-      // the transform's second pass, before its last barrier, was the last to read buf0
+      for (int s = 0; s < 16; ++s) {
+        if constexpr (FILT == 0) {
+          x[s] = xg[s];
+        } else {
+          float f;
+          uint32_t h;
+          if constexpr (ONE) {
+            h = phase_of(uAn[0], msq(s, j)) + (FILT == 3 ? 0 : base_hi(msq(s, j)));
+          } else {
+            h = hi[s];
+            hi[s] += step[s];
+          }
+          if constexpr (FILT == 3) {  // Re{bracket * exp(-i phi_k)}, phi_k = pi lambda z_k q^2
+            float sn, cs;
+            sincos_half_turns((int32_t)h, &sn, &cs);
+            f = fmaf(sp[s], cs, -cp[s] * sn);
+          } else {  // real part of the Eq. 11 bracket
+            const float e = FILT == 2 ? positive_eps(__ldg(eps_k + (bins[s / 4] >> 8 * (s % 4) & 255u))) : eps0;
+            f = inverse_ctf(sin_half_turns((int32_t)h), e);
+          }
+          x[s] = make_float2(xg[s].x * f, xg[s].y * f);
+        }
+      }
+      fft16::group_fft_db<P, true>(x, buf0, buf1, tw, j, gsync);
+      float2* out = Tj + (size_t)k * c.half * c.tp;
+      if constexpr (!BLEND) {
+        // elements s >= 8 (v >= P/2) are never kept, so the last pass's butterflies that only feed them are
+        // dropped
 #pragma unroll
-      for (int s = 0; s < 8; ++s) buf0[fft16::pad(j + s * TT)] = x[s];
-      gsync();
-      if (ok) store_blended(buf0, out, c, j, TT, [](int v) { return fft16::pad(v); });
-      gsync();  // the next transform's first pass writes buf0
+        for (int s = 0; s < 8; ++s)
+          if (keep[s]) out[s * TT] = x[s];
+      } else {
+        // the transform's second pass, before its last barrier, was the last to read buf0
+#pragma unroll
+        for (int s = 0; s < 8; ++s) buf0[fft16::pad(j + s * TT)] = x[s];
+        gsync();
+        if (ok) store_blended(buf0, out, c, j, TT, [](int v) { return fft16::pad(v); });
+        gsync();  // the next transform's first pass writes buf0
+      }
     }
-  }
   }
 }
 
