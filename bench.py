@@ -19,6 +19,7 @@ import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -53,8 +54,8 @@ WORKLOAD_TEXT = {
 # stack precision each workload is specified with
 DEFAULT_STACK = {"mid": "f32", "small": "f32", "learned": "bf16", "slab": "bf16", "batch": "bf16"}
 
-# DRAM traffic per launch (bytes) from ncu captures, keyed by kernel and workload and
-# valid only for the kernel source they were taken on (sha256 of the file).
+# DRAM traffic per launch (bytes) from ncu captures (profiles/captures_current.md), keyed by kernel and workload
+# and valid only for the kernel source they were taken on (sha256 of the file and the project headers that it includes).
 NCU_TRAFFIC: dict = {
     # mid (float32): one 40-direction launch each, scaled by 120/40 to the bench's blocks (the
     # backprojection's volume read-modify-write does not scale; its figure overstates it)
@@ -94,8 +95,16 @@ def ncu_traffic(kernel: str, workload: str, stack: str, filt: str):
 
 
 def _src_hash(name: str) -> str:
-    p = os.path.join(ROOT, "paper_2206_09151_gb300", "csrc", name)
-    return hashlib.sha256(open(p, "rb").read()).hexdigest()[:16]
+    """Of a kernel's source: the file and every project header that it includes, directly or not."""
+    csrc = os.path.join(ROOT, "paper_2206_09151_gb300", "csrc")
+    texts, todo = {}, [name]
+    while todo:
+        f = todo.pop()
+        p = os.path.join(csrc, f)
+        if f not in texts and os.path.exists(p):
+            texts[f] = open(p, "rb").read()
+            todo += [m.decode() for m in re.findall(rb'#include "([^"]+)"', texts[f])]
+    return hashlib.sha256(b"".join(texts[f] for f in sorted(texts))).hexdigest()[:16]
 
 
 def load_peaks() -> tuple[dict, str]:
@@ -460,7 +469,7 @@ def run_ours(args):
     algo = algorithmic_bytes(cfg, r, 2 if args.stack == "bf16" else 4, counts)
     kernels = {}
     bp_src = ("backproject_tma.cu" if r.bp_kernel_used == "tma" else
-              "backproject_cols.cuh" if args.bp_kernel == "auto" else "backproject.cu")
+              "backproject_cols.cu" if r.column_stacks else "backproject.cu")
     kernel_src = ["stage_a.cu", "columns.cu" if r.padded <= 512 else "stage_a.cu", "rows_inv.cu", bp_src]
     for q, name in enumerate(KERNELS):
         per_launch_ms = kern_ms[q] / max(kern_n[q], 1)
@@ -829,6 +838,8 @@ def run_fourier(args):
         gsub = -(-D // max(1, min(D, (1 << 30) // (cfg["nv"] * (r.padded // 2 + 1) * 8 + (r.padded // 2 + 1)
                                                    * r.padded * 8))))
         launches = dens + 3 * gsub + 1 + fft3
+        if nsr > 0:  # cells next to the noise threshold: summed again (over their spectra again, where those were not
+            launches += (1 if gsub == 1 else 3 * gsub) + 1  # all kept) and settled
         roofline = None
     line = {"metric": METRIC, "value": U / (ms_step / 1e3), "unit": UNIT, "n_gpus": 1, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
@@ -848,8 +859,8 @@ def run_fourier(args):
         line["swap_ct_ms"] = ms_step - sum(tail_ms) / args.steps
         line["swap_phase_ms"] = phase_ms
     else:
-        line["roofline_note"] = ("one call; its per-view splat (8 float atomics per accumulator and sample) and "
-                                 "3D passes are broken down by the launch list in profiles/")
+        line["roofline_note"] = ("one call; its per-view splat (a vector and a scalar reduction per corner and sample) "
+                                 "and 3D passes are broken down by the launch list in profiles/")
     print(json.dumps(line))
     r.close()
 

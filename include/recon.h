@@ -286,6 +286,9 @@ int recon_run_batch(int n, const recon_plan_t* plans, const float* const* images
  * plan launch (the resolution of RECON_BP_AUTO): RECON_BP_DIRECT (the single-axis or the
  * general direct kernel), RECON_BP_STAGED or RECON_BP_TMA.  No CUDA call. */
 int recon_plan_bp_kernel(recon_plan_t plan, int* kernel);
+/* *yes = 1 where the whole runs of a plan that answers RECON_BP_DIRECT keep column stacks (see
+ * RECON_BP_AUTO) and launch their kernel, else 0.  No CUDA call. */
+int recon_plan_column_stacks(recon_plan_t plan, int* yes);
 
 /* Depth of field (Sec. 1): DOF = delta^2 / (2 lambda).  Layers thinner than the DOF
  * keep every voxel within its layer's focus; a thicker layer is the plan-time warning of

@@ -103,6 +103,7 @@ def load_library(path: str = LIB_PATH):
     L.recon_plan_dof.argtypes = [vp, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double)]
     L.recon_plan_layers.argtypes = [vp, ctypes.POINTER(ip)]
     L.recon_plan_bp_kernel.argtypes = [vp, ctypes.POINTER(ip)]
+    L.recon_plan_column_stacks.argtypes = [vp, ctypes.POINTER(ip)]
     L.recon_swap_workspace_size.argtypes = [vp, ctypes.POINTER(sz)]
     L.recon_swap_ct.argtypes = [vp, vp, vp, sz, vp]
     L.recon_swap_phase.argtypes = [vp, ctypes.c_double, ctypes.c_double, vp, vp, sz, vp]
@@ -140,7 +141,7 @@ def load_library(path: str = LIB_PATH):
                  "recon_batch_workspace_size", "recon_batch_run", "recon_batch_run_graph", "recon_batch_destroy",
                  "recon_run_batch_workspace_size", "recon_run_batch", "recon_plan_dof", "recon_layers_for_dof",
                  "recon_plan_layers", "recon_swap_workspace_size", "recon_swap_ct", "recon_swap_phase",
-                 "recon_grid_workspace_size", "recon_grid_run", "recon_selftest_wait_limit", "recon_plan_bp_kernel",
+                 "recon_grid_workspace_size", "recon_grid_run", "recon_selftest_wait_limit", "recon_plan_bp_kernel", "recon_plan_column_stacks",
                  "recon_run_host", "recon_run_host_workspace_size", "recon_batch_run_host",
                  "recon_batch_run_host_workspace_size"):
         getattr(L, name).restype = ctypes.c_int
@@ -247,6 +248,13 @@ def recon_plan_layers(plan) -> int:
     n = ctypes.c_int()
     _check(load_library().recon_plan_layers(plan, ctypes.byref(n)), "recon_plan_layers")
     return n.value
+
+
+def recon_plan_column_stacks(plan) -> bool:
+    """Whether the plan's whole runs keep column stacks between the two stages."""
+    k = ctypes.c_int()
+    _check(load_library().recon_plan_column_stacks(plan, ctypes.byref(k)), "recon_plan_column_stacks")
+    return bool(k.value)
 
 
 def recon_plan_bp_kernel(plan) -> int:

@@ -707,6 +707,12 @@ int recon_plan_bp_kernel(recon_plan_t p, int* kernel) {
   return RECON_OK;
 }
 
+int recon_plan_column_stacks(recon_plan_t p, int* yes) {
+  if (!p || !yes) return fail(RECON_E_INVALID_ARG, "recon_plan_column_stacks: null argument");
+  *yes = p->run_cols ? 1 : 0;
+  return RECON_OK;
+}
+
 int recon_plan_dof(recon_plan_t p, double* pitch_max, double* dof) {
   if (!p) return fail(RECON_E_INVALID_ARG, "recon_plan_dof: null plan");
   if (pitch_max) *pitch_max = p->pitch_max;

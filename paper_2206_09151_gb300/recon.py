@@ -60,6 +60,7 @@ class Reconstructor:
         self.nz_layers = _abi.recon_plan_layers(self.plan)
         # the backprojection kernel the plan runs ("direct", "staged" or "tma")
         self.bp_kernel_used = {v: k for k, v in _BP_KERNELS.items()}[_abi.recon_plan_bp_kernel(self.plan)]
+        self.column_stacks = _abi.recon_plan_column_stacks(self.plan)
         self.ws_bytes = _abi.recon_workspace_size(self.plan)
         # recon_run_host's workspace: the same head plus two direction blocks of images
         self.ws_bytes_host = _abi.recon_run_host_workspace_size(self.plan)
