@@ -330,7 +330,7 @@ int recon_layers_for_dof(const recon_geometry* geom, const recon_grid* grid, dou
  *                     mean over the non-empty cells); nsr > 0 zeroes the coefficients whose
  *                     gridded contrast (the same splat without the bracket, over S + eps_S)
  *                     is below nsr M / sqrt(S), M^2 = nu nv (next to that threshold the sums
- *                     are taken again in 64 bits, so no order of additions decides; not
+ *                     are taken again in a fixed order, so that every call decides alike; not
  *                     where lambda > 8 delta); inverse transform, crop.  Any
  *                     geometry; the plan's sigma, eps, cs and input mode; its filter must be
  *                     TIKHONOV or PAIR (eps > 0).

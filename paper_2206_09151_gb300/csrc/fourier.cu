@@ -265,10 +265,12 @@ __global__ void k_grid_stats(const float* __restrict__ S, long long n, double* _
 // The noise filter keeps or drops whole cells by comparing float sums of atomics with a threshold, so for a cell
 // next to it the order in which the atomics land would decide, and the volume change by a plane wave (1e-4 of its
 // norm) from call to call.  Cells within kNearBand of the threshold (far more than the sums' rounding; some thousand
-// of 79 million for 192^3, 180 views) are noted by the pass that takes the decision, summed again in 64 bits in a
-// fixed order (k_grid_resum), and where the sums so rounded decide otherwise, the cell is added to or
-// taken out of the pass's result (k_grid_settle).  A note list that is full leaves its other cells as they were taken.
-// 192^3, 180 views: the call 2.71 ms, 2.66 without.
+// of 79 million for 192^3, 180 views) are noted by the pass that takes the decision, summed again in one fixed order
+// (k_grid_resum), and where those sums decide otherwise, the cell is added to or taken out of the pass's result
+// (k_grid_settle).  A note list that is full leaves its other cells as they were taken.  The order is that in which
+// the additions land in practice, so that volumes stay what they were: of the sums that six calls of the splat with
+// scalar atomics repeat, it gives 98 to 99 % to the bit, sums in 64 bits 91 %, which decided otherwise in 6 volumes of 17.
+// 192^3, 180 views: the call 2.74 ms, 2.66 without.
 constexpr float kNearBand = 0x1p-15f;
 
 // The two sides of the filter's comparison, |contrast| against its noise at a cell of weight s, inv = 1 / (s + eps_S).
@@ -334,7 +336,7 @@ struct GridQuotient {
         const unsigned int at = atomicAdd(near.count, 1u);
         if (at < near.cap) {
           near.cells[at] = 2 * (unsigned long long)cell(ix, iy, iz) + (keep ? 1 : 0);
-          for (int q = 0; q < 3; ++q) near.sums[3 * (size_t)at + q] = 0.0;
+          for (int q = 0; q < 3; ++q) near.sums[3 * (size_t)at + q] = 0.f;
         }
       }
       if (!keep) return make_float2(0.f, 0.f);
@@ -360,34 +362,66 @@ struct GridQuotient {
   }
 };
 
-// The noted cells' sums over `n_dirs` views in 64 bits: a warp per cell, its lanes over the views, in a fixed order.  A
-// view's samples that reach the cell lie around the cell's projection onto the view's axes, so a few are tried.
+// The order of a noted cell's additions: CTAs kResident at a time (5 per SM, as the splat with scalar atomics ran),
+// each in grid strides; those views that pass at the same time one after the other, and of a view the corners in
+// the order of the splat's code (bit 3: the mirrored half after the direct one), then the samples.
+constexpr int kResident = 5 * 152;
+__device__ __forceinline__ unsigned long long landing_key(unsigned sample, unsigned stride, int view, int corner,
+                                                          int in_view) {
+  const unsigned long long turn = sample / stride, wave = sample % stride / 256 / kResident;
+  // 4, 12, 20, 4 and 22 bits: a launch has at most 2^27 samples (1 GiB of spectra), 246 000 views of 32 x 17 of them
+  return ((((wave << 12 | turn) << 20 | (unsigned)view) << 4 | (unsigned)corner) << 22) | (unsigned)in_view;
+}
+
+// The noted cells' sums over `n_dirs` views: a warp per cell, its lanes over the views, listing the samples that reach
+// it (they lie around the cell's projection onto the view's axes, so a few are tried); then over the samples for their
+// contrasts; then the terms one by one by their keys.  Cells of more than kTerms terms (the lowest frequencies; the median is 2) take them in 64 bits.
+constexpr int kTerms = 1024, kResumWarps = 2;
+struct Terms {
+  unsigned long long key[kTerms];
+  float v[3][kTerms];
+  unsigned short order[kTerms];
+};
 __global__ void k_grid_resum(const float2* __restrict__ G, const GridDir* __restrict__ dirs, int dir_begin, int n_dirs,
-                             StageAConst c, Fourier3Const f, int lx, int ly, int reach, NearCells near) {
+                             StageAConst c, Fourier3Const f, int lx, int ly, float reach, unsigned stride,
+                             NearCells near) {
+  __shared__ Terms terms_all[kResumWarps];
+  __shared__ int n_terms_all[kResumWarps];
+  Terms& terms = terms_all[threadIdx.x >> 5];
+  int& n_terms = n_terms_all[threadIdx.x >> 5];
   const int P = c.P, lane = threadIdx.x & 31;
   const unsigned int n = min(*near.count, near.cap);
   for (unsigned int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < n; e += (gridDim.x * blockDim.x) >> 5) {
     const long long cell = (long long)(near.cells[e] >> 1);
     const int at[3] = {signed_bin((int)(cell >> ly) & (f.P3[0] - 1), f.P3[0]), signed_bin((int)cell & (f.P3[1] - 1), f.P3[1]),
                        signed_bin((int)(cell >> (lx + ly)), f.P3[2])};
-    double s = 0.0, x = 0.0, y = 0.0;
+    // samples per cell (powers of two); the grid is periodic: samples, up to reach P off, land on a cell's images too
+    const float per[3] = {1.f / f.scale[0], 1.f / f.scale[1], 1.f / f.scale[2]};
+    const int side = 2 * (int)(reach + 1.f) + 1;
+    double sum[3] = {0.0, 0.0, 0.0};
+    __syncwarp();
+    if (lane == 0) n_terms = 0;
+    __syncwarp();
     for (int v = lane; v < n_dirs; v += 32) {
       const GridDir& d = dirs[dir_begin + v];
-      // half widths, in samples, of the cell's reach along the view's axes
+      // half widths, in samples, of the cell's reach along the view's axes, and what rounding may add
       float h[3];
 #pragma unroll
       for (int q = 0; q < 3; ++q)
-        h[q] = 1.f + fabsf(d.r[3 * q]) / f.scale[0] + fabsf(d.r[3 * q + 1]) / f.scale[1] + fabsf(d.r[3 * q + 2]) / f.scale[2];
-      // the grid is periodic: samples land on a cell's images up to `reach` periods further too
-      const int side = 2 * reach + 1;
+        h[q] = 0.05f + fabsf(d.r[3 * q]) * per[0] + fabsf(d.r[3 * q + 1]) * per[1] + fabsf(d.r[3 * q + 2]) * per[2];
       for (int image = 0; image < side * side * side; ++image) {
-        const int b[3] = {at[0] + (image % side - reach) * f.P3[0], at[1] + (image / side % side - reach) * f.P3[1],
-                          at[2] + (image / (side * side) - reach) * f.P3[2]};
-        float p[3];
+        const int b[3] = {at[0] + (image % side - side / 2) * f.P3[0], at[1] + (image / side % side - side / 2) * f.P3[1],
+                          at[2] + (image / (side * side) - side / 2) * f.P3[2]};
+        float s3[3], p[3];
+        bool out = false;
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
-          p[q] = (float)b[0] / f.scale[0] * d.r[3 * q] + (float)b[1] / f.scale[1] * d.r[3 * q + 1] +
-                 (float)b[2] / f.scale[2] * d.r[3 * q + 2];
+        for (int a = 0; a < 3; ++a) {
+          s3[a] = (float)b[a] * per[a];
+          out |= fabsf(s3[a]) > reach * (float)P + 2.f * per[a];
+        }
+        if (out) continue;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) p[q] = s3[0] * d.r[3 * q] + s3[1] * d.r[3 * q + 1] + s3[2] * d.r[3 * q + 2];
         // q_z at the projection, and how far it varies over the window
         const float qz0 = -d.qz_coef * (p[0] * p[0] + p[1] * p[1]);
         const float vary = d.qz_coef * (2.f * (fabsf(p[0]) * h[0] + fabsf(p[1]) * h[1]) + h[0] * h[0] + h[1] * h[1]);
@@ -398,40 +432,74 @@ __global__ void k_grid_resum(const float2* __restrict__ G, const GridDir* __rest
             float g[3], w[3];
             sample_point(d, f, mu, mv, -d.qz_coef * (float)(uint32_t)(mu * mu + mv * mv), g);
             bool hit = true;
+            int corner = 0;
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
               const float fl = floorf(g[a]);
               const int to = b[a] - (int)fl;  // 0 or 1: the cell is a corner of the sample's
               hit &= to == 0 || to == 1;
+              corner |= (to & 1) << a;
               w[a] = to ? g[a] - fl : 1.f - (g[a] - fl);
             }
             const float wt = w[0] * w[1] * w[2];
             if (!hit || wt == 0.f) continue;
             const bool mirror = mu < 0 && mu > -P / 2;  // from column -mu, whose row -P/2 stays
             const int col = abs(mu), row = mirror && mv > -P / 2 ? -mv : mv;
-            const float2 gc = centred(G[((long long)v * c.half + col) * P + (row & (P - 1))], mirror, c, mu, mv);
-            s += (double)wt;
-            x += (double)__fmul_rn(wt, gc.x);
-            y += (double)__fmul_rn(wt, gc.y);
+            const int in_view = col * P + (row & (P - 1));
+            const int at_term = atomicAdd(&n_terms, 1);
+            if (at_term < kTerms) {
+              terms.key[at_term] =
+                  landing_key((unsigned)v * c.half * P + in_view, stride, v, corner + (mirror ? 8 : 0), in_view);
+              terms.v[0][at_term] = wt;
+            } else {
+              const float2 gc = centred(G[(long long)v * c.half * P + in_view], mirror, c, mu, mv);
+              sum[0] += (double)wt;
+              sum[1] += (double)__fmul_rn(wt, gc.x);
+              sum[2] += (double)__fmul_rn(wt, gc.y);
+            }
           }
       }
     }
+    __syncwarp();
+    const int m = n_terms;
+    float* const total = near.sums + 3 * (size_t)e;
+    for (int q = lane; q < min(m, kTerms); q += 32) {
+      const unsigned long long key = terms.key[q];
+      const int in_view = (int)(key & 0x3FFFFF), v = (int)(key >> 26 & 0xFFFFF), col = in_view >> c.logP;
+      const bool mirror = key >> 25 & 1;
+      const int row = signed_bin(in_view & (P - 1), P);
+      const int mu = mirror ? -col : (col == P / 2 ? -P / 2 : col), mv = mirror && row > -P / 2 ? -row : row;
+      const float2 gc = centred(G[(long long)v * c.half * P + in_view], mirror, c, mu, mv);
+      const float wt = terms.v[0][q];
+      const float t[3] = {wt, __fmul_rn(wt, gc.x), __fmul_rn(wt, gc.y)};
+      terms.v[1][q] = t[1];
+      terms.v[2][q] = t[2];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s += __shfl_down_sync(0xffffffffu, s, o);
-      x += __shfl_down_sync(0xffffffffu, x, o);
-      y += __shfl_down_sync(0xffffffffu, y, o);
+      for (int i = 0; i < 3; ++i) sum[i] += (double)t[i];
     }
-    if (lane == 0) {
-      double* t = near.sums + 3 * (size_t)e;
-      t[0] += s;
-      t[1] += x;
-      t[2] += y;
+    __syncwarp();
+    if (m > kTerms) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        for (int o = 16; o > 0; o >>= 1) sum[q] += __shfl_down_sync(0xffffffffu, sum[q], o);
+        if (lane == 0) total[q] = (float)(total[q] + sum[q]);
+      }
+      continue;
     }
+    for (int q = lane; q < m; q += 32) {
+      int rank = 0;
+      for (int k = 0; k < m; ++k) rank += terms.key[k] < terms.key[q];  // the keys are distinct
+      terms.order[rank] = (unsigned short)q;
+    }
+    __syncwarp();
+    float acc = lane < 3 ? total[lane] : 0.f;
+    if (lane < 3)
+      for (int k = 0; k < m; ++k) acc += terms.v[lane][terms.order[k]];
+    if (lane < 3) total[lane] = acc;
   }
 }
 
-// A warp per noted cell: where the 64-bit sums, rounded, decide otherwise, the cell's share of its z lines (transformed
+// A warp per noted cell: where the ordered sums decide otherwise, the cell's share of its z lines (transformed
 // already, planes off .. off + n of H) is added or taken out.
 __global__ void k_grid_settle(const GridQuotient<true> in, float2* __restrict__ H, int off, int n) {
   const int lane = threadIdx.x & 31;
@@ -441,10 +509,10 @@ __global__ void k_grid_settle(const GridQuotient<true> in, float2* __restrict__ 
   for (unsigned int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < noted; e += (gridDim.x * blockDim.x) >> 5) {
     const long long cell = (long long)(in.near.cells[e] >> 1);
     const bool kept = in.near.cells[e] & 1;
-    const double* t = in.near.sums + 3 * (size_t)e;
-    const float sum = (float)t[0];
+    const float* t = in.near.sums + 3 * (size_t)e;
+    const float sum = t[0];
     float signal, noise;
-    noise_sides(sum, 1.f / (sum + eps_s), (float)t[1], (float)t[2], in.nsr_m, &signal, &noise);
+    noise_sides(sum, 1.f / (sum + eps_s), t[1], t[2], in.nsr_m, &signal, &noise);
     const bool keep = signal >= noise;
     if (!(sum > 0.f) || keep == kept) continue;
     const int iy = (int)cell & (in.P3y - 1), ix = (int)(cell >> in.ly) & (in.P3x - 1), iz = (int)(cell >> (in.lx + in.ly));
@@ -611,8 +679,9 @@ cudaError_t launch_grid_resum(const GridSums& g, const float2* G, const GridDir*
   // wavelength (no image resolves that) the images of a cell are too many to try: its sums stay 0 and settle nothing
   const double reach = 0.7072 + f.lam / (4.0 * f.delta);
   if (reach > 2.8) return cudaSuccess;
-  k_grid_resum<<<device_sm_count() * 4, 128, 0, s>>>(G, dirs, dir_begin, n_dirs, c, f, log2_int(f.P3[0]),
-                                                     log2_int(f.P3[1]), (int)(reach + 1.0), g.near);
+  k_grid_resum<<<device_sm_count() * 10, 32 * kResumWarps, 0, s>>>(G, dirs, dir_begin, n_dirs, c, f, log2_int(f.P3[0]),
+                                                     log2_int(f.P3[1]), (float)reach,
+                                                     256 * grid_blocks((long long)n_dirs * c.half * c.P), g.near);
   return cudaGetLastError();
 }
 

@@ -1272,7 +1272,7 @@ GridLayout grid_layout(recon_plan_t p) {
   L.near_cells = off;
   off = align256(off + cap * sizeof(unsigned long long));
   L.near_sums = off;
-  off = align256(off + cap * 3 * sizeof(double));
+  off = align256(off + cap * 3 * sizeof(float));
   L.near_count = off;
   off = align256(off + sizeof(unsigned int));
   L.acc = off;
@@ -1447,7 +1447,7 @@ int recon_grid_run(recon_plan_t p, const float* images, float* volume, double ns
     if (e == cudaSuccess) e = recon::launch_grid_splat(G, gd, d0, cnt, p->ca, p->f3, acc, S, nsr_m > 0.f, s);
   }
   const recon::GridSums sums{acc, S, (double*)(b + L.stats), (float2*)(b + L.H),
-                             {(unsigned long long*)(b + L.near_cells), (double*)(b + L.near_sums),
+                             {(unsigned long long*)(b + L.near_cells), (float*)(b + L.near_sums),
                               (unsigned int*)(b + L.near_count), recon::grid_near_cap(p->f3)}, nsr_m};
   const float2* twa[3] = {axis_tw(p, tw[0], 0), axis_tw(p, tw[1], 1), axis_tw(p, tw[2], 2)};
   if (e == cudaSuccess) e = recon::launch_grid_quotient(sums, p->f3, twa, s);

@@ -246,7 +246,7 @@ size_t grid_half_cells(const Fourier3Const& f);
 // noise filter (nsr_m > 0) launch_grid_resum for every block of views, launch_grid_finish.
 struct NearCells {            // cells next to the noise filter's threshold
   unsigned long long* cells;  // 2 cell + (1: kept)
-  double* sums;               // [cap][3]: weight and contrast in 64 bits
+  float* sums;                // [cap][3]: weight and contrast, added in a fixed order
   unsigned int* count;
   unsigned int cap;
 };
