@@ -59,23 +59,25 @@ DEFAULT_STACK = {"mid": "f32", "small": "f32", "learned": "bf16", "slab": "bf16"
 NCU_TRAFFIC: dict = {
     # mid (float32): one 40-direction launch each, scaled by 120/40 to the bench's blocks (the
     # backprojection's volume read-modify-write does not scale; its figure overstates it)
-    ("k_cols", "mid", "f32"): {"bytes_per_launch": (63.224576e6 + 667.314944e6) * 3, "l2_hit_pct": 21.5,
-                               "src": "e4953fc265cd679c"},
-    ("k_backproject", "mid", "f32"): {"bytes_per_launch": (275.10272e6 + 46.691072e6) * 3, "l2_hit_pct": 57.7,
-                                      # 133.4 M warp instructions for 40 x 256^3 updates
-                                      "warp_inst_per_update": 133431471 / (40 * 256 ** 3),
-                                      "src": "2ba57b89bf0b5fc9"},
+    ("k_cols", "mid", "f32"): {"bytes_per_launch": (63.3344e6 + 667.562752e6) * 3, "l2_hit_pct": 21.3,
+                               "src": "2d9e1fd857c49452"},
+    ("k_rows_inv", "mid", "f32"): {"bytes_per_launch": (673.760512e6 + 306.35008e6) * 3, "l2_hit_pct": 26.6,
+                                   "src": "95dd4de02b89cbe3"},
+    ("k_backproject", "mid", "f32"): {"bytes_per_launch": (274.756864e6 + 46.555648e6) * 3, "l2_hit_pct": 58.1,
+                                      # 134.6 M warp instructions for 40 x 256^3 updates
+                                      "warp_inst_per_update": 134635754 / (40 * 256 ** 3),
+                                      "src": "7b2aa83f6dcb63f1"},
     # slab (bf16 stack): the column kernel from one 3-direction sub-block launch (the bench's
     # launch size); the TMA-staged backprojection from a 6-direction launch, its reads scaled
     # by 56/6 to the bench's 56-direction blocks (the stack boxes grow with the directions),
     # plus the volume read of an accumulating block and the volume write (1.07 GB each)
-    ("k_cols", "slab", "bf16"): {"bytes_per_launch": 53.836032e6 + 1.550214e9, "l2_hit_pct": 8.2,
-                                 "src": "8f3f2da5c9c0ceae"},
-    ("k_backproject", "slab", "bf16"): {"bytes_per_launch": 3.747824e9 * 56 / 6 + 1.073742e9 + 1.057885e9,
-                                        "l2_hit_pct": 56.8,
+    ("k_cols", "slab", "bf16"): {"bytes_per_launch": 53.828608e6 + 1.550140928e9, "l2_hit_pct": 8.2,
+                                 "src": "d216764a88be403a"},
+    ("k_backproject", "slab", "bf16"): {"bytes_per_launch": 3.750213632e9 * 56 / 6 + 1.073742e9 + 1.058193e9,
+                                        "l2_hit_pct": 56.7,
                                         # 1.443 G warp instructions for 6 x 1024^2 x 256 updates
-                                        "warp_inst_per_update": 1443406912 / (6 * 1024 * 1024 * 256),
-                                        "src": "8816bb7eb471e21e"},
+                                        "warp_inst_per_update": 1443325640 / (6 * 1024 * 1024 * 256),
+                                        "src": "f9ec9417a2390cbf"},
 }
 
 
