@@ -270,7 +270,7 @@ __global__ void k_grid_stats(const float* __restrict__ S, long long n, double* _
 // (k_grid_settle).  A note list that is full leaves its other cells as they were taken.  The order is that in which
 // the additions land in practice, so that volumes stay what they were: of the sums that six calls of the splat with
 // scalar atomics repeat, it gives 98 to 99 % to the bit, sums in 64 bits 91 %, which decided otherwise in 6 volumes of 17.
-// 192^3, 180 views: the call 2.74 ms, 2.66 without.
+// 192^3, 180 views: the call 2.67 ms, 2.66 without.
 constexpr float kNearBand = 0x1p-15f;
 
 // The two sides of the filter's comparison, |contrast| against its noise at a cell of weight s, inv = 1 / (s + eps_S).
@@ -373,9 +373,10 @@ __device__ __forceinline__ unsigned long long landing_key(unsigned sample, unsig
   return ((((wave << 12 | turn) << 20 | (unsigned)view) << 4 | (unsigned)corner) << 22) | (unsigned)in_view;
 }
 
-// The noted cells' sums over `n_dirs` views: a warp per cell, its lanes over the views, listing the samples that reach
-// it (they lie around the cell's projection onto the view's axes, so a few are tried); then over the samples for their
-// contrasts; then the terms one by one by their keys.  Cells of more than kTerms terms (the lowest frequencies; the median is 2) take them in 64 bits.
+// The noted cells' sums over `n_dirs` views, a warp per cell: its lanes over the views (and the periodic images of the
+// cell), a few of which have samples near the cell's projection onto their axes; over those samples, listing the ones
+// that reach the cell; over the list for the contrasts; then the terms one by one by their keys.  Cells of more than
+// kTerms terms (the lowest frequencies, or volumes much smaller than the images; the median is 2) take them in 64 bits.
 constexpr int kTerms = 1024, kResumWarps = 2;
 struct Terms {
   unsigned long long key[kTerms];
@@ -402,33 +403,46 @@ __global__ void k_grid_resum(const float2* __restrict__ G, const GridDir* __rest
     __syncwarp();
     if (lane == 0) n_terms = 0;
     __syncwarp();
-    for (int v = lane; v < n_dirs; v += 32) {
+    // whether view v has samples around the point s3 (in samples along the grid's axes), and their window
+    const auto window = [&](int v, const float (&s3)[3], int (&lo)[2], int (&n)[2]) {
       const GridDir& d = dirs[dir_begin + v];
-      // half widths, in samples, of the cell's reach along the view's axes, and what rounding may add
-      float h[3];
+      float p[3], h[3];
 #pragma unroll
-      for (int q = 0; q < 3; ++q)
+      for (int q = 0; q < 3; ++q) {
+        p[q] = s3[0] * d.r[3 * q] + s3[1] * d.r[3 * q + 1] + s3[2] * d.r[3 * q + 2];
+        // half widths, in samples, of the cell's reach along the view's axes, and what rounding may add
         h[q] = 0.05f + fabsf(d.r[3 * q]) * per[0] + fabsf(d.r[3 * q + 1]) * per[1] + fabsf(d.r[3 * q + 2]) * per[2];
-      for (int image = 0; image < side * side * side; ++image) {
-        const int b[3] = {at[0] + (image % side - side / 2) * f.P3[0], at[1] + (image / side % side - side / 2) * f.P3[1],
-                          at[2] + (image / (side * side) - side / 2) * f.P3[2]};
-        float s3[3], p[3];
-        bool out = false;
+      }
+      // q_z at the projection, and how far it varies over the window
+      const float qz0 = -d.qz_coef * (p[0] * p[0] + p[1] * p[1]);
+      const float vary = d.qz_coef * (2.f * (fabsf(p[0]) * h[0] + fabsf(p[1]) * h[1]) + h[0] * h[0] + h[1] * h[1]);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          s3[a] = (float)b[a] * per[a];
-          out |= fabsf(s3[a]) > reach * (float)P + 2.f * per[a];
-        }
-        if (out) continue;
+      for (int q = 0; q < 2; ++q) {
+        lo[q] = max(-P / 2, (int)ceilf(p[q] - h[q]));
+        n[q] = min(P / 2 - 1, (int)floorf(p[q] + h[q])) - lo[q] + 1;
+      }
+      return fabsf(p[2] - qz0) <= h[2] + vary && n[0] > 0 && n[1] > 0;
+    };
+    for (int image = 0; image < side * side * side; ++image) {
+      const int b[3] = {at[0] + (image % side - side / 2) * f.P3[0], at[1] + (image / side % side - side / 2) * f.P3[1],
+                        at[2] + (image / (side * side) - side / 2) * f.P3[2]};
+      float s3[3];
+      bool out = false;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) p[q] = s3[0] * d.r[3 * q] + s3[1] * d.r[3 * q + 1] + s3[2] * d.r[3 * q + 2];
-        // q_z at the projection, and how far it varies over the window
-        const float qz0 = -d.qz_coef * (p[0] * p[0] + p[1] * p[1]);
-        const float vary = d.qz_coef * (2.f * (fabsf(p[0]) * h[0] + fabsf(p[1]) * h[1]) + h[0] * h[0] + h[1] * h[1]);
-        if (fabsf(p[2] - qz0) > h[2] + vary) continue;
-        const int u1 = min(P / 2 - 1, (int)floorf(p[0] + h[0])), v1 = min(P / 2 - 1, (int)floorf(p[1] + h[1]));
-        for (int mu = max(-P / 2, (int)ceilf(p[0] - h[0])); mu <= u1; ++mu)
-          for (int mv = max(-P / 2, (int)ceilf(p[1] - h[1])); mv <= v1; ++mv) {
+      for (int a = 0; a < 3; ++a) {
+        s3[a] = (float)b[a] * per[a];
+        out |= fabsf(s3[a]) > reach * (float)P + 2.f * per[a];
+      }
+      if (out) continue;
+      for (int first = 0; first < n_dirs; first += 32) {
+        int lo[2], n_w[2];
+        unsigned todo = __ballot_sync(0xffffffffu, first + lane < n_dirs && window(first + lane, s3, lo, n_w));
+        for (; todo; todo &= todo - 1) {  // the lanes over the window's samples
+          const int v = first + __ffs(todo) - 1;
+          window(v, s3, lo, n_w);
+          const GridDir& d = dirs[dir_begin + v];
+          for (int q0 = lane; q0 < n_w[0] * n_w[1]; q0 += 32) {
+            const int mu = lo[0] + q0 / n_w[1], mv = lo[1] + q0 % n_w[1];
             float g[3], w[3];
             sample_point(d, f, mu, mv, -d.qz_coef * (float)(uint32_t)(mu * mu + mv * mv), g);
             bool hit = true;
@@ -458,6 +472,8 @@ __global__ void k_grid_resum(const float2* __restrict__ G, const GridDir* __rest
               sum[2] += (double)__fmul_rn(wt, gc.y);
             }
           }
+          __syncwarp();
+        }
       }
     }
     __syncwarp();

@@ -112,15 +112,16 @@ def test_line_transforms_of_every_length_match_oracle(grid):
     assert rel_l2(got, ref) <= TOL_F32, rel_l2(got, ref)
 
 
-def test_noise_filter_decides_alike_in_whatever_order_its_sums_are_added():
+@pytest.mark.parametrize("side,n,D", [(24, 24, 150), (12, 48, 60)])
+def test_noise_filter_decides_alike_in_whatever_order_its_sums_are_added(side, n, D):
     """The noise filter keeps or drops whole cells, so a cell next to the threshold must not hang on the
     order of the float atomics that sum it.  Steps of the volume over nsr, one cell pair each, are bisected down to
-    neighbouring float32 thresholds; there and a few steps around, every call gives one and the same volume."""
+    neighbouring float32 thresholds; there and a few steps around, every call gives one and the same volume.  Also a volume much smaller than the images,
+    whose cells take thousands of samples each."""
     from paper_2206_09151_gb300.recon import Reconstructor
-    n, D = 24, 150
     rng = np.random.default_rng(7)
     img = torch.from_numpy((1.0 + 0.1 * rng.standard_normal((D, n, n))).astype(np.float32)).cuda()
-    r = Reconstructor(ph.cone_rotations(D, 60.0, seed=3), n, n, (n, n, n), lam=4e-10, delta=1e-9,
+    r = Reconstructor(ph.cone_rotations(D, 60.0, seed=3), n, n, (side, side, side), lam=4e-10, delta=1e-9,
                       defocus=rng.uniform(10e-9, 20e-9, D), nz_layers=2, sigma=0.3, eps=1e-2, ramp="density")
 
     def vol(bits):  # at the float32 threshold nsr sqrt(nu nv) with these bits
@@ -129,8 +130,8 @@ def test_noise_filter_decides_alike_in_whatever_order_its_sums_are_added():
     def same(a, b):
         return float((a - b).norm()) <= 1e-5 * float(b.norm())
 
-    for t in (0.3, 0.8, 1.5, 2.5, 4.0):
-        lo, hi = (int(np.float32(x).view(np.int32)) for x in (t, t * 1.05))
+    for t in (0.3, 0.8, 1.5, 2.5, 4.0) if side == n else (1.0, 2.0, 4.0):
+        lo, hi = (int(np.float32(x).view(np.int32)) for x in (t, t * (1.05 if side == n else 1.5)))
         vlo = vol(lo)
         assert not same(vlo, vol(hi))
         while hi - lo > 1:
